@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "lb_ctx.h"
+#include "lb_fix64.cuh"
 
 
 namespace {
@@ -217,6 +218,7 @@ lbk::FluidArgs fluid_args(const lb_ctx *h, int cur, uint32_t step_off) {
     }
     for (int k = 10; k <= 18; ++k) a.pd.kg[k - 10] = (1.0 / 36.0) / bk[k] * rate(k);
     for (int k = 4; k <= 18; ++k) a.pd.kn[k - 4] = (1.0 / 36.0) / bk[k] * h->sig[k - 4] * 3.4641016151377544;
+    a.fx = h->fx;
     a.pf.rho0 = (float)a.pd.rho0;
     a.pf.omega = (float)a.pd.omega;
     for (int k = 0; k < 6; ++k) {
@@ -399,6 +401,13 @@ lb_status lb_create(const lb_params *p, void *cuda_stream, lb_handle *out) {
             const double gk = mode == 4 ? p->gamma_bulk : (mode <= 9 ? p->gamma_shear : (mode <= 15 ? p->gamma_odd : p->gamma_even));
             h->sig[k] = std::sqrt(3.0 * p->kT * b[k] * (1.0 - gk * gk));
         }
+    }
+    if (!h->fp32) {
+        double rates[15];
+        for (int k = 0; k < 15; ++k)
+            rates[k] = p->collision == 0 ? 1.0 - 1.0 / p->tau
+                     : (k == 0 ? p->gamma_bulk : (k <= 5 ? p->gamma_shear : (k <= 11 ? p->gamma_odd : p->gamma_even)));
+        h->fx = lbk::fix_params(p->rho0, p->kT, rates);
     }
     // block shape: x fastest, 128 threads
     int bx = ((p->nx + 31) / 32) * 32;

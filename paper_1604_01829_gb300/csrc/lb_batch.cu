@@ -20,7 +20,7 @@
 #include <vector>
 
 #include "../../include/lb.h"
-#include "lb_collide.cuh"
+#include "lb_fix64.cuh"
 #include "lb_couple.cuh"
 
 // register caps of the FP32 fluid kernel per parity (resident CTAs of 128
@@ -30,6 +30,10 @@
 #endif
 #ifndef LB_BATCH_REGS_ODD
 #define LB_BATCH_REGS_ODD 64
+#endif
+// of the FP64 fluid kernel (fixed-point collision)
+#ifndef LB_BATCH_REGS_F64
+#define LB_BATCH_REGS_F64 128
 #endif
 
 namespace lbk {
@@ -66,6 +70,7 @@ struct BInst {
     float gf[3];
     CollParams<double> pd;
     CollParams<float> pf;
+    FixParams fx;                // FP64 storage
 };
 
 struct BatchArgs {
@@ -75,6 +80,7 @@ struct BatchArgs {
     int n, ntiles, chunk, order;
     CollParams<double> pd;       // collision constants shared by all instances (COMMON kernels)
     CollParams<float> pf;
+    FixParams fx;
     void *pool;
     const void *F;               // spread force of this step (pool, storage precision), nullptr without bodies
     const int *tiles;
@@ -144,8 +150,8 @@ __device__ __forceinline__ void compact_odd_store(T *P, uint32_t base, uint32_t 
 }
 
 template <typename T, int COLL, bool NOISE, bool ODD, bool COMMON>
-__global__ void __maxnreg__(sizeof(T) == 4 ? (ODD ? LB_BATCH_REGS_ODD : LB_BATCH_REGS_EVEN) : 255)
-    k_batch_collide(const BatchArgs a) {
+__global__ void __maxnreg__(sizeof(T) == 4 ? (ODD ? LB_BATCH_REGS_ODD : LB_BATCH_REGS_EVEN) : LB_BATCH_REGS_F64)
+    k_batch_collide(const __grid_constant__ BatchArgs a) {
     using R = T;
     constexpr bool DEV = sizeof(T) == 4;
     for (int it = 0;; ++it) {
@@ -194,24 +200,28 @@ __global__ void __maxnreg__(sizeof(T) == 4 ? (ODD ? LB_BATCH_REGS_ODD : LB_BATCH
         const int zo[3] = {((int)z == 0 ? g.nz - 1 : (int)z - 1) * nxy, (int)z * nxy,
                            ((int)z == g.nz - 1 ? 0 : (int)z + 1) * nxy};
         auto at = [&](int i, uint32_t node) -> T & { return P[base + (uint32_t)i * N + chk(node, N, a.err)]; };
+        auto load = [&](R (&f)[19]) {
+            if (!ODD) {
+                const uint32_t m = compact ? w : n;
+#pragma unroll
+                for (int i = 0; i < 19; ++i) f[i] = at(i, m);
+            } else if (!compact) {
+                f[0] = at(0, n);
+#pragma unroll
+                for (int i = 1; i < 19; ++i)
+                    f[i] = at(opp(i), (uint32_t)(xo[1 - cx(i)] + yo[1 - cy(i)] + zo[1 - cz(i)]));
+            } else {
+                // the upstream node x - c_i: its compact position from the
+                // neighbour table, -1 for a wall node (the population bounced back)
+                const uint4 rec = __ldg(reinterpret_cast<const uint4 *>(g.cnbr) + chk(j, (long long)I.ncs, a.err));
+                const uint32_t nl = I.nax, sj = (uint32_t)g.csj, sa = (uint32_t)g.csa;
+                if (g.pore_axis == 2) compact_odd_load<2>(P, base, N, rec, j, l, nl, sj, sa, w, f, a.err);
+                else if (g.pore_axis == 1) compact_odd_load<1>(P, base, N, rec, j, l, nl, sj, sa, w, f, a.err);
+                else compact_odd_load<0>(P, base, N, rec, j, l, nl, sj, sa, w, f, a.err);
+            }
+        };
         R f[19];
-        if (!ODD) {
-            const uint32_t m = compact ? w : n;
-#pragma unroll
-            for (int i = 0; i < 19; ++i) f[i] = at(i, m);
-        } else if (!compact) {
-            f[0] = at(0, n);
-#pragma unroll
-            for (int i = 1; i < 19; ++i) f[i] = at(opp(i), (uint32_t)(xo[1 - cx(i)] + yo[1 - cy(i)] + zo[1 - cz(i)]));
-        } else {
-            // the upstream node x - c_i: its compact position from the
-            // neighbour table, -1 for a wall node (the population bounced back)
-            const uint4 rec = __ldg(reinterpret_cast<const uint4 *>(g.cnbr) + chk(j, (long long)I.ncs, a.err));
-            const uint32_t nl = I.nax, sj = (uint32_t)g.csj, sa = (uint32_t)g.csa;
-            if (g.pore_axis == 2) compact_odd_load<2>(P, base, N, rec, j, l, nl, sj, sa, w, f, a.err);
-            else if (g.pore_axis == 1) compact_odd_load<1>(P, base, N, rec, j, l, nl, sj, sa, w, f, a.err);
-            else compact_odd_load<0>(P, base, N, rec, j, l, nl, sj, sa, w, f, a.err);
-        }
+        load(f);
         R Fx, Fy, Fz;
         if constexpr (DEV) { Fx = I.gf[0]; Fy = I.gf[1]; Fz = I.gf[2]; }
         else { Fx = I.gd[0]; Fy = I.gd[1]; Fz = I.gd[2]; }
@@ -226,7 +236,8 @@ __global__ void __maxnreg__(sizeof(T) == 4 ? (ODD ? LB_BATCH_REGS_ODD : LB_BATCH
         if (NOISE) step = (uint32_t)(*a.step_base) + a.step_off;
         const uint2 key = make_uint2(I.key0, I.key1);
         if constexpr (DEV) collide<R, true, COLL, NOISE>(f, Fx, Fy, Fz, COMMON ? a.pf : I.pf, key, I.instance, n, step);
-        else collide<R, false, COLL, NOISE>(f, Fx, Fy, Fz, COMMON ? a.pd : I.pd, key, I.instance, n, step);
+        else collide_node_f64<COLL, NOISE>(f, Fx, Fy, Fz, COMMON ? a.fx : I.fx, COMMON ? a.pd : I.pd, key, I.instance, n,
+                                           step, load);
         // re-read the plane layout for the stores instead of keeping 19 plane
         // offsets live across the collision (register pressure)
         const uint32_t base2 = *(const volatile uint32_t *)&a.inst[k].off;
@@ -571,6 +582,11 @@ void fill_coll(const lb_params &p, BInst &I) {
         const double g = rate(k);
         const double sig = (p.collision == 1 && p.kT > 0.0) ? std::sqrt(3.0 * p.kT * bk[k] * (1.0 - g * g)) : 0.0;
         I.pd.kn[k - 4] = (1.0 / 36.0) / bk[k] * sig * 3.4641016151377544;
+    }
+    if (p.precision == 64) {
+        double rates[15];
+        for (int k = 4; k <= 18; ++k) rates[k - 4] = p.collision == 0 ? 1.0 - 1.0 / p.tau : rate(k);
+        I.fx = lbk::fix_params(p.rho0, p.kT, rates);
     }
     I.pf.rho0 = (float)I.pd.rho0;
     I.pf.omega = (float)I.pd.omega;
@@ -935,6 +951,7 @@ lb_status launch_step(lb_batch_ctx *h, int k, bool finish_prev, bool record, boo
     a.n = h->n;
     a.ntiles = h->ntiles;
     a.pd = h->hinst[0].pd;
+    a.fx = h->hinst[0].fx;
     a.pf = h->hinst[0].pf;
     const int res = h->resident[odd ? 1 : 0];
     int grid = h->sms * std::min(h->bpsm, res > 0 ? res : h->bpsm);

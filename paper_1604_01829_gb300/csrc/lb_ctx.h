@@ -40,6 +40,7 @@ struct lb_ctx {
     long long step = 0;                     // host mirror
     long long nfluid = 0;
     double sig[15] = {};
+    lbk::FixParams fx{};                    // FP64 storage: constants of the fixed-point collision
     // bead force fields (double buffered) and their 4x4x4 tile flags
     void *Fbuf[2] = {nullptr, nullptr};     // [3][N] each, storage precision
     int *tiles[2] = {nullptr, nullptr};      // 4x4x4 tile flags of each force buffer

@@ -21,7 +21,7 @@
 #include <algorithm>
 #include <cmath>
 
-#include "lb_collide.cuh"
+#include "lb_fix64.cuh"
 
 // Minimum resident blocks of 128 threads per SM requested for the FP32
 // collide kernels (caps their registers; FP64 kernels are not capped):
@@ -34,6 +34,9 @@
 #endif
 #ifndef LB_CS_MINB_NOISE
 #define LB_CS_MINB_NOISE 7
+#endif
+#ifndef LB_CS_MINB_F64
+#define LB_CS_MINB_F64 4
 #endif
 
 namespace lbk {
@@ -86,8 +89,8 @@ __device__ __forceinline__ uint32_t pore_section_index(const Geom &g, int x, int
 // ------------------------------------------------------- collide and stream
 
 template <typename T, int COLL, bool NOISE, bool ODD, bool PORE, bool OOP = false>
-__global__ void __launch_bounds__(128, sizeof(T) == 4 ? (NOISE ? LB_CS_MINB_NOISE : LB_CS_MINB) : 1)
-    k_collide_stream(const FluidArgs a) {
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? (NOISE ? LB_CS_MINB_NOISE : LB_CS_MINB) : LB_CS_MINB_F64)
+    k_collide_stream(const __grid_constant__ FluidArgs a) {
     using R = T;
     constexpr bool DEV = sizeof(T) == 4;
     const Geom &g = a.g;
@@ -134,7 +137,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (NOISE ? LB_CS_MINB_NOIS
     // odd step: population i arrives from the upstream node n - c_i, where it
     // sits in the opposite slot; halfway bounce-back takes the population that
     // left towards a wall (plus the moving-wall term of a channel wall upstream)
-    auto load_odd = [&](auto nb) {
+    auto load_odd = [&](R (&f)[19], auto nb) {
         f[0] = A[n];
 #pragma unroll
         for (int i = 1; i < 19; ++i) {
@@ -144,14 +147,17 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (NOISE ? LB_CS_MINB_NOIS
                 f[i] = plane(opp(i))[chk(nb(-cx(i), -cy(i), -cz(i)), N, a.err)];
         }
     };
-    if (!ODD) {
+    auto load = [&](R (&f)[19]) {
+        if (!ODD) {
 #pragma unroll
-        for (int i = 0; i < 19; ++i) f[i] = plane(i)[chk(n, N, a.err)];
-    } else if (row_in) {
-        load_odd(nb_in);
-    } else {
-        load_odd(nb_any);
-    }
+            for (int i = 0; i < 19; ++i) f[i] = plane(i)[chk(n, N, a.err)];
+        } else if (row_in) {
+            load_odd(f, nb_in);
+        } else {
+            load_odd(f, nb_any);
+        }
+    };
+    load(f);
 
     R Fx, Fy, Fz;
     if constexpr (sizeof(R) == 4) {
@@ -170,7 +176,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (NOISE ? LB_CS_MINB_NOIS
 
     const uint2 key = make_uint2(a.key0, a.key1);
     if constexpr (sizeof(R) == 4) collide<R, DEV, COLL, NOISE>(f, Fx, Fy, Fz, a.pf, key, a.instance, (uint32_t)n, step);
-    else collide<R, DEV, COLL, NOISE>(f, Fx, Fy, Fz, a.pd, key, a.instance, (uint32_t)n, step);
+    else collide_node_f64<COLL, NOISE>(f, Fx, Fy, Fz, a.fx, a.pd, key, a.instance, (uint32_t)n, step, load);
 
     // odd step: f*_i goes to the downstream node n + c_i, the upstream node of
     // link opp(i) there; a wall downstream returns it into the own slot

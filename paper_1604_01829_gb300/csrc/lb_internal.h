@@ -25,12 +25,27 @@ struct CollParams {
                                  //   applied to a centred uniform variate in (-1/2, 1/2) (FP32: times 2^-32)
 };
 
+// A 64-bit factor as h 2^32 + l with l signed, and the constants of the
+// fixed-point evaluation of the FP64 collision (lb_fix64.cuh).
+struct FixPair {
+    int h, l;
+};
+struct FixParams {
+    int on;                      // 0: not usable for these parameters (FP64 arithmetic then)
+    int cb, ce;                  // exponent constants of the conversions
+    double fs;                   // 2^(61 - k) / 12, k the exponent of the scaled unit
+    FixPair ke[15];              // modes 4-18: c_k (1 - g_k) at 2^64
+    FixPair ks[6];               // modes 4-9: c_k (1 + g_k) / 2 at 2^64
+    FixPair kn[15];              // modes 4-18: noise amplitude over sqrt(rho) of the scaled unit, at 2^64
+};
+
 // Everything the fused collide-and-stream kernel reads besides populations.
 struct FluidArgs {
     Geom g;
     void *f;                     // populations: double[19][N] (FP64) or float[19][N] deviations
     CollParams<double> pd;
     CollParams<float> pf;
+    FixParams fx;                // FP64 storage
     const double *gforce;        // device: uniform force density (3)
     const float *gforce_f;       // device: the same, rounded to FP32
     const void *Fn;              // device: spread bead force [3][N] in the storage precision, or nullptr
