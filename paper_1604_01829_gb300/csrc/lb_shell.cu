@@ -16,7 +16,9 @@
 // Integration: damped leapfrog with unit mass, v <- (1 - eta dt) v + dt F,
 // r <- r + dt v.
 //
-// Design: one thread block per shell, the shell's positions and velocities in
+// Design: one thread block per shell; the automatic pair search keeps
+// neighbour lists (k_relax_list). The explicit all-pairs and cell-list
+// searches: the shell's positions and velocities in
 // shared memory (structure of arrays, 6 n values: 192 KB for 4096 beads in
 // FP64), each thread owning up to 4 beads. A step reads every position once per owned
 // bead group (shared-memory broadcast: all lanes of a warp read the same j),
@@ -38,7 +40,6 @@ namespace {
 
 constexpr int kShellThreads = 1024;
 constexpr int kMaxCells = 4096;                     // cells per shell at most
-constexpr int kCellsFrom = 256;                     // automatic pair search: cell list from this many beads
 constexpr double kWcaCut = 1.122462048309373;      // 2^(1/6)
 
 template <typename R>
@@ -59,6 +60,7 @@ struct ShellArgs {
     const double *cbox;       // [nshells][3] half-widths L
     int max_cells;            // largest grid (shared-memory extent)
     int *err;                 // index checks of checked builds (LB_CHECKS): bit 2 on failure
+    R rl2, move2;             // neighbour lists: (range + skin)^2 and the squared move that outdates them
 };
 
 __device__ __forceinline__ float rdiv(float a, float b) { return __fdividef(a, b); }
@@ -90,6 +92,46 @@ __device__ __forceinline__ void surface_point(R x, R y, R z, R a, R b, R c, R &s
     sx = da > R(0) ? rdiv(x * a2, da) : R(0);
     sy = db > R(0) ? rdiv(y * b2, db) : R(0);
     sz = dc > R(0) ? rdiv(z * c2, dc) : R(0);
+}
+
+// The same point by Newton's iteration from a guess t (the bead's root of the
+// step before; updated). F is convex and falls on (-m^2, inf): from the left
+// of the root the iteration climbs to it without passing, from the right one
+// step leads to the left, and lo = -m^2 + m |x_m| (F(lo) >= 0) bounds it from
+// below. It ends after a step shorter than `tol` times the distance to the
+// nearest pole, whose square is below rounding: one step is usual where a
+// bead has moved by little. A bead for which it does not end so (the root at
+// the pole: no unique nearest point) takes the bisection.
+template <typename R>
+__device__ __forceinline__ void surface_point_near(R x, R y, R z, R a, R b, R c, R &t, R &sx, R &sy, R &sz) {
+    constexpr R tol = sizeof(R) == 8 ? R(0x1p-28) : R(0x1p-13);
+    const R a2 = a * a, b2 = b * b, c2 = c * c, xa = x * a, yb = y * b, zc = z * c;
+    const R m = fmin(a, fmin(b, c)), m2 = m * m;
+    R xm = R(0);
+    if (a == m) xm = fmax(xm, fabs(x));
+    if (b == m) xm = fmax(xm, fabs(y));
+    if (c == m) xm = fmax(xm, fabs(z));
+    const R lo = -m2 + m * xm;
+    t = fmax(t, lo);
+    for (int it = 0; it < 24; ++it) {
+        const R ia = rdiv(R(1), t + a2), ib = rdiv(R(1), t + b2), ic = rdiv(R(1), t + c2);
+        const R u = xa * ia, v = yb * ib, w = zc * ic;
+        const R F = u * u + v * v + w * w - R(1), D = u * u * ia + v * v * ib + w * w * ic;
+        const R d = rdiv(R(0.5) * F, D), tn = t + d;
+        // a NaN (0/0 at the pole) never ends the loop
+        if (fabs(d) <= tol * (t + m2) && tn > lo) {
+            // 1/(t + d + a^2) from 1/(t + a^2): the next term, (d ia)^3, is below rounding
+            const R ea = d * ia, eb = d * ib, ec = d * ic;
+            t = tn;
+            sx = x * a2 * (ia - ia * (ea - ea * ea));
+            sy = y * b2 * (ib - ib * (eb - eb * eb));
+            sz = z * c2 * (ic - ic * (ec - ec * ec));
+            return;
+        }
+        t = fmax(tn, lo);
+    }
+    surface_point(x, y, z, a, b, c, sx, sy, sz);
+    t = lo;
 }
 
 // Block-wide exclusive scan of cnt[0..C) into start[0..C] (start[C] = total),
@@ -311,6 +353,169 @@ __global__ void __launch_bounds__(kShellThreads) k_relax_shells(const ShellArgs<
     }
 }
 
+// Pair search through per-bead neighbour lists that last many steps: list
+// column i holds the beads within rl = the WCA range + skin of bead i when it
+// was built, in index order, and stays complete until some bead has moved by
+// skin / 2; the pairs outside the range add nothing, so every step sums what
+// the all-pairs search sums, in the same order. A list longer than kListLen
+// is not kept: its bead tests all pairs.
+//
+// One block per shell, positions in two shared buffers (one barrier a step),
+// velocities, list references and surface roots in registers. Bound by the
+// latency of ~550 dependent instructions per warp and step and one barrier
+// (ncu: issue 30 %, shared-memory pipe 9 %); the searches above spend 40
+// halvings (three divisions each) and n pair tests per bead. Measured on
+// GB300 per step, FP32: 203 shells of up to 344 beads 32.2 -> 2.9 us (all
+// pairs before), one (15, 5, 5) raspberry 29.0 -> 3.0 us (cell list before),
+// one shell of 2400 beads 117 -> 14.8 us (cell list); FP64, the 203 shells:
+// 1134 -> 98 us (its divisions on the FP64 pipe).
+constexpr int kListLen = 32;
+#ifndef LB_LIST_SKIN
+#define LB_LIST_SKIN 0.15
+#endif
+
+// threads of a block at most: FP64 beads need twice the registers
+template <typename R>
+constexpr int list_threads() { return sizeof(R) == 8 ? 512 : 1024; }
+
+template <typename R, int BPT>
+__global__ void __launch_bounds__(list_threads<R>()) k_relax_list(const ShellArgs<R> a) {
+    extern __shared__ unsigned char smem_raw[];
+    R *pos = reinterpret_cast<R *>(smem_raw);                          // [2][3][max_count]
+    uint16_t *list = reinterpret_cast<uint16_t *>(pos + 6 * (size_t)a.max_count);   // [kListLen][max_count]
+    const int M = a.max_count;
+    const int s = blockIdx.x;
+    const int n = a.count[s];
+    double *X = a.xyz + 3 * a.offset[s];
+    const R ax = (R)a.axes[3 * s], ay = (R)a.axes[3 * s + 1], az = (R)a.axes[3 * s + 2];
+    R xi[BPT], yi[BPT], zi[BPT], vx[BPT], vy[BPT], vz[BPT], rx[BPT], ry[BPT], rz[BPT], t[BPT];
+    int len[BPT];
+#pragma unroll
+    for (int b = 0; b < BPT; ++b) {
+        const int i = threadIdx.x + b * blockDim.x;
+        xi[b] = yi[b] = zi[b] = vx[b] = vy[b] = vz[b] = rx[b] = ry[b] = rz[b] = t[b] = R(0);
+        len[b] = 0;
+        if (i < n) {
+            xi[b] = (R)X[3 * i];
+            yi[b] = (R)X[3 * i + 1];
+            zi[b] = (R)X[3 * i + 2];
+            pos[i] = xi[b];
+            pos[M + i] = yi[b];
+            pos[2 * M + i] = zi[b];
+        }
+    }
+    bool rebuild = true;
+    __syncthreads();
+    for (long long step = 0; step < a.steps; ++step) {
+        const R *px = pos + (step & 1) * 3 * (size_t)M, *py = px + M, *pz = py + M;
+        R *nx = pos + ((step + 1) & 1) * 3 * (size_t)M, *ny = nx + M, *nz = ny + M;
+        if (rebuild) {                       // each thread its own beads' columns: no barrier needed
+#pragma unroll
+            for (int b = 0; b < BPT; ++b) {
+                const int i = threadIdx.x + b * blockDim.x;
+                if (i >= n) continue;
+                int k = 0;
+                for (int j = 0; j < n; ++j) {
+                    const R dx = xi[b] - px[j], dy = yi[b] - py[j], dz = zi[b] - pz[j];
+                    if (dx * dx + dy * dy + dz * dz < a.rl2 && j != i) {
+                        if (k < kListLen) list[(size_t)k * M + i] = (uint16_t)j;
+                        ++k;
+                    }
+                }
+                // padded to whole groups of four with the bead itself
+                for (int q = k; q < ((k + 3) & ~3) && q < kListLen; ++q) list[(size_t)q * M + i] = (uint16_t)i;
+                len[b] = k <= kListLen ? k : -1;
+                rx[b] = xi[b];
+                ry[b] = yi[b];
+                rz[b] = zi[b];
+            }
+        }
+        bool moved = false;
+#pragma unroll
+        for (int b = 0; b < BPT; ++b) {
+            const int i = threadIdx.x + b * blockDim.x;
+            if (i >= n) continue;
+            const R x = xi[b], y = yi[b], z = zi[b];
+            R sx, sy, sz;
+            surface_point_near(x, y, z, ax, ay, az, t[b], sx, sy, sz);
+            R fx = -a.k2 * (x - sx), fy = -a.k2 * (y - sy), fz = -a.k2 * (z - sz);
+            auto pair = [&](int j) {
+                const R dx = x - px[j], dy = y - py[j], dz = z - pz[j];
+                const R r2 = dx * dx + dy * dy + dz * dz;
+                if (r2 < a.rc2 && j != i) {
+                    const R s2 = rdiv(a.sig2, r2);
+                    const R s6 = s2 * s2 * s2;
+                    const R fm = rdiv(a.eps24 * (R(2) * s6 * s6 - s6), r2);
+                    fx += fm * dx;
+                    fy += fm * dy;
+                    fz += fm * dz;
+                }
+            };
+            if (len[b] < 0) {
+                for (int j = 0; j < n; ++j) pair(j);
+            } else if constexpr (sizeof(R) == 8) {
+                for (int k = 0; k < len[b]; ++k) pair(chk((int)list[(size_t)k * M + i], n, a.err));
+            } else {
+                // four at a time without a branch: their loads and divisions overlap
+                for (int k = 0; k < len[b]; k += 4) {
+                    R dx[4], dy[4], dz[4], fm[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const int j = chk((int)list[(size_t)(k + q) * M + i], n, a.err);
+                        dx[q] = x - px[j];
+                        dy[q] = y - py[j];
+                        dz[q] = z - pz[j];
+                        const R r2 = dx[q] * dx[q] + dy[q] * dy[q] + dz[q] * dz[q];
+                        const R ir2 = rdiv(R(1), r2), s2 = a.sig2 * ir2, s6 = s2 * s2 * s2;
+                        fm[q] = r2 < a.rc2 && j != i ? a.eps24 * (R(2) * s6 * s6 - s6) * ir2 : R(0);
+                    }
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        fx += fm[q] * dx[q];
+                        fy += fm[q] * dy[q];
+                        fz += fm[q] * dz[q];
+                    }
+                }
+            }
+            vx[b] = a.damp * vx[b] + a.dt * fx;
+            vy[b] = a.damp * vy[b] + a.dt * fy;
+            vz[b] = a.damp * vz[b] + a.dt * fz;
+            xi[b] = x + a.dt * vx[b];
+            yi[b] = y + a.dt * vy[b];
+            zi[b] = z + a.dt * vz[b];
+            nx[i] = xi[b];
+            ny[i] = yi[b];
+            nz[i] = zi[b];
+            const R ux = xi[b] - rx[b], uy = yi[b] - ry[b], uz = zi[b] - rz[b];
+            moved |= !(ux * ux + uy * uy + uz * uz < a.move2);
+        }
+        rebuild = __syncthreads_or(moved);   // the next step's positions are complete
+    }
+#pragma unroll
+    for (int b = 0; b < BPT; ++b) {
+        const int i = threadIdx.x + b * blockDim.x;
+        if (i >= n) continue;
+        R x = xi[b], y = yi[b], z = zi[b];
+        if (a.project_final) surface_point(xi[b], yi[b], zi[b], ax, ay, az, x, y, z);
+        X[3 * i] = (double)x;
+        X[3 * i + 1] = (double)y;
+        X[3 * i + 2] = (double)z;
+    }
+}
+
+size_t list_smem(size_t rsize, int max_count) {
+    return 6 * rsize * (size_t)max_count + sizeof(uint16_t) * kListLen * (size_t)max_count;
+}
+
+template <typename R, int BPT>
+cudaError_t launch_list_t(const ShellArgs<R> &a, int nshells, int threads, cudaStream_t s) {
+    const size_t smem = list_smem(sizeof(R), a.max_count);
+    cudaError_t e = cudaFuncSetAttribute(k_relax_list<R, BPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_relax_list<R, BPT><<<nshells, threads, smem, s>>>(a);
+    return cudaGetLastError();
+}
+
 size_t shell_smem(size_t rsize, int max_count, int max_cells, bool cells) {
     return 6 * rsize * (size_t)max_count + (cells ? sizeof(int) * (2 * (size_t)max_count + 2 * (size_t)max_cells + 1) : 0);
 }
@@ -326,7 +531,8 @@ cudaError_t launch_shells_t(const ShellArgs<R> &a, int nshells, int threads, cud
 }
 
 template <typename R>
-cudaError_t launch_shells(ShellArgs<R> a, const lb_shell_params &p, int nshells, bool cells, cudaStream_t s) {
+cudaError_t launch_shells(ShellArgs<R> a, const lb_shell_params &p, int nshells, bool cells, bool lists,
+                          cudaStream_t s) {
     a.k2 = (R)(2.0 * p.k_surface);
     a.sig2 = (R)(p.sigma * p.sigma);
     a.rc2 = (R)(kWcaCut * kWcaCut * p.sigma * p.sigma);
@@ -336,9 +542,22 @@ cudaError_t launch_shells(ShellArgs<R> a, const lb_shell_params &p, int nshells,
     a.steps = p.steps;
     a.project_final = p.project_final;
     // beads per thread: 1, 2 or 4; threads a multiple of the warp
-    const int bpt = a.max_count <= kShellThreads ? 1 : (a.max_count <= 2 * kShellThreads ? 2 : 4);
+    const int cap = lists ? list_threads<R>() : kShellThreads;
+    const int bpt = a.max_count <= cap ? 1 : (a.max_count <= 2 * cap ? 2 : 4);
     int threads = (a.max_count + bpt - 1) / bpt;
     threads = ((threads + 31) / 32) * 32;
+    if (lists) {
+        // skin: 0.15 sigma (about 9 listed beads at one bead per unit area, a
+        // few rebuilds in the first 1000 steps; 0.05 to 0.15 within 3 %, 2400
+        // beads 22.8 / 16.6 / 14.8 us per step at 0.05 / 0.1 / 0.15); 0.98:
+        // the margin of the rounding of distances and moves
+        const double skin = LB_LIST_SKIN * p.sigma, rl = kWcaCut * p.sigma + skin;
+        a.rl2 = (R)(rl * rl);
+        a.move2 = (R)(0.98 * 0.25 * skin * skin);
+        if (bpt == 1) return launch_list_t<R, 1>(a, nshells, threads, s);
+        if (bpt == 2) return launch_list_t<R, 2>(a, nshells, threads, s);
+        return launch_list_t<R, 4>(a, nshells, threads, s);
+    }
     if (cells) {
         if (bpt == 1) return launch_shells_t<R, 1, true>(a, nshells, threads, s);
         if (bpt == 2) return launch_shells_t<R, 2, true>(a, nshells, threads, s);
@@ -416,13 +635,12 @@ extern "C" lb_status lb_relax_shells(int nshells, const double *axes, const int 
         return fail(LB_ERR_ARG, "the cell list does not fit in shared memory for this shell size and precision");
     if (lbk::shell_smem(rsize, max_count, 1, false) > (size_t)optin)
         return fail(LB_ERR_ARG, "the shell does not fit in shared memory at this precision");
-    // automatic: the cell list pays off when a block per shell is latency-bound
-    // (few shells for the SMs) or the shells are large; many small shells fill
-    // the GPU and are faster testing all pairs (measured on GB300)
-    int nsm = 0;
-    if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) nsm = 1;
-    const bool auto_cells = max_count >= 1024 || (max_count >= lbk::kCellsFrom && nshells <= 2 * nsm);
-    const bool cells = p->pair_search == 2 || (p->pair_search == 0 && auto_cells && cells_fit);
+    // automatic: neighbour lists wherever they fit (4 beads a thread at most);
+    // the larger shells (2048 beads in FP64, about 2640 in FP32 and more) take
+    // the cell list when it fits, 4 times faster there than all pairs
+    const int list_cap = 4 * (p->precision == 64 ? lbk::list_threads<double>() : lbk::list_threads<float>());
+    const bool lists = p->pair_search == 0 && max_count <= list_cap && lbk::list_smem(rsize, max_count) <= (size_t)optin;
+    const bool cells = p->pair_search == 2 || (p->pair_search == 0 && !lists && cells_fit);
 
     cudaStream_t st = (cudaStream_t)cuda_stream;
     const size_t nd = (size_t)3 * nshells + (size_t)3 * total + (size_t)3 * nshells;
@@ -453,12 +671,12 @@ extern "C" lb_status lb_relax_shells(int nshells, const double *axes, const int 
             lbk::ShellArgs<double> a{};
             a.axes = daxes; a.count = dcount; a.offset = doff; a.xyz = dxyz; a.max_count = max_count;
             a.cgrid = dgrid; a.cbox = dbox; a.max_cells = cells ? max_cells : 1; a.err = derr;
-            e = lbk::launch_shells<double>(a, *p, nshells, cells, st);
+            e = lbk::launch_shells<double>(a, *p, nshells, cells, lists, st);
         } else {
             lbk::ShellArgs<float> a{};
             a.axes = daxes; a.count = dcount; a.offset = doff; a.xyz = dxyz; a.max_count = max_count;
             a.cgrid = dgrid; a.cbox = dbox; a.max_cells = cells ? max_cells : 1; a.err = derr;
-            e = lbk::launch_shells<float>(a, *p, nshells, cells, st);
+            e = lbk::launch_shells<float>(a, *p, nshells, cells, lists, st);
         }
     }
     int herr = 0;
