@@ -187,7 +187,8 @@ cudaError_t copy_records(const double *ring, int every, int cap, long long k0, l
 
 // MSD analysis of recorded trajectories (lb_traj.cu); all pointers device
 cudaError_t launch_msd(const double *X, const double *q, int nrec, int nbodies, int max_lag, const double *p_ref,
-                       double *work, double *out, cudaStream_t s);
+                       void *work, double *out, cudaStream_t s);
+size_t msd_work_bytes(int nrec, int nbodies);
 cudaError_t launch_couple(const CoupleArgs &a, cudaStream_t s);
 // end of a group of steps: second half kick of every body and the step
 // counter advance, in one launch (nbodies may be 0)

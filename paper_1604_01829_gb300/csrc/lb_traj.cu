@@ -22,19 +22,24 @@
 // as atan2(|p x p'|, p . p'), the same angle as the printed arccosine of the
 // dot product of the unit vectors without its loss of precision at small
 // angles.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/lb.h"
+#include "lb_fix64.cuh"
 #include "lb_rigid.cuh"
 
 namespace lbk {
 
 namespace {
 
-constexpr int kW = 9;   // work per (body, record): p-hat, body-frame trajectory, body-frame angles
+// Work per body, columns of nrec values each (SoA): p-hat (3), body-frame
+// trajectory (3), body-frame angles (3).
+constexpr int kW = 9;
 
 __device__ __forceinline__ double dot3(const double *a, const double *b) {
     return a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
@@ -56,87 +61,508 @@ __global__ void k_msd_prep(const double *X, const double *q, int nrec, int nb, c
     const double *qk = q + ((long long)b * nrec + k) * 4;
     double ak[3][3];
     axes_of(qk, ak);
-    double *w = work + t * kW;
+    double *w = work + (long long)b * nrec * kW + k;
     const double pn = sqrt(dot3(p_ref, p_ref));
-    for (int r = 0; r < 3; ++r) w[r] = (ak[0][r] * p_ref[0] + ak[1][r] * p_ref[1] + ak[2][r] * p_ref[2]) / pn;
+    double p[3];
+    for (int r = 0; r < 3; ++r) p[r] = (ak[0][r] * p_ref[0] + ak[1][r] * p_ref[1] + ak[2][r] * p_ref[2]) / pn;
+    // a quaternion that is not a unit one to rounding: the length is taken out
+    // (the squared chord of k_msd_angle scales with it)
+    const double off = fma(p[0], p[0], fma(p[1], p[1], fma(p[2], p[2], -1.0)));
+    const double len = fabs(off) > 0x1p-50 ? sqrt(dot3(p, p)) : 1.0;
+    for (int r = 0; r < 3; ++r) w[(long long)r * nrec] = p[r] / len;
     if (k == 0) {
-        for (int c = 3; c < kW; ++c) w[c] = 0.0;
+        for (int c = 3; c < kW; ++c) w[(long long)c * nrec] = 0.0;
         return;
     }
     double ap[3][3];
     axes_of(qk - 4, ap);
     const double *Xk = X + ((long long)b * nrec + k) * 3;
     const double d[3] = {Xk[0] - Xk[-3], Xk[1] - Xk[-2], Xk[2] - Xk[-1]};
-    for (int c = 0; c < 3; ++c) w[3 + c] = dot3(ap[c], d);
+    for (int c = 0; c < 3; ++c) w[(long long)(3 + c) * nrec] = dot3(ap[c], d);
     // i, j, k of step k against those of step k-1 (projection method)
-    w[6] = atan2(dot3(ak[2], ap[1]), dot3(ak[2], ap[2]));
-    w[7] = atan2(dot3(ak[0], ap[2]), dot3(ak[0], ap[0]));
-    w[8] = atan2(dot3(ak[1], ap[0]), dot3(ak[1], ap[1]));
-}
-
-// one thread per (body, column 3..8): running sums over the records, in order
-__global__ void k_msd_scan(int nrec, int nb, double *work) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= nb * 6) return;
-    const int b = t / 6, c = 3 + t % 6;
-    double *w = work + (long long)b * nrec * kW + c;
-    double s = 0.0;
-    for (int k = 0; k < nrec; ++k) {
-        s += w[(long long)k * kW];
-        w[(long long)k * kW] = s;
-    }
+    w[6LL * nrec] = atan2(dot3(ak[2], ap[1]), dot3(ak[2], ap[2]));
+    w[7LL * nrec] = atan2(dot3(ak[0], ap[2]), dot3(ak[0], ap[0]));
+    w[8LL * nrec] = atan2(dot3(ak[1], ap[0]), dot3(ak[1], ap[1]));
 }
 
 constexpr int kThreads = 256;
 
-// one block per (lag, body): averages over all time origins
-__global__ void __launch_bounds__(kThreads) k_msd_lags(const double *X, int nrec, int nb, int max_lag,
-                                                     const double *work, double *out) {
-    const int l = blockIdx.x + 1, b = blockIdx.y;
-    const int n = nrec - l;
-    double acc[LB_MSD_COLS];
-    for (int c = 0; c < LB_MSD_COLS; ++c) acc[c] = 0.0;
-    const double *Xb = X + (long long)b * nrec * 3;
-    const double *wb = work + (long long)b * nrec * kW;
-    for (int t = threadIdx.x; t < n; t += kThreads) {
-        const double *x0 = Xb + (long long)t * 3, *x1 = Xb + (long long)(t + l) * 3;
-        const double *w0 = wb + (long long)t * kW, *w1 = wb + (long long)(t + l) * kW;
-        for (int a = 0; a < 3; ++a) {
-            const double dx = x1[a] - x0[a];
-            acc[a] += dx * dx;
-            const double db = w1[3 + a] - w0[3 + a];
-            acc[3 + a] += db * db;
-            const double dr = w1[6 + a] - w0[6 + a];
-            acc[7 + a] += dr * dr;
-        }
-        const double cr[3] = {w0[1] * w1[2] - w0[2] * w1[1], w0[2] * w1[0] - w0[0] * w1[2],
-                              w0[0] * w1[1] - w0[1] * w1[0]};
-        const double th = atan2(sqrt(dot3(cr, cr)), dot3(w0, w1));
-        acc[6] += th * th;
-    }
-    __shared__ double red[LB_MSD_COLS][kThreads / 32];
+// one block per (column 3..8, body): running sums over the records; each
+// thread a contiguous run, the runs' totals by warp scans
+__global__ void __launch_bounds__(kThreads) k_msd_scan(int nrec, double *work) {
+    double *w = work + ((long long)blockIdx.y * kW + 3 + blockIdx.x) * nrec;
+    const int per = (nrec + kThreads - 1) / kThreads;
+    const int k0 = min(nrec, (int)threadIdx.x * per), k1 = min(nrec, k0 + per);
+    double s = 0.0;
+    for (int k = k0; k < k1; ++k) s += w[k];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int c = 0; c < LB_MSD_COLS; ++c) {
-        double v = acc[c];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) red[c][warp] = v;
+    double v = s;
+    for (int o = 1; o < 32; o <<= 1) {
+        const double u = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += u;
     }
+    __shared__ double tot[kThreads / 32];
+    if (lane == 31) tot[warp] = v;
     __syncthreads();
-    if (threadIdx.x < LB_MSD_COLS) {
-        double v = 0.0;
-        for (int w = 0; w < kThreads / 32; ++w) v += red[threadIdx.x][w];
-        out[((long long)b * max_lag + (l - 1)) * LB_MSD_COLS + threadIdx.x] = v / (double)n;
+    double base = __shfl_up_sync(0xffffffffu, v, 1);
+    if (lane == 0) base = 0.0;
+    double before = 0.0;
+    for (int u = 0; u < warp; ++u) before += tot[u];
+    base += before;
+    for (int k = k0; k < k1; ++k) {
+        base += w[k];
+        w[k] = base;
+    }
+}
+
+// The averages over time origins in integers. GB300 issues FP64 at 2 lanes
+// per SM and clock; a pair of records takes 85 FP64 instructions (9 squared
+// differences and an arctangent), which bound the FP64 kernel below at 15.0
+// ms for 64 bodies x 4000 records x 400 lags. As 57-bit integers the
+// differences are exact, the squares are three 32-bit products summed in 64
+// and then 128 bits, and the squared angle is a power series: integer work at
+// 64 times the rate. Measured for that case: 0.54 ms (k_msd_disp, 12 warp
+// instructions per 32 pairs and column) and 1.69 ms (k_msd_angle, bound by
+// its ~330, the polynomial mostly), the whole call 15.8 -> 2.85 ms.
+constexpr int kFixCols = 12;       // X (3), body-frame trajectory (3), angles (3), p-hat (3)
+constexpr int kFixBits = 56;       // |value| < 2^56 about the middle of a column's range
+constexpr int kRun = 15;           // consecutive origins per lane and tile (odd: no bank conflicts)
+constexpr int kTile = 32 * kRun;   // origins per tile
+constexpr int kTilesPerSum = 8;    // tiles until the 128-bit sums (< 2^114 a term, 3840 terms) are taken off
+constexpr int kWarps = 8;
+
+// a value v of a column as h 2^29 + l, 0 <= l < 2^29: the difference of two is
+// (h1 - h0) 2^29 + (l1 - l0), two subtractions without a carry
+struct Limbs {
+    int l, h;
+};
+
+__device__ __forceinline__ Limbs limbs(long long v) {
+    Limbs o;
+    o.l = (int)((unsigned)v & 0x1FFFFFFFu);
+    o.h = (int)(v >> 29);
+    return o;
+}
+
+// One block per (column, body): the column as integers about the middle of
+// its range, value = fix 2^unit; bad[body] is set where a value is not finite
+// or the scale is extreme (the FP64 kernel then takes the body).
+__global__ void __launch_bounds__(kThreads) k_msd_fix(const double *X, const double *work, int nrec, Limbs *fix,
+                                                    int *unit, int *bad) {
+    const int c = blockIdx.x, b = blockIdx.y;
+    const double *src;
+    long long st = 1;
+    if (c < 3) {
+        src = X + (long long)b * nrec * 3 + c;
+        st = 3;
+    } else {
+        src = work + ((long long)b * kW + (c < 9 ? c : c - 9)) * nrec;
+    }
+    Limbs *dst = fix + ((long long)b * kFixCols + c) * nrec;
+    __shared__ double smax[kThreads];
+    __shared__ long long slo[kThreads], shi[kThreads];
+    const int t = threadIdx.x;
+    double m = 0.0;
+    bool fine = true;
+    for (int k = t; k < nrec; k += kThreads) {
+        const double v = fabs(src[k * st]);
+        fine = fine && v < 0x1p400;
+        if (v > m) m = v;
+    }
+    smax[t] = m;
+    fine = __syncthreads_and(fine);
+    for (int w = kThreads / 2; w > 0; w >>= 1) {
+        if (t < w && smax[t + w] > smax[t]) smax[t] = smax[t + w];
+        __syncthreads();
+    }
+    m = smax[0];
+    if (!fine || (m > 0.0 && m < 0x1p-400)) {
+        if (t == 0) bad[b] = 1;
+        return;
+    }
+    if (c >= 9) {
+        // p-hat: components of a unit vector at 2^56, the last rounding errors
+        // of its length taken out (p - p off / 2, off = |p|^2 - 1 exactly)
+        const double *p = work + (long long)b * kW * nrec;
+        for (int k = t; k < nrec; k += kThreads) {
+            long long v[3];
+            __int128 sum = -((__int128)1 << 112);
+            for (int r = 0; r < 3; ++r) {
+                v[r] = __double2ll_rn(p[(long long)r * nrec + k] * 0x1p56);
+                sum += (__int128)v[r] * v[r];
+            }
+            const long long mine = c == 9 ? v[0] : (c == 10 ? v[1] : v[2]);
+            dst[k] = limbs(mine - (long long)((__int128)mine * (long long)sum >> 113));
+        }
+        if (t == 0) unit[b * kFixCols + c] = -56;
+        return;
+    }
+    int e = 0;
+    frexp(m, &e);                                  // m < 2^e
+    const double up = ldexp(1.0, 61 - e);
+    long long lo = 0x7FFFFFFFFFFFFFFFLL, hi = -0x7FFFFFFFFFFFFFFFLL;
+    for (int k = t; k < nrec; k += kThreads) {
+        const long long v = __double2ll_rn(src[k * st] * up);
+        if (v < lo) lo = v;
+        if (v > hi) hi = v;
+    }
+    slo[t] = lo;
+    shi[t] = hi;
+    __syncthreads();
+    for (int w = kThreads / 2; w > 0; w >>= 1) {
+        if (t < w) {
+            if (slo[t + w] < slo[t]) slo[t] = slo[t + w];
+            if (shi[t + w] > shi[t]) shi[t] = shi[t + w];
+        }
+        __syncthreads();
+    }
+    lo = slo[0];
+    hi = shi[0];
+    const long long mid = lo / 2 + hi / 2, half = (hi - lo) / 2 + 2;
+    int sh = 0;
+    while ((half >> sh) >= (1LL << kFixBits) - 1) ++sh;
+    const long long rnd = sh ? 1LL << (sh - 1) : 0;
+    for (int k = t; k < nrec; k += kThreads) dst[k] = limbs((__double2ll_rn(src[k * st] * up) - mid + rnd) >> sh);
+    if (t == 0) unit[b * kFixCols + c] = e - 61 + sh;
+}
+
+typedef unsigned __int128 U128;
+
+__device__ __forceinline__ U128 shfl_xor128(U128 v, int o) {
+    unsigned long long lo = (unsigned long long)v, hi = (unsigned long long)(v >> 64);
+    lo = __shfl_xor_sync(0xffffffffu, lo, o);
+    hi = __shfl_xor_sync(0xffffffffu, hi, o);
+    return ((U128)hi << 64) | lo;
+}
+
+// from the low end up, so that only the last addition rounds noticeably
+__device__ __forceinline__ double to_double(U128 v) {
+    const unsigned long long lo = (unsigned long long)v, hi = (unsigned long long)(v >> 64);
+    const double c = fma((double)(unsigned)(lo >> 32), 0x1p32, (double)(unsigned)lo);
+    return fma((double)(unsigned)(hi >> 32), 0x1p96, fma((double)(unsigned)hi, 0x1p64, c));
+}
+
+// Squared differences of one column (grid y) of one body (grid z): each warp
+// takes 8 lags, each lane 15 consecutive origins per tile and a sliding
+// window of 8 later records in registers (a quarter load per pair).
+constexpr int kLags = 8;
+__global__ void __launch_bounds__(32 * kWarps) k_msd_disp(const Limbs *fix, const int *unit, const int *bad,
+                                                         int nrec, int max_lag, double *out) {
+    const int c = blockIdx.y, b = blockIdx.z;
+    if (bad[b]) return;
+    const Limbs *x = fix + ((long long)b * kFixCols + c) * nrec;
+    __shared__ Limbs s0[kTile], s1[kTile + kLags * kWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lb0 = blockIdx.x * kLags * kWarps + 1;      // first lag of the block
+    const int l0 = lb0 + warp * kLags;                    // of the warp
+    U128 acc[kLags];
+#pragma unroll
+    for (int q = 0; q < kLags; ++q) acc[q] = 0;
+    double total = 0.0;                                   // lane q: of lag l0 + q
+    auto take = [&]() {
+#pragma unroll
+        for (int q = 0; q < kLags; ++q) {
+            for (int o = 16; o > 0; o >>= 1) acc[q] += shfl_xor128(acc[q], o);
+        }
+        U128 mine = acc[0];
+#pragma unroll
+        for (int q = 1; q < kLags; ++q)
+            if (lane == q) mine = acc[q];
+        total += to_double(mine);
+#pragma unroll
+        for (int q = 0; q < kLags; ++q) acc[q] = 0;
+    };
+    int tiles = 0;
+    for (int t0 = 0; t0 + lb0 < nrec; t0 += kTile) {
+        for (int i = threadIdx.x; i < kTile; i += 32 * kWarps) s0[i] = t0 + i < nrec ? x[t0 + i] : Limbs{0, 0};
+        for (int i = threadIdx.x; i < kTile + kLags * kWarps; i += 32 * kWarps)
+            s1[i] = t0 + lb0 + i < nrec ? x[t0 + lb0 + i] : Limbs{0, 0};
+        __syncthreads();
+        auto tile = [&](auto edge) {
+            constexpr bool EDGE = decltype(edge)::value;
+            const Limbs *p0 = s0 + lane * kRun, *p1 = s1 + warp * kLags + lane * kRun;
+            Limbs w[kLags];
+            long long A0[kLags], A1[kLags], A2[kLags];
+#pragma unroll
+            for (int q = 0; q < kLags; ++q) {
+                w[q] = p1[q];
+                A0[q] = A1[q] = A2[q] = 0;
+            }
+            const int room = nrec - (t0 + lane * kRun) - l0;      // pair (i, q) exists where i + q < room
+#pragma unroll
+            for (int i = 0; i < kRun; ++i) {
+                const Limbs a = p0[i];
+#pragma unroll
+                for (int q = 0; q < kLags; ++q) {
+                    // D = d1 2^29 + d0: |d1| <= 2^28, |d0| < 2^29
+                    int d0 = w[(i + q) % kLags].l - a.l, d1 = w[(i + q) % kLags].h - a.h;
+                    if (EDGE && i + q >= room) d0 = d1 = 0;
+                    A0[q] += (long long)d0 * d0;
+                    A1[q] += (long long)d1 * d0;
+                    A2[q] += (long long)d1 * d1;
+                }
+                if (i + 1 < kRun) w[i % kLags] = p1[i + kLags];
+            }
+#pragma unroll
+            for (int q = 0; q < kLags; ++q)
+                acc[q] += (U128)(unsigned long long)A0[q] + ((U128)(__int128)A1[q] << 30) +
+                          ((U128)(unsigned long long)A2[q] << 58);
+        };
+        if (l0 <= max_lag) {                              // warp-uniform
+            if (t0 + kTile + l0 + kLags <= nrec) tile(std::false_type{});
+            else tile(std::true_type{});
+            if (++tiles == kTilesPerSum) {
+                take();
+                tiles = 0;
+            }
+        }
+        __syncthreads();
+    }
+    if (l0 > max_lag) return;
+    take();
+    const int l = l0 + lane;
+    if (lane < kLags && l <= max_lag) {
+        const int col = c < 6 ? c : c + 1;
+        out[((long long)b * max_lag + (l - 1)) * LB_MSD_COLS + col] =
+            ldexp(total, 2 * unit[b * kFixCols + c]) / (double)(nrec - l);
+    }
+}
+
+// The squared angle between unit vectors at distance d apart: with z = d^2 =
+// 4 sin^2(theta/2), theta^2 = 4 asin^2(sqrt(z)/2) = sum_n 2 z^n / (n^2 C(2n, n))
+// = z + z^2 k(z). k on [0, 2] (angles up to 90 degrees) as the polynomial in
+// u = z/2 - 1/2 that interpolates its series at 19 Chebyshev nodes (error
+// below 2^-55; powers 0-11 at 2^64, 12-18 at 2^kAsinSqBits).
+constexpr int kAsinSqBits = 45;
+__constant__ long long kAsinSq[12] = {
+    1782374425807430006LL,
+    588604380132131925LL,
+    241213464260874337LL,
+    110996215031437458LL,
+    54884372548530884LL,
+    28496654949892514LL,
+    15326638144275224LL,
+    8465569096850234LL,
+    4774105254303728LL,
+    2737667270170072LL,
+    1591456043319638LL,
+    935016549813558LL,
+};
+__constant__ int kAsinSq32[7] = {1058753029, 642436037, 387510425, 203554602, 123855014, 139058146, 85944151};
+
+__global__ void __launch_bounds__(32 * kWarps) k_msd_angle(const Limbs *fix, const int *bad, int nrec, int max_lag,
+                                                         double *out) {
+    constexpr int LG = 4;                                 // lags per warp
+    const int b = blockIdx.y;
+    if (bad[b]) return;
+    const Limbs *x = fix + ((long long)b * kFixCols + 9) * nrec;
+    __shared__ Limbs s0[3][kTile], s1[3][kTile + LG * kWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lb0 = blockIdx.x * LG * kWarps + 1, l0 = lb0 + warp * LG;
+    U128 accz[LG], accr[LG];                              // sums of z at 2^112 and of z^2 k at 2^116
+    double slow[LG];                                      // sums of the angles beyond 176 degrees (FP64)
+#pragma unroll
+    for (int q = 0; q < LG; ++q) {
+        accz[q] = accr[q] = 0;
+        slow[q] = 0.0;
+    }
+    double total = 0.0;
+    auto take = [&]() {
+#pragma unroll
+        for (int q = 0; q < LG; ++q) {
+            for (int o = 16; o > 0; o >>= 1) {
+                accz[q] += shfl_xor128(accz[q], o);
+                accr[q] += shfl_xor128(accr[q], o);
+            }
+            if (__any_sync(0xffffffffu, slow[q] != 0.0))
+                for (int o = 16; o > 0; o >>= 1) slow[q] += __shfl_xor_sync(0xffffffffu, slow[q], o);
+        }
+        U128 mz = accz[0], mr = accr[0];
+        double ms = slow[0];
+#pragma unroll
+        for (int q = 1; q < LG; ++q)
+            if (lane == q) {
+                mz = accz[q];
+                mr = accr[q];
+                ms = slow[q];
+            }
+        total += fma(to_double(mz + (mr >> 4)), 0x1p-112, ms);
+#pragma unroll
+        for (int q = 0; q < LG; ++q) {
+            accz[q] = accr[q] = 0;
+            slow[q] = 0.0;
+        }
+    };
+    int tiles = 0;
+    for (int t0 = 0; t0 + lb0 < nrec; t0 += kTile) {
+        for (int c = 0; c < 3; ++c) {
+            const Limbs *xc = x + (long long)c * nrec;
+            for (int i = threadIdx.x; i < kTile; i += 32 * kWarps) s0[c][i] = t0 + i < nrec ? xc[t0 + i] : Limbs{0, 0};
+            for (int i = threadIdx.x; i < kTile + LG * kWarps; i += 32 * kWarps)
+                s1[c][i] = t0 + lb0 + i < nrec ? xc[t0 + lb0 + i] : Limbs{0, 0};
+        }
+        __syncthreads();
+        if (l0 <= max_lag) {
+            const int at0 = lane * kRun, at1 = warp * LG + lane * kRun;
+            const int room = nrec - (t0 + lane * kRun) - l0;
+            long long A0[LG], A1[LG], A2[LG];
+#pragma unroll
+            for (int q = 0; q < LG; ++q) A0[q] = A1[q] = A2[q] = 0;
+            for (int i = 0; i < kRun; ++i) {
+                const Limbs a[3] = {s0[0][at0 + i], s0[1][at0 + i], s0[2][at0 + i]};
+#pragma unroll
+                for (int q = 0; q < LG; ++q) {
+                    const Limbs v[3] = {s1[0][at1 + i + q], s1[1][at1 + i + q], s1[2][at1 + i + q]};
+                    long long a0 = 0, a1 = 0, a2 = 0;
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) {
+                        const int d0 = v[c].l - a[c].l, d1 = v[c].h - a[c].h;     // |d1| <= 2^28
+                        a0 += (long long)d0 * d0;
+                        a1 += (long long)d1 * d0;
+                        a2 += (long long)d1 * d1;
+                    }
+                    long long z = a2 + (a1 >> 28);                           // at 2^54
+                    const bool in = i + q < room;
+                    const bool far = in && z >= (1LL << 55);                 // beyond 90 degrees
+                    if (!in || far) {
+                        a0 = a1 = a2 = 0;
+                        z = 0;
+                    }
+                    if (far) {                   // the supplement's squared chord, from the sum of the vectors
+                        long long t1 = 0, t2 = 0;
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) {
+                            const int e0 = v[c].l + a[c].l, e1 = v[c].h + a[c].h;
+                            t1 += (long long)e1 * e0;
+                            t2 += (long long)e1 * e1;
+                        }
+                        z = t2 + (t1 >> 28);
+                    }
+                    if (z < 0) z = 0;
+                    // k by Horner's rule in u = z/2 - 1/2, |u| <= 1/2: the inner seven
+                    // steps (below 2^-14, and times u^12 at the end) in 32 bits
+                    const long long half = z << 8, u = half - (1LL << 62);   // z/2 and u at 2^63
+                    const int u32 = (int)(u >> 31);
+                    int ki = kAsinSq32[6];
+#pragma unroll
+                    for (int j = 5; j >= 0; --j) ki = kAsinSq32[j] + __mulhi(ki, u32);
+                    long long k = (long long)ki << (64 - kAsinSqBits);
+                    const FixPair up = fix_split(u);
+#pragma unroll
+                    for (int j = 11; j >= 0; --j) k = kAsinSq[j] + (fix_mul(fix_split(k), up) << 1);
+                    const long long B = fix_mul(fix_split(k), fix_split(half));   // z k at 2^62
+                    if (!far) {
+                        accr[q] += (U128)(unsigned long long)z * (unsigned long long)B;
+                    } else if (z >= (1LL << 46)) {
+                        // theta = pi - s, s^2 = z (1 + z k), s from an integer square root
+                        const bool low = z < (1LL << 50);                    // below 2^-4: 16 s^2
+                        const long long zz = z << (low ? 11 : 7);             // at 2^61 (2^65)
+                        long long r = fix_sqrt(zz + (fix_mul(fix_split(zz), fix_split(B)) << 2));
+                        if (low) r >>= 2;
+                        const FixPair th = fix_split(7244019458077122842LL - r);   // pi 2^61
+                        a2 = fix_mul(th, th) >> 4;                           // theta^2 at 2^54
+                    } else {
+                        auto val = [](Limbs x) { return fma((double)x.h, 0x1p29, (double)x.l); };
+                        const double w0[3] = {val(a[0]), val(a[1]), val(a[2])};
+                        const double w1[3] = {val(v[0]), val(v[1]), val(v[2])};
+                        const double cr[3] = {w0[1] * w1[2] - w0[2] * w1[1], w0[2] * w1[0] - w0[0] * w1[2],
+                                              w0[0] * w1[1] - w0[1] * w1[0]};
+                        const double th = atan2(sqrt(dot3(cr, cr)), dot3(w0, w1));
+                        slow[q] += th * th;
+                    }
+                    A0[q] += a0;
+                    A1[q] += a1;
+                    A2[q] += a2;
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < LG; ++q)
+                accz[q] += (U128)(unsigned long long)A0[q] + ((U128)(__int128)A1[q] << 30) +
+                           ((U128)(unsigned long long)A2[q] << 58);
+            if (++tiles == kTilesPerSum) {
+                take();
+                tiles = 0;
+            }
+        }
+        __syncthreads();
+    }
+    if (l0 > max_lag) return;
+    take();
+    const int l = l0 + lane;
+    if (lane < LG && l <= max_lag)
+        out[((long long)b * max_lag + (l - 1)) * LB_MSD_COLS + 6] = total / (double)(nrec - l);
+}
+
+// The same averages in FP64 (blocks over lags and bodies), for the bodies
+// that k_msd_fix marked: non-finite values spread to the lags they take part
+// in.
+__global__ void __launch_bounds__(kThreads) k_msd_lags(const double *X, int nrec, int max_lag, const double *work,
+                                                     const int *bad, double *out) {
+    const int b = blockIdx.y;
+    if (!bad[b]) return;
+    for (int l = blockIdx.x + 1; l <= max_lag; l += gridDim.x) {
+        const int n = nrec - l;
+        double acc[LB_MSD_COLS];
+        for (int c = 0; c < LB_MSD_COLS; ++c) acc[c] = 0.0;
+        const double *Xb = X + (long long)b * nrec * 3;
+        const double *wb = work + (long long)b * nrec * kW;
+        for (int t = threadIdx.x; t < n; t += kThreads) {
+            const double *x0 = Xb + (long long)t * 3, *x1 = Xb + (long long)(t + l) * 3;
+            auto w0 = [&](int c) { return wb[(long long)c * nrec + t]; };
+            auto w1 = [&](int c) { return wb[(long long)c * nrec + t + l]; };
+            for (int a = 0; a < 3; ++a) {
+                const double dx = x1[a] - x0[a];
+                acc[a] += dx * dx;
+                const double db = w1(3 + a) - w0(3 + a);
+                acc[3 + a] += db * db;
+                const double dr = w1(6 + a) - w0(6 + a);
+                acc[7 + a] += dr * dr;
+            }
+            const double p[3] = {w0(0), w0(1), w0(2)}, r[3] = {w1(0), w1(1), w1(2)};
+            const double cr[3] = {p[1] * r[2] - p[2] * r[1], p[2] * r[0] - p[0] * r[2], p[0] * r[1] - p[1] * r[0]};
+            const double th = atan2(sqrt(dot3(cr, cr)), dot3(p, r));
+            acc[6] += th * th;
+        }
+        __shared__ double red[LB_MSD_COLS][kThreads / 32];
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        for (int c = 0; c < LB_MSD_COLS; ++c) {
+            double v = acc[c];
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+            if (lane == 0) red[c][warp] = v;
+        }
+        __syncthreads();
+        if (threadIdx.x < LB_MSD_COLS) {
+            double v = 0.0;
+            for (int w = 0; w < kThreads / 32; ++w) v += red[threadIdx.x][w];
+            out[((long long)b * max_lag + (l - 1)) * LB_MSD_COLS + threadIdx.x] = v / (double)n;
+        }
+        __syncthreads();                     // red is reused
     }
 }
 
 }  // namespace
 
+size_t msd_work_bytes(int nrec, int nbodies) {
+    const size_t n = (size_t)nrec * nbodies;
+    return n * kW * sizeof(double) + n * kFixCols * sizeof(Limbs) + (size_t)nbodies * (kFixCols + 1) * sizeof(int);
+}
+
 cudaError_t launch_msd(const double *X, const double *q, int nrec, int nbodies, int max_lag, const double *p_ref,
-                       double *work, double *out, cudaStream_t s) {
-    const long long nt = (long long)nrec * nbodies;
-    k_msd_prep<<<(unsigned)((nt + 255) / 256), 256, 0, s>>>(X, q, nrec, nbodies, p_ref, work);
-    k_msd_scan<<<(unsigned)((6 * nbodies + 127) / 128), 128, 0, s>>>(nrec, nbodies, work);
-    k_msd_lags<<<dim3((unsigned)max_lag, (unsigned)nbodies), kThreads, 0, s>>>(X, nrec, nbodies, max_lag, work, out);
+                       void *work, double *out, cudaStream_t s) {
+    const size_t n = (size_t)nrec * nbodies;
+    double *w = static_cast<double *>(work);
+    Limbs *fix = reinterpret_cast<Limbs *>(w + n * kW);
+    int *unit = reinterpret_cast<int *>(fix + n * kFixCols), *bad = unit + (size_t)nbodies * kFixCols;
+    cudaError_t e = cudaMemsetAsync(bad, 0, sizeof(int) * nbodies, s);
+    if (e != cudaSuccess) return e;
+    k_msd_prep<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(X, q, nrec, nbodies, p_ref, w);
+    k_msd_scan<<<dim3(6, (unsigned)nbodies), kThreads, 0, s>>>(nrec, w);
+    k_msd_fix<<<dim3(kFixCols, (unsigned)nbodies), kThreads, 0, s>>>(X, w, nrec, fix, unit, bad);
+    const unsigned gd = (unsigned)((max_lag + kLags * kWarps - 1) / (kLags * kWarps));
+    k_msd_disp<<<dim3(gd, 9, (unsigned)nbodies), 32 * kWarps, 0, s>>>(fix, unit, bad, nrec, max_lag, out);
+    const unsigned ga = (unsigned)((max_lag + 4 * kWarps - 1) / (4 * kWarps));
+    k_msd_angle<<<dim3(ga, (unsigned)nbodies), 32 * kWarps, 0, s>>>(fix, bad, nrec, max_lag, out);
+    k_msd_lags<<<dim3((unsigned)std::min(max_lag, std::max(8, 2048 / nbodies)), (unsigned)nbodies), kThreads, 0, s>>>(X, nrec, max_lag, w, bad, out);
     return cudaGetLastError();
 }
 
@@ -198,7 +624,7 @@ extern "C" lb_status lb_msd_trajectory(const double *X, const double *q, int nre
         return fail(LB_ERR_ARG, "p_ref must be non-zero");
     cudaStream_t s = (cudaStream_t)cuda_stream;
     const size_t nX = (size_t)nrec * nbodies * 3, nq = (size_t)nrec * nbodies * 4;
-    const size_t nw = (size_t)nrec * nbodies * lbk::kW, no = (size_t)max_lag * nbodies * LB_MSD_COLS;
+    const size_t nw = (lbk::msd_work_bytes(nrec, nbodies) + 7) / 8, no = (size_t)max_lag * nbodies * LB_MSD_COLS;
     double *d = nullptr;
     const size_t total = nX + nq + nw + no + 3;
     cudaError_t e = cudaMalloc((void **)&d, total * sizeof(double));
