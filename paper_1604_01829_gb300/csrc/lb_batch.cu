@@ -375,12 +375,10 @@ __global__ void k_batch_pre(Body *bodies, int nb, int finish_prev, T *F, int *ti
                             const int *tcount, const BInst *inst, const long long *flag_start, int n,
                             Recorder rec, int list_cap, long long ttot, int *err, double dt) {
     const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (threadIdx.x == 0 && blockIdx.x < nb) {     // one body per block
-        Body B = bodies[blockIdx.x];
-        if (finish_prev) kick2(B, dt);
-        kick_drift(B, dt);
-        bodies[blockIdx.x] = B;
-        record_body(rec, B, blockIdx.x, nb);
+    if (threadIdx.x < 32 && blockIdx.x < nb) {     // one body per block
+        Body *B = bodies + blockIdx.x;
+        if (finish_prev) body_update<true, true>(B, threadIdx.x, dt, nullptr, blockIdx.x, nb, rec);
+        else body_update<false, true>(B, threadIdx.x, dt, nullptr, blockIdx.x, nb, rec);
     }
     if (!tiles) return;
     // one thread per (listed tile, node of the tile)

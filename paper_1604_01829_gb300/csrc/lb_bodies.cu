@@ -1,6 +1,6 @@
 // Raspberry kernels (Ustach & Faller, arXiv:1604.01829):
 //  - rigid-body integration of the centre of mass by velocity Verlet and of
-//    the orientation by a quaternion (Sec. 2.3), one thread per body in FP64;
+//    the orientation by a quaternion (Sec. 2.3), one warp per body in FP64;
 //  - virtual sites r_b = X + R(q) s_b, v_b = V + omega x (r_b - X) (Sec. 1.2);
 //  - friction coupling F_b = -gamma (v_b - u(r_b)) + f_s, Eq.
 //    (latticeboltzmannfriction) in Sec. 1.1, with u trilinearly interpolated
@@ -13,7 +13,7 @@ namespace lbk {
 
 namespace {
 
-// Step prologue in one launch: thread 0 of blocks [0, nb) finishes the
+// Step prologue in one launch: warp 0 of blocks [0, nb) finishes the
 // previous step's body (second half kick) if asked and starts this step's
 // (half kick, drift, rotation); every thread also clears nodes of the
 // flagged 4x4x4 tiles of this step's spread-force buffer.
@@ -21,21 +21,11 @@ template <typename T>
 __global__ void k_step_pre(Body *bodies, int nb, int finish_prev, T *F, int *tiles, const int *tlist,
                            const int *tcount, Geom g, int ntx, int nty, Recorder rec, double dt, const double *ext) {
     const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    // one body per block, so the FP64 work of the bodies spreads over SMs;
-    // a private copy means one read and one write of the record
-    if (threadIdx.x == 0 && blockIdx.x < nb) {
-        Body B = bodies[blockIdx.x];
-        if (finish_prev) kick2(B, dt);
-        if (ext) {                     // this step's external force and torque (host-written, mapped)
-            const int b = blockIdx.x;
-            for (int a = 0; a < 3; ++a) {
-                B.F_ext[a] = ext[3 * b + a];
-                B.T_ext[a] = ext[3 * nb + 3 * b + a];
-            }
-        }
-        kick_drift(B, dt);
-        bodies[blockIdx.x] = B;
-        record_body(rec, B, blockIdx.x, nb);
+    // one body per block, so the FP64 work of the bodies spreads over SMs
+    if (threadIdx.x < 32 && blockIdx.x < nb) {
+        Body *B = bodies + blockIdx.x;
+        if (finish_prev) body_update<true, true>(B, threadIdx.x, dt, ext, blockIdx.x, nb, rec);
+        else body_update<false, true>(B, threadIdx.x, dt, ext, blockIdx.x, nb, rec);
     }
     if (!tiles) return;
     // one thread per (listed tile, node of the tile): zero the force, drop the flag
@@ -61,19 +51,16 @@ __global__ void k_step_pre(Body *bodies, int nb, int finish_prev, T *F, int *til
 // device error word, so the host reads them without a copy.
 __global__ void k_finish(Body *bodies, int nb, double dt, unsigned long long *step, unsigned int by, double *out,
                          const int *err) {
-    const int b = blockIdx.x;
-    if (threadIdx.x != 0) return;
+    const int b = blockIdx.x, lane = threadIdx.x;
     if (b < nb) {
-        Body B = bodies[b];
-        kick2(B, dt);
-        bodies[b] = B;
-        if (out)
-            for (int a = 0; a < 3; ++a) {
-                out[6 * b + a] = B.F_tot[a];
-                out[6 * b + 3 + a] = B.T_tot[a];
-            }
+        const Recorder none{};
+        body_update<true, false>(bodies + b, lane, dt, nullptr, b, nb, none);
+        if (out && lane < 3) {           // as this lane wrote them
+            out[6 * b + lane] = bodies[b].F_tot[lane];
+            out[6 * b + 3 + lane] = bodies[b].T_tot[lane];
+        }
     }
-    if (b == 0) {
+    if (b == 0 && lane == 0) {
         *step += by;
         if (out) out[6 * nb] = err ? (double)*err : 0.0;
     }
@@ -84,13 +71,7 @@ __global__ void k_finish(Body *bodies, int nb, double dt, unsigned long long *st
 // record after the last substep's drift).
 __global__ void k_substep(Body *bodies, int nb, double dt, Recorder rec) {
     const int b = blockIdx.x;
-    if (threadIdx.x == 0 && b < nb) {
-        Body B = bodies[b];
-        kick2(B, dt);
-        kick_drift(B, dt);
-        bodies[b] = B;
-        record_body(rec, B, b, nb);
-    }
+    if (b < nb) body_update<true, true>(bodies + b, threadIdx.x, dt, nullptr, b, nb, rec);
 }
 
 __global__ void k_wall_beads(const WallBeads w, Body *bodies, const double *s, const int *bead_body, int nbeads) {
