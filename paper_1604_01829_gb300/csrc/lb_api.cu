@@ -109,10 +109,10 @@ lb_status upload_bodies(lb_ctx *h) {
         }
         LB_CUDA(h, cudaMemsetAsync(h->dFbead, 0, sizeof(double) * 3 * (size_t)std::max(nbeads, 1), h->stream));
         // host-mapped body I/O; without it (allocation refused) the copies below serve
-        if (cudaHostAlloc((void **)&h->io_map, sizeof(double) * (12 * (size_t)nb + 1), cudaHostAllocMapped) == cudaSuccess &&
+        if (cudaHostAlloc((void **)&h->io_map, sizeof(double) * (25 * (size_t)nb + 1), cudaHostAllocMapped) == cudaSuccess &&
             cudaHostGetDevicePointer((void **)&h->io_dmap, h->io_map, 0) == cudaSuccess &&
             cudaEventCreateWithFlags(&h->ev_io, cudaEventDisableTiming) == cudaSuccess) {
-            std::memset(h->io_map, 0, sizeof(double) * (12 * (size_t)nb + 1));
+            std::memset(h->io_map, 0, sizeof(double) * (25 * (size_t)nb + 1));
             for (int b = 0; b < nb; ++b)
                 for (int a = 0; a < 3; ++a) {
                     h->io_map[3 * b + a] = h->hb[b].F_ext[a];
@@ -131,8 +131,8 @@ lb_status upload_bodies(lb_ctx *h) {
             if ((s = dev_alloc(h, &h->Fbuf[k], fbytes)) != LB_OK) return s;
             if ((s = dev_alloc(h, &h->tiles[k], tbytes)) != LB_OK) return s;
             if ((s = dev_alloc(h, &h->tlist[k], sizeof(int) * (size_t)h->list_cap)) != LB_OK) return s;
-            if ((s = dev_alloc(h, &h->tcount[k], sizeof(int))) != LB_OK) return s;
-            LB_CUDA(h, cudaMemsetAsync(h->tcount[k], 0, sizeof(int), h->stream));
+            if ((s = dev_alloc(h, &h->tcount[k], 2 * sizeof(int))) != LB_OK) return s;
+            LB_CUDA(h, cudaMemsetAsync(h->tcount[k], 0, 2 * sizeof(int), h->stream));
             LB_CUDA(h, cudaMemsetAsync(h->Fbuf[k], 0, fbytes, h->stream));
             LB_CUDA(h, cudaMemsetAsync(h->tiles[k], 0, tbytes, h->stream));
         }
@@ -201,6 +201,8 @@ lbk::FluidArgs fluid_args(const lb_ctx *h, int cur, uint32_t step_off) {
     a.g = h->g;
     a.f = h->f;
     a.masks = h->dmask;
+    a.fpos = h->dfpos;
+    a.nfpos = h->nfpos;
     // MRT coefficients with c_k = w_diag / b_k = (1/36) / b_k folded in
     static const double bk[19] = {1.0, 1.0 / 3, 1.0 / 3, 1.0 / 3, 2.0 / 3, 4.0 / 3, 4.0 / 9, 1.0 / 9, 1.0 / 9,
                                   1.0 / 9, 2.0 / 3, 2.0 / 3, 2.0 / 3, 2.0 / 9, 2.0 / 9, 2.0 / 9, 2.0, 4.0 / 3,
@@ -467,7 +469,7 @@ lb_status lb_destroy(lb_handle h) {
     lbk::adj_free(h);
     void *bufs[] = {h->f, h->gforce, h->gforce_f, h->step_dev, h->err_dev, h->Fbuf[0], h->Fbuf[1], h->tiles[0], h->tiles[1],
                     h->tlist[0], h->tlist[1], h->tcount[0], h->tcount[1],
-                    h->db, h->ds, h->dsf, h->dbody_of, h->dFbead, h->partials, h->out4, h->rec, h->dmask, h->dwchan};
+                    h->db, h->ds, h->dsf, h->dbody_of, h->dFbead, h->partials, h->out4, h->rec, h->dmask, h->dfpos, h->dwchan};
     for (void *b : bufs)
         if (b) cudaFree(b);
     for (cudaEvent_t e : h->ev) cudaEventDestroy(e);
@@ -509,6 +511,32 @@ lb_status lb_set_pore(lb_handle h, double radius, int axis) {
     lb_status s = dev_alloc(h, &h->dmask, sizeof(uint32_t) * (size_t)lbk::pore_section_size(h->g));
     if (s != LB_OK) return s;
     LB_CUDA(h, lbk::launch_build_masks(h->g, h->dmask, h->stream));
+    // the fluid positions among them, so that the fluid kernel has no threads
+    // on wall nodes
+    std::vector<uint32_t> mask((size_t)lbk::pore_section_size(h->g));
+    LB_CUDA(h, cudaMemcpyAsync(mask.data(), h->dmask, mask.size() * sizeof(uint32_t), cudaMemcpyDeviceToHost,
+                               h->stream));
+    LB_CUDA(h, cudaStreamSynchronize(h->stream));
+    const int na = axis == 0 ? h->g.ny : h->g.nx;
+    std::vector<uint4> pos;
+    for (size_t k = 0; k < mask.size(); ++k)
+        if (!(mask[k] >> 31)) {
+            uint4 r;
+            r.x = (uint32_t)(k % na);
+            r.y = (uint32_t)(k / na);
+            r.z = mask[k];
+            r.w = 0;
+            pos.push_back(r);
+        }
+    if (h->dfpos) {
+        cudaFree(h->dfpos);
+        h->dfpos = nullptr;
+    }
+    h->nfpos = (int)pos.size();
+    if (!pos.empty()) {
+        if ((s = dev_alloc(h, &h->dfpos, sizeof(uint4) * pos.size())) != LB_OK) return s;
+        LB_CUDA(h, cudaMemcpy(h->dfpos, pos.data(), sizeof(uint4) * pos.size(), cudaMemcpyHostToDevice));
+    }
     // populations of new wall nodes are never read; nothing else changes
     return LB_OK;
 }
@@ -621,6 +649,7 @@ lb_status lb_set_body_state(lb_handle h, int id, const double X[3], const double
         if (!(qn > 0.0)) return fail(h, LB_ERR_ARG, "quaternion must be non-zero");
         for (int a = 0; a < 4; ++a) b.q[a] = q[a] / qn;
     }
+    h->out_fresh = false;
     return push_bodies(h);
 }
 
@@ -669,7 +698,8 @@ namespace {
 // previous step's second half kick if finish_prev, this step's kick and
 // drift, the clearing of its spread-force tiles. On stream `st`. The first
 // step of a group (k = 0) has no fluid kernel of this group beside it, so its
-// clearing takes a full-GPU grid.
+// clearing takes a full-GPU grid. The list of this buffer's tiles is left
+// empty for the step's coupling.
 lb_status launch_step_prologue(lb_ctx *h, int k, bool finish_prev, cudaStream_t st) {
     const int nb = (int)h->hb.size();
     const bool coupled = nb > 0 && !h->hbody_of.empty();
@@ -682,8 +712,6 @@ lb_status launch_step_prologue(lb_ctx *h, int k, bool finish_prev, cudaStream_t 
                                          h->list_cap, h->g, h->ntx, h->nty, rec, st, 1.0 / nsub, h->io_dmap,
                                          k == 0);
     if (e != cudaSuccess) return cuda_fail(h, e, "step_pre launch");
-    // the list of this buffer restarts empty for this step's coupling
-    if (coupled) LB_CUDA(h, cudaMemsetAsync(h->tcount[cur], 0, sizeof(int), st));
     return LB_OK;
 }
 
@@ -733,10 +761,9 @@ lb_status launch_step_coupling(lb_ctx *h, int k, int sub) {
     c.ntiles = (long long)h->ntx * h->nty * h->ntz;
     c.list_cap = h->list_cap;
     c.nbodies = (int)h->hb.size();
+    c.wall = h->wall;
     cudaError_t e = lbk::launch_couple(c, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "couple launch");
-    e = lbk::launch_wall_beads(h->wall, h->db, h->ds, h->dbody_of, nbeads, h->stream);
-    if (e != cudaSuccess) return cuda_fail(h, e, "wall beads launch");
     return LB_OK;
 }
 
@@ -996,6 +1023,19 @@ lb_status lb_forces_all(lb_handle h, int nbodies, double *F, double *T) {
 lb_status lb_get_body(lb_handle h, int id, double X[3], double V[3], double q[4], double w[3]) {
     if (check_handle(h) != LB_OK) return LB_ERR_ARG;
     if (id < 0 || id >= (int)h->hb.size()) return fail(h, LB_ERR_ARG, "bad body id");
+    if (h->io_map && h->out_fresh) {
+        // as the last group's finishing launch left it in host-mapped memory
+        LB_CUDA(h, cudaStreamSynchronize(h->stream));
+        const double *st = h->io_map + 12 * h->hb.size() + 1 + 13 * (size_t)id;
+        for (int a = 0; a < 3; ++a) {
+            if (X) X[a] = st[a];
+            if (V) V[a] = st[3 + a];
+            if (w) w[a] = st[10 + a];
+        }
+        if (q)
+            for (int a = 0; a < 4; ++a) q[a] = st[6 + a];
+        return LB_OK;
+    }
     lb_status s = pull_bodies(h);
     if (s != LB_OK) return s;
     const Body &b = h->hb[id];

@@ -292,6 +292,7 @@ struct BatchCouple {
     double dt, noise_scale;       // MD substep length 1/n; bead noise amplitude factor sqrt(n)
     float dt_f;                  // dt rounded to FP32
     uint32_t call;                // Philox call word of the bead noise: 4 + substep
+    int any_wall;                 // some instance has pore-wall beads
 };
 
 // 1: lb_batch_step launches every step eagerly instead of replaying the
@@ -355,24 +356,15 @@ __global__ void __maxnreg__(sizeof(T) == 4 ? LB_BATCH_COUPLE_REGS : 255) k_batch
     a.step_base = b.step_base;
     a.step_off = b.step_off;
     couple_bead<T>(a, k, active ? b.bead_rng[k] : 0, t & 7, threadIdx.x & 31, active);
-}
-
-// pore-wall beads of each bead's instance (one thread per bead)
-__global__ void k_batch_wall(const BInst *inst, Body *bodies, const double *s, const int *bead_body, int nbeads,
-                             int nbodies, int *err) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nbeads) return;
-    const BInst &I = inst[bodies[chk(bead_body[k], nbodies, err)].inst];
-    if (!I.wall.on) return;
-    const WallBeads w = I.wall;
-    wall_bead_body(w, bodies, s, bead_body, k);
+    if (b.any_wall && active && (t & 7) == 1 && I.wall.on)
+        couple_wall(I.wall, b.bodies, chk(b.bead_body[k], b.nbodies, b.err), b.s, k);
 }
 
 // previous step's second half kick (optional), this step's kick and drift,
 // and the clearing of every flagged tile of this step's force pool
 template <typename T>
 __global__ void k_batch_pre(Body *bodies, int nb, int finish_prev, T *F, int *tiles, const int *tlist,
-                            const int *tcount, const BInst *inst, const long long *flag_start, int n,
+                            int *tcount, const BInst *inst, const long long *flag_start, int n,
                             Recorder rec, int list_cap, long long ttot, int *err, double dt) {
     const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (threadIdx.x < 32 && blockIdx.x < nb) {     // one body per block
@@ -404,6 +396,7 @@ __global__ void k_batch_pre(Body *bodies, int nb, int finish_prev, T *F, int *ti
         }
         if (l == 0) tiles[gt] = 0;
     }
+    restart_list(tcount);
 }
 
 template <typename T>
@@ -504,8 +497,14 @@ struct lb_batch_ctx {
     // schedule
     int TS = 128, bpsm = 8, order = 0, ntiles = 0, sms = 0;
     int resident[2] = {0, 0};               // resident CTAs per SM of the even / odd fluid kernel at TS threads
-    // graph of two steps
-    cudaGraphExec_t gexec = nullptr;
+    // graphs of two steps and of eight
+    cudaGraphExec_t gexec = nullptr, gexec8 = nullptr;
+    // force and torque totals, the error word and the states of the bodies in
+    // host-mapped pinned memory, written at the end of each group of steps
+    // (layout of k_finish); out: 0 not those of the current state, 1 written by
+    // steps still queued, 2 ready to read
+    double *io_map = nullptr, *io_dmap = nullptr;
+    int out = 0;
     bool any_wall = false;                  // some instance has pore-wall beads
     // fluid positions (BInst::loff) of the pore instances and their compact
     // layout's position map and neighbour table (Geom::cmap, Geom::cnbr)
@@ -558,6 +557,14 @@ lb_status balloc(lb_batch_ctx *h, P **ptr, size_t bytes) {
     if (e != cudaSuccess) return bfail(h, LB_ERR_CUDA, std::string("cudaMalloc: ") + cudaGetErrorString(e));
     h->dev_bytes += bytes;
     return LB_OK;
+}
+
+void drop_graphs(lb_batch_ctx *h) {
+    for (cudaGraphExec_t *g : {&h->gexec, &h->gexec8})
+        if (*g) {
+            cudaGraphExecDestroy(*g);
+            *g = nullptr;
+        }
 }
 
 void fill_coll(const lb_params &p, BInst &I) {
@@ -646,10 +653,7 @@ lb_status rebuild_schedule(lb_batch_ctx *h) {
     BCUDA(h, cudaMemcpyAsync(h->dtile_start, ts.data(), sizeof(int) * (h->n + 1), cudaMemcpyHostToDevice, h->stream));
     BCUDA(h, cudaMemcpyAsync(h->dtile_inst, ti.data(), sizeof(int) * (size_t)acc, cudaMemcpyHostToDevice, h->stream));
     BCUDA(h, cudaStreamSynchronize(h->stream));
-    if (h->gexec) {
-        cudaGraphExecDestroy(h->gexec);
-        h->gexec = nullptr;
-    }
+    drop_graphs(h);
     // resident CTAs of the even- and odd-step fluid kernels at this tile size
     // (their register counts differ): each parity's persistent grid never
     // exceeds its own, so every CTA runs concurrently
@@ -831,16 +835,26 @@ lb_status upload(lb_batch_ctx *h) {
             for (int j = 0; j < nbeads; ++j) h->hbead_inst[j] = h->hb[h->hbody_of[j]].inst;
             BCUDA(h, cudaMemcpyAsync(h->dbead_inst, h->hbead_inst.data(), sizeof(int) * nbeads, cudaMemcpyHostToDevice, h->stream));
         }
+        // host-mapped totals and states; without it (allocation refused) they are copied
+        const size_t mb = sizeof(double) * (19 * (size_t)nb + 1);
+        if (cudaHostAlloc((void **)&h->io_map, mb, cudaHostAllocMapped) == cudaSuccess &&
+            cudaHostGetDevicePointer((void **)&h->io_dmap, h->io_map, 0) == cudaSuccess) {
+            std::memset(h->io_map, 0, mb);
+        } else {
+            cudaGetLastError();
+            if (h->io_map) cudaFreeHost(h->io_map);
+            h->io_map = h->io_dmap = nullptr;
+        }
         const size_t fb = (h->fp32 ? sizeof(float) : sizeof(double)) * 3 * (size_t)h->Ftot;
         h->list_cap = (int)std::min<long long>(h->Ttot, 8LL * std::max(nbeads, 1));
         for (int k = 0; k < 2; ++k) {
             if ((s = balloc(h, &h->Fbuf[k], fb)) != LB_OK) return s;
             if ((s = balloc(h, &h->tiles[k], sizeof(int) * (size_t)h->Ttot)) != LB_OK) return s;
             if ((s = balloc(h, &h->tlist[k], sizeof(int) * (size_t)h->list_cap)) != LB_OK) return s;
-            if ((s = balloc(h, &h->tcount[k], sizeof(int))) != LB_OK) return s;
+            if ((s = balloc(h, &h->tcount[k], 2 * sizeof(int))) != LB_OK) return s;
             BCUDA(h, cudaMemsetAsync(h->Fbuf[k], 0, fb, h->stream));
             BCUDA(h, cudaMemsetAsync(h->tiles[k], 0, sizeof(int) * (size_t)h->Ttot, h->stream));
-            BCUDA(h, cudaMemsetAsync(h->tcount[k], 0, sizeof(int), h->stream));
+            BCUDA(h, cudaMemsetAsync(h->tcount[k], 0, 2 * sizeof(int), h->stream));
         }
     }
     BCUDA(h, cudaStreamSynchronize(h->stream));
@@ -885,7 +899,6 @@ lb_status launch_step(lb_batch_ctx *h, int k, bool finish_prev, bool record, boo
                 coupled ? h->tiles[cur] : nullptr, h->tlist[cur], h->tcount[cur], h->dinst, h->dflag_start, h->n,
                 rec, h->list_cap, h->Ttot, h->derr, dt);
         BCUDA(h, cudaGetLastError());
-        if (coupled) BCUDA(h, cudaMemsetAsync(h->tcount[cur], 0, sizeof(int), ps));
         if (side) {
             BCUDA(h, cudaEventRecord(h->ev_join, h->side));
             BCUDA(h, cudaStreamWaitEvent(h->stream, h->ev_join, 0));
@@ -920,7 +933,9 @@ lb_status launch_step(lb_batch_ctx *h, int k, bool finish_prev, bool record, boo
         c.dt = dt;
         c.noise_scale = std::sqrt((double)nsub);
         c.dt_f = (float)dt;
-        const unsigned grid = (unsigned)((8LL * nbeads + 127) / 128);
+        c.any_wall = h->any_wall ? 1 : 0;
+        const int cb = lbk::couple_block(nbeads);
+        const unsigned grid = (unsigned)((8LL * nbeads + cb - 1) / cb);
         for (int sub = 0; sub < nsub; ++sub) {
             if (sub > 0) {   // bodies move by dt between the couplings of one LB step
                 const lbk::Recorder rec{sub == nsub - 1 ? h->rec : nullptr, h->rec_every, h->rec_cap, h->step_dev,
@@ -928,14 +943,9 @@ lb_status launch_step(lb_batch_ctx *h, int k, bool finish_prev, bool record, boo
                 BCUDA(h, lbk::launch_substep(h->db, nb, dt, rec, h->stream));
             }
             c.call = 4u + (uint32_t)sub;
-            if (h->fp32) lbk::k_batch_couple<float><<<grid, 128, 0, h->stream>>>(c);
-            else lbk::k_batch_couple<double><<<grid, 128, 0, h->stream>>>(c);
+            if (h->fp32) lbk::k_batch_couple<float><<<grid, cb, 0, h->stream>>>(c);
+            else lbk::k_batch_couple<double><<<grid, cb, 0, h->stream>>>(c);
             BCUDA(h, cudaGetLastError());
-            if (h->any_wall) {
-                lbk::k_batch_wall<<<(nbeads + 127) / 128, 128, 0, h->stream>>>(h->dinst, h->db, h->ds, h->dbody_of,
-                                                                              nbeads, nb, h->derr);
-                BCUDA(h, cudaGetLastError());
-            }
         }
     }
     if (nb > 0 && more && side) {               // the next prologue may start now
@@ -998,7 +1008,8 @@ lb_status launch_step(lb_batch_ctx *h, int k, bool finish_prev, bool record, boo
 
 lb_status finish_steps(lb_batch_ctx *h, int nsteps) {
     const int nb = (int)h->hb.size();
-    BCUDA(h, lbk::launch_finish(h->db, nb, 1.0 / h->nsub, h->step_dev, (unsigned)nsteps, h->stream));
+    BCUDA(h, lbk::launch_finish(h->db, nb, 1.0 / h->nsub, h->step_dev, (unsigned)nsteps, h->stream, h->io_dmap,
+                                h->derr));
     return LB_OK;
 }
 
@@ -1022,21 +1033,25 @@ lb_status eager_steps(lb_batch_ctx *h, int nsteps) {
     return s;
 }
 
-// two steps (even, odd) + second half kick + counter advance, as one graph
-lb_status ensure_graph(lb_batch_ctx *h) {
-    if (h->gexec) return LB_OK;
+// two or eight steps from an even step count + second half kick + counter
+// advance, as one graph (eight: the closing launch and the graph's own launch
+// once per eight steps; 64 boxes of 24^3: 39.3 against 44.2 us per step with
+// pairs only, 256 uneven instances 677 against 686)
+lb_status ensure_graph(lb_batch_ctx *h, int n) {
+    cudaGraphExec_t &slot = n == 8 ? h->gexec8 : h->gexec;
+    if (slot) return LB_OK;
     cudaGraph_t graph = nullptr;
     BCUDA(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-    lb_status s = launch_step(h, 0, false, false, true);
-    if (s == LB_OK) s = launch_step(h, 1, true, false, false);
-    if (s == LB_OK) s = finish_steps(h, 2);
+    lb_status s = LB_OK;
+    for (int k = 0; k < n && s == LB_OK; ++k) s = launch_step(h, k, k > 0, false, k + 1 < n);
+    if (s == LB_OK) s = finish_steps(h, n);
     cudaError_t e = cudaStreamEndCapture(h->stream, &graph);
     if (s != LB_OK) {
         if (graph) cudaGraphDestroy(graph);
         return s;
     }
     if (e != cudaSuccess) return bfail(h, LB_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(e));
-    e = cudaGraphInstantiate(&h->gexec, graph, 0);
+    e = cudaGraphInstantiate(&slot, graph, 0);
     cudaGraphDestroy(graph);
     if (e != cudaSuccess) return bfail(h, LB_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
     return LB_OK;
@@ -1198,7 +1213,7 @@ lb_status lb_batch_destroy(lb_batch_handle h) {
     if (!h) return LB_OK;
     if (h->stream) cudaStreamSynchronize(h->stream);
     if (h->side) cudaStreamSynchronize(h->side);
-    if (h->gexec) cudaGraphExecDestroy(h->gexec);
+    drop_graphs(h);
     void *bufs[] = {h->pool, h->Fbuf[0], h->Fbuf[1], h->tiles[0], h->tiles[1], h->tlist[0], h->tlist[1], h->tcount[0],
                     h->tcount[1], h->dinst, h->dtile_start, h->dtile_inst,
                     h->dflag_start, h->step_dev, h->db, h->ds, h->dsf, h->dbody_of, h->dbead_rng, h->dbead_inst, h->dFbead, h->rec, h->dcmap, h->dcnbr, h->dfluid,
@@ -1206,6 +1221,7 @@ lb_status lb_batch_destroy(lb_batch_handle h) {
     for (void *b : bufs)
         if (b) cudaFree(b);
     if (h->herr) cudaFreeHost(h->herr);
+    if (h->io_map) cudaFreeHost(h->io_map);
     for (cudaEvent_t e : h->ev) cudaEventDestroy(e);
     if (h->ev_fork) cudaEventDestroy(h->ev_fork);
     if (h->ev_join) cudaEventDestroy(h->ev_join);
@@ -1298,10 +1314,22 @@ lb_status lb_batch_add_raspberry(lb_batch_handle h, int k, const double *beads, 
     return LB_OK;
 }
 
+namespace {
+lb_status step_batch(lb_batch_ctx *h, int nsteps);
+}
+
 lb_status lb_batch_step(lb_batch_handle h, int nsteps) {
     if (!h) return bfail(nullptr, LB_ERR_ARG, "null handle");
     if (nsteps < 0) return bfail(h, LB_ERR_ARG, "nsteps must be >= 0");
     if (nsteps == 0) return LB_OK;
+    h->out = 0;
+    const lb_status s = step_batch(h, nsteps);
+    if (s == LB_OK && h->io_map) h->out = 1;
+    return s;
+}
+
+namespace {
+lb_status step_batch(lb_batch_ctx *h, int nsteps) {
     lb_status s = upload(h);
     if (s != LB_OK) return s;
     if (h->timing || LB_BATCH_EAGER) return eager_steps(h, nsteps);
@@ -1309,15 +1337,18 @@ lb_status lb_batch_step(lb_batch_handle h, int nsteps) {
         if ((s = eager_steps(h, 1)) != LB_OK) return s;
         --nsteps;
     }
-    const int pairs = nsteps / 2;
-    if (pairs > 0) {
-        if ((s = ensure_graph(h)) != LB_OK) return s;
-        for (int r = 0; r < pairs; ++r) BCUDA(h, cudaGraphLaunch(h->gexec, h->stream));
-        h->step += 2LL * pairs;
+    for (const int n : {8, 2}) {
+        const int times = nsteps / n;
+        if (times == 0) continue;
+        if ((s = ensure_graph(h, n)) != LB_OK) return s;
+        for (int r = 0; r < times; ++r) BCUDA(h, cudaGraphLaunch(n == 8 ? h->gexec8 : h->gexec, h->stream));
+        h->step += (long long)n * times;
+        nsteps -= n * times;
     }
     if (nsteps & 1) return eager_steps(h, 1);
     return LB_OK;
 }
+}  // namespace
 
 lb_status lb_batch_record_bodies(lb_batch_handle h, int every, int capacity) {
     if (!h) return bfail(nullptr, LB_ERR_ARG, "null handle");
@@ -1330,10 +1361,7 @@ lb_status lb_batch_record_bodies(lb_batch_handle h, int every, int capacity) {
         h->rec = nullptr;
     }
     h->rec_every = h->rec_cap = 0;
-    if (h->gexec) {                        // the captured steps hold the old recorder
-        cudaGraphExecDestroy(h->gexec);
-        h->gexec = nullptr;
-    }
+    drop_graphs(h);
     if (every == 0) return LB_OK;
     lb_status s = upload(h);               // the body set is fixed from here on
     if (s != LB_OK) return s;
@@ -1361,13 +1389,38 @@ namespace {
 // Synchronises the stream (completing the copies the caller queued) and
 // returns LB_ERR_STATE once if an index check of a checked build failed
 // since the last check (the word is then cleared).
-lb_status bcheck_device(lb_batch_ctx *h) {
-    BCUDA(h, cudaMemcpyAsync(h->herr, h->derr, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-    BCUDA(h, cudaStreamSynchronize(h->stream));
-    if (*h->herr & 2) {
+lb_status berror_word(lb_batch_ctx *h, int e) {
+    if (e & 2) {
         BCUDA(h, cudaMemsetAsync(h->derr, 0, sizeof(int), h->stream));
         return bfail(h, LB_ERR_STATE, "an index check of the checked build failed (an index outside its array)");
     }
+    return LB_OK;
+}
+
+lb_status bcheck_device(lb_batch_ctx *h) {
+    BCUDA(h, cudaMemcpyAsync(h->herr, h->derr, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    BCUDA(h, cudaStreamSynchronize(h->stream));
+    if (*h->herr && h->io_map) h->io_map[6 * h->hb.size()] = 0.0;   // reported here, not again from the mapped copy
+    return berror_word(h, *h->herr);
+}
+
+// The mapped totals and states, once the steps that write them have run
+// (nullptr: not those of the current state, read by copies).
+lb_status mapped_out(lb_batch_ctx *h, const double **out) {
+    *out = nullptr;
+    if (h->out == 0) return LB_OK;
+    if (h->out == 1) {
+        BCUDA(h, cudaStreamSynchronize(h->stream));
+        h->out = 2;
+    }
+    const size_t nb = h->hb.size();
+    const int e = (int)h->io_map[6 * nb];
+    if (e) {
+        h->io_map[6 * nb] = 0.0;
+        lb_status s = berror_word(h, e);
+        if (s != LB_OK) return s;
+    }
+    *out = h->io_map;
     return LB_OK;
 }
 
@@ -1382,6 +1435,15 @@ lb_status lb_batch_forces(lb_batch_handle h, int k, int body, double F[3], doubl
         for (int a = 0; a < 3; ++a) { if (F) F[a] = 0; if (T) T[a] = 0; }
         return LB_OK;
     }
+    const double *out = nullptr;
+    if ((s = mapped_out(h, &out)) != LB_OK) return s;
+    if (out) {
+        for (int a = 0; a < 3; ++a) {
+            if (F) F[a] = out[6 * id + a];
+            if (T) T[a] = out[6 * id + 3 + a];
+        }
+        return LB_OK;
+    }
     if (F) BCUDA(h, cudaMemcpyAsync(F, &h->db[id].F_tot[0], 3 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     if (T) BCUDA(h, cudaMemcpyAsync(T, &h->db[id].T_tot[0], 3 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     return bcheck_device(h);
@@ -1392,6 +1454,18 @@ lb_status lb_batch_get_body(lb_batch_handle h, int k, int body, double X[3], dou
     if (s != LB_OK) return s;
     if (body < 0 || body >= (int)h->inst_bodies[k].size()) return bfail(h, LB_ERR_ARG, "bad body id");
     const int id = h->inst_bodies[k][body];
+    const double *out = nullptr;
+    if ((s = mapped_out(h, &out)) != LB_OK) return s;
+    if (out) {
+        const double *st = out + 6 * h->hb.size() + 1 + 13 * (size_t)id;
+        for (int a = 0; a < 3; ++a) {
+            if (X) X[a] = st[a];
+            if (V) V[a] = st[3 + a];
+            if (w) w[a] = st[10 + a];
+        }
+        if (q) for (int a = 0; a < 4; ++a) q[a] = st[6 + a];
+        return LB_OK;
+    }
     Body b = h->hb[id];
     if (h->uploaded) {
         BCUDA(h, cudaMemcpyAsync(&b, &h->db[id], sizeof(Body), cudaMemcpyDeviceToHost, h->stream));
@@ -1566,11 +1640,9 @@ lb_status lb_batch_autotune(lb_batch_handle h, int trial_steps, int chosen[3], d
     release();
     h->timing = timing;
     h->rec = rec_saved;
+    h->out = 0;                       // the mapped totals are a trial's
     if (s != LB_OK) {
-        if (h->gexec) {
-            cudaGraphExecDestroy(h->gexec);
-            h->gexec = nullptr;
-        }
+        drop_graphs(h);
         return s;
     }
     s = lb_batch_set_schedule(h, bt, bb, bo);
@@ -1690,10 +1762,7 @@ lb_status lb_batch_checkpoint_load(lb_batch_handle h, const void *host, size_t b
         c.body_bytes != mine.body_bytes || c.total != mine.total)
         return bfail(h, LB_ERR_STATE, "the checkpoint was taken from a batch with other instances or bodies");
     if (bytes < c.total) return bfail(h, LB_ERR_ARG, "buffer shorter than the checkpoint");
-    if (h->gexec) {                        // the captured steps start from the saved parity again
-        cudaGraphExecDestroy(h->gexec);
-        h->gexec = nullptr;
-    }
+    drop_graphs(h);
     const char *p = static_cast<const char *>(host) + sizeof(c);
     for (auto &sec : batch_ckpt_sections(h)) {
         BCUDA(h, cudaMemcpyAsync(sec.first, p, sec.second, cudaMemcpyHostToDevice, h->stream));
@@ -1703,6 +1772,7 @@ lb_status lb_batch_checkpoint_load(lb_batch_handle h, const void *host, size_t b
     BCUDA(h, cudaMemcpyAsync(h->step_dev, &st, sizeof(st), cudaMemcpyHostToDevice, h->stream));
     BCUDA(h, cudaStreamSynchronize(h->stream));
     h->step = c.step;
+    h->out = 0;
     return LB_OK;
 }
 

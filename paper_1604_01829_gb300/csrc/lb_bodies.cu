@@ -19,7 +19,7 @@ namespace {
 // flagged 4x4x4 tiles of this step's spread-force buffer.
 template <typename T>
 __global__ void k_step_pre(Body *bodies, int nb, int finish_prev, T *F, int *tiles, const int *tlist,
-                           const int *tcount, Geom g, int ntx, int nty, Recorder rec, double dt, const double *ext) {
+                           int *tcount, Geom g, int ntx, int nty, Recorder rec, double dt, const double *ext) {
     const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     // one body per block, so the FP64 work of the bodies spreads over SMs
     if (threadIdx.x < 32 && blockIdx.x < nb) {
@@ -43,21 +43,31 @@ __global__ void k_step_pre(Body *bodies, int nb, int finish_prev, T *F, int *til
         }
         if (l == 0) tiles[tile] = 0;
     }
+    restart_list(tcount);
 }
 
 // The end of a group of steps in one launch: the last step's second half
 // kick (one body per block) and the advance of the device step counter;
-// with `out` (host-mapped) also every body's force and torque totals and the
-// device error word, so the host reads them without a copy.
+// with `out` (host-mapped) also every body's force and torque totals (6 a
+// body), the device error word and every body's X, V, q, w (13 a body), so
+// the host reads them without a copy.
 __global__ void k_finish(Body *bodies, int nb, double dt, unsigned long long *step, unsigned int by, double *out,
                          const int *err) {
     const int b = blockIdx.x, lane = threadIdx.x;
     if (b < nb) {
         const Recorder none{};
         body_update<true, false>(bodies + b, lane, dt, nullptr, b, nb, none);
-        if (out && lane < 3) {           // as this lane wrote them
-            out[6 * b + lane] = bodies[b].F_tot[lane];
-            out[6 * b + 3 + lane] = bodies[b].T_tot[lane];
+        if (out) {                       // each lane what it wrote itself (X and q are the prologue's)
+            const Body &B = bodies[b];
+            double *st = out + 6 * nb + 1 + 13 * b;
+            if (lane < 3) {
+                out[6 * b + lane] = B.F_tot[lane];
+                out[6 * b + 3 + lane] = B.T_tot[lane];
+                st[lane] = B.X[lane];
+                st[3 + lane] = B.V[lane];
+                st[10 + lane] = B.w[lane];
+            }
+            if (lane < 4) st[6 + lane] = B.q[lane];
         }
     }
     if (b == 0 && lane == 0) {
@@ -74,11 +84,6 @@ __global__ void k_substep(Body *bodies, int nb, double dt, Recorder rec) {
     if (b < nb) body_update<true, true>(bodies + b, threadIdx.x, dt, nullptr, b, nb, rec);
 }
 
-__global__ void k_wall_beads(const WallBeads w, Body *bodies, const double *s, const int *bead_body, int nbeads) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < nbeads) wall_bead_body(w, bodies, s, bead_body, k);
-}
-
 // threads per block of the body prologue when it runs beside a fluid kernel
 #ifndef LB_PRE_BLOCK
 #define LB_PRE_BLOCK 256
@@ -90,16 +95,31 @@ __global__ void k_wall_beads(const WallBeads w, Body *bodies, const double *s, c
 #define LB_COUPLE_REGS 64
 #endif
 template <typename T>
-__global__ void __launch_bounds__(128) __maxnreg__(sizeof(T) == 4 ? LB_COUPLE_REGS : 255) k_couple(const CoupleArgs a) {
+__global__ void __launch_bounds__(128) __maxnreg__(sizeof(T) == 4 ? LB_COUPLE_REGS : 255) k_couple(const __grid_constant__ CoupleArgs a) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int k = t >> 3;
     couple_bead<T>(a, k, k, t & 7, threadIdx.x & 31, k < a.nbeads);
+    if (a.wall.on && k < a.nbeads && (t & 7) == 1) 
+        couple_wall(a.wall, a.bodies, chk(a.bead_body[k], a.nbodies, a.err), a.s, k);
 }
 
 }  // namespace
 
+int sm_count() {
+    static const int sms = [] {     // initialised once, thread-safe
+        int dev = 0, n = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) !=
+                                                      cudaSuccess || n <= 0)
+            n = 152;
+        return n;
+    }();
+    return sms;
+}
+
+int couple_block(int nbeads) { return nbeads <= 16 * sm_count() ? 32 : 128; }
+
 cudaError_t launch_step_pre(Body *b, int nbodies, bool finish_prev, void *F, bool fp32, int *tiles, const int *tlist,
-                            const int *tcount, int list_cap, const Geom &g, int ntx, int nty, const Recorder &rec,
+                            int *tcount, int list_cap, const Geom &g, int ntx, int nty, const Recorder &rec,
                             cudaStream_t s, double dt, const double *ext, bool alone) {
     // one block per body, and for the tile clearing (grid-stride) at most a
     // quarter of the SMs' worth of blocks when the kernel runs beside the
@@ -108,13 +128,7 @@ cudaError_t launch_step_pre(Body *b, int nbodies, bool finish_prev, void *F, boo
     // 0.4372 ms against 0.4392 with a full-GPU grid, the step 0.4620 against
     // 0.4641); 8 blocks per SM when nothing runs beside it (the first step of
     // a group, e.g. every step of a one-step-per-call control loop)
-    static const int sms = [] {     // initialised once, thread-safe
-        int dev = 0, n = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) !=
-                                                      cudaSuccess || n <= 0)
-            n = 152;
-        return n;
-    }();
+    const int sms = sm_count();
     long long n = 64LL * list_cap;
     const int bs = alone ? 256 : LB_PRE_BLOCK;
     const long long cap = (alone ? 8LL * sms : (long long)(sms + 3) / 4) * bs;
@@ -128,16 +142,10 @@ cudaError_t launch_step_pre(Body *b, int nbodies, bool finish_prev, void *F, boo
 
 cudaError_t launch_couple(const CoupleArgs &a, cudaStream_t s) {
     if (a.nbeads <= 0) return cudaSuccess;
-    const unsigned grid = (unsigned)((8LL * a.nbeads + 127) / 128);
-    if (a.fp32) k_couple<float><<<grid, 128, 0, s>>>(a);
-    else k_couple<double><<<grid, 128, 0, s>>>(a);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_wall_beads(const WallBeads &w, Body *b, const double *s, const int *bead_body, int nbeads,
-                              cudaStream_t st) {
-    if (!w.on || nbeads <= 0) return cudaSuccess;
-    k_wall_beads<<<(nbeads + 127) / 128, 128, 0, st>>>(w, b, s, bead_body, nbeads);
+    const int block = couple_block(a.nbeads);
+    const unsigned grid = (unsigned)((8LL * a.nbeads + block - 1) / block);
+    if (a.fp32) k_couple<float><<<grid, block, 0, s>>>(a);
+    else k_couple<double><<<grid, block, 0, s>>>(a);
     return cudaGetLastError();
 }
 

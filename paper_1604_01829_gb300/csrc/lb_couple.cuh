@@ -90,12 +90,10 @@ __device__ __forceinline__ void wall_bead_force(const WallBeads &w, const double
     }
 }
 
-// Force and torque of the pore-wall beads on every bead of a body (one
-// thread per bead, FP64): added to the body's accumulators, not the fluid.
-__device__ __forceinline__ void wall_bead_body(const WallBeads &w, Body *bodies, const double *s,
-                                               const int *bead_body, int k) {
-    Body &B = bodies[bead_body[k]];
-    const double s0 = s[3 * k], s1 = s[3 * k + 1], s2 = s[3 * k + 2];
+// Force and torque of the pore-wall beads on bead k (FP64): added to the
+// body's accumulators, not the fluid. Out of line, so that the coupling's
+// registers do not include it: few beads come near the wall.
+inline __device__ __noinline__ void wall_bead_body(const WallBeads &w, Body &B, double s0, double s1, double s2) {
     double rel[3], r[3], F[3], tq[3];
     for (int q = 0; q < 3; ++q) {
         rel[q] = B.R[3 * q] * s0 + B.R[3 * q + 1] * s1 + B.R[3 * q + 2] * s2;
@@ -108,6 +106,20 @@ __device__ __forceinline__ void wall_bead_body(const WallBeads &w, Body *bodies,
         atomicAdd(&B.acc[q], F[q]);
         atomicAdd(&B.acc[3 + q], tq[q]);
     }
+}
+
+// The wall beads' part of a bead's coupling, by one lane: the bead is first
+// tested in FP32 (its distance from the axis to ~1e-5, against a margin of
+// 1e-3 of the wall's reach) and left alone when no wall bead can be near.
+__device__ __forceinline__ void couple_wall(const WallBeads &w, Body *bodies, int body, const double *s, int k) {
+    Body &B = bodies[body];
+    const int u = w.axis == 0 ? 1 : 0, v = w.axis == 2 ? 1 : 2;
+    const float s0 = (float)s[3 * k], s1 = (float)s[3 * k + 1], s2 = (float)s[3 * k + 2];
+    const float du = (float)(B.X[u] - w.cu) + (B.Rf[3 * u] * s0 + B.Rf[3 * u + 1] * s1 + B.Rf[3 * u + 2] * s2);
+    const float dv = (float)(B.X[v] - w.cv) + (B.Rf[3 * v] * s0 + B.Rf[3 * v + 1] * s1 + B.Rf[3 * v + 2] * s2);
+    const float near = w.reach_f;
+    if (near > 0.f && du * du + dv * dv < near * near) return;
+    wall_bead_body(w, B, s[3 * k], s[3 * k + 1], s[3 * k + 2]);
 }
 
 // Flags `tile` in the tile flags of this step's force buffer when this lane

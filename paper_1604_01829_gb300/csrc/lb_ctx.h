@@ -31,6 +31,8 @@ struct lb_ctx {
     int *err_dev = nullptr;                 // device error word of bounded waits
     int *err_host = nullptr;                // pinned host copy of it (read in the caller's synchronisation)
     uint32_t *dmask = nullptr;              // pore wall masks across the axis (launch_build_masks)
+    uint4 *dfpos = nullptr;                 // fluid positions across the pore axis (FluidArgs::fpos)
+    int nfpos = 0;
     double pore_R = 0.0;                    // pore radius (lb_set_pore)
     double *dwchan = nullptr;               // channel walls: Geom::wchan
     lbk::WallBeads wall{};                  // pore-wall beads (lb_set_pore_beads)
@@ -45,7 +47,7 @@ struct lb_ctx {
     void *Fbuf[2] = {nullptr, nullptr};     // [3][N] each, storage precision
     int *tiles[2] = {nullptr, nullptr};      // 4x4x4 tile flags of each force buffer
     int *tlist[2] = {nullptr, nullptr};      // flagged tiles of each buffer
-    int *tcount[2] = {nullptr, nullptr};     // entries of tlist
+    int *tcount[2] = {nullptr, nullptr};     // entries of tlist, and the clearing kernel's ticket
     int list_cap = 0;
     int ntx = 0, nty = 0, ntz = 0;
     // bodies
@@ -62,12 +64,13 @@ struct lb_ctx {
     // per-step body I/O in host-mapped pinned memory (Grace-Blackwell: the
     // GPU reads and writes it over the coherent chip-to-chip link, no copy):
     // [0, 6 nb) external forces then torques ([3 nb] each, host-written, read
-    // by each step's prologue), [6 nb, 12 nb) force and torque totals per body
-    // and [12 nb] the error word (written at the end of each group of steps)
+    // by each step's prologue), [6 nb, 12 nb) force and torque totals per body,
+    // [12 nb] the error word and then 13 nb values of X, V, q, w per body
+    // (written at the end of each group of steps)
     double *io_map = nullptr;          // host address
     double *io_dmap = nullptr;         // device address of the same memory
     cudaEvent_t ev_io = nullptr;       // after the last group that reads the external forces
-    bool out_fresh = false;            // the totals there are those of the current state
+    bool out_fresh = false;            // the totals and states there are those of the current state
     bool uploaded = false;
     // reductions
     double *partials = nullptr;

@@ -199,7 +199,8 @@ LB_FIX_FN bool collide_fix(const double (&f)[19], double (&o)[19], double Fx, do
     const L rho = v[0] + Sax + Sd;
     const L tx = d7 + d9 + d11 + d13, ty = d7 - d9 + d15 + d17, tz = d11 - d13 + d15 - d17;
 
-    const bool forced = Fx != 0.0 || Fy != 0.0 || Fz != 0.0;
+    // any component not 0 (tested as bits: no FP64 instruction)
+    const bool forced = ((fix_bits(Fx) | fix_bits(Fy) | fix_bits(Fz)) << 1) != 0;
     L Fq[3] = {0, 0, 0}, cF[3] = {0, 0, 0};
     if (forced) {
         const double F[3] = {Fx, Fy, Fz};

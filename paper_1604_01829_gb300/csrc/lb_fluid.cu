@@ -94,19 +94,30 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (NOISE ? LB_CS_MINB_NOIS
     using R = T;
     constexpr bool DEV = sizeof(T) == 4;
     const Geom &g = a.g;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
-    if (x >= g.nx || y >= g.ny) return;
+    int x = blockIdx.x * blockDim.x + threadIdx.x;
+    int y = blockIdx.y * blockDim.y + threadIdx.y;
+    int z = blockIdx.z;
+    uint32_t wmask = 0;                      // bit i: the upstream node x - c_i is a wall node
+    if (PORE && a.fpos) {
+        // one thread per fluid node: position j of the list across the axis,
+        // coordinate l along it (x fastest in either)
+        const int j = g.pore_axis == 0 ? y : x, l = g.pore_axis == 0 ? x : y;
+        if (j >= a.nfpos || l >= (g.pore_axis == 0 ? g.nx : (g.pore_axis == 1 ? g.ny : g.nz))) return;
+        const uint4 p = __ldg(a.fpos + j);
+        wmask = p.z;
+        if (g.pore_axis == 2) { x = (int)p.x; y = (int)p.y; z = l; }
+        else if (g.pore_axis == 1) { x = (int)p.x; y = l; z = (int)p.y; }
+        else { x = l; y = (int)p.x; z = (int)p.y; }
+    } else {
+        if (x >= g.nx || y >= g.ny) return;
+        if (PORE) {
+            wmask = __ldg(a.masks + pore_section_index(g, x, y, z));
+            if (wmask >> 31) return;         // wall node: holds no fluid
+        }
+    }
     T *A = static_cast<T *>(a.f);
     const long long N = g.N;
     const unsigned n = (unsigned)x + (unsigned)g.nx * ((unsigned)y + (unsigned)g.ny * (unsigned)z);
-
-    uint32_t wmask = 0;                      // bit i: the upstream node x - c_i is a wall node
-    if (PORE) {
-        wmask = __ldg(a.masks + pore_section_index(g, x, y, z));
-        if (wmask >> 31) return;             // wall node: holds no fluid
-    }
 
     // Neighbour node n + (dx, dy, dz) with periodic wrap (32-bit; the node
     // count is limited to 2^31 at creation), from per-axis wrapped offsets.
@@ -200,8 +211,27 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (NOISE ? LB_CS_MINB_NOIS
 }
 
 template <typename T, int COLL, bool NOISE, bool OOP = false>
-cudaError_t launch_cs_t(const FluidArgs &a, bool odd, dim3 block, cudaStream_t s) {
-    const dim3 grid((a.g.nx + block.x - 1) / block.x, (a.g.ny + block.y - 1) / block.y, a.g.nz);
+cudaError_t launch_cs_t(const FluidArgs &args, bool odd, dim3 block, cudaStream_t s) {
+    FluidArgs a = args;
+    dim3 grid((a.g.nx + block.x - 1) / block.x, (a.g.ny + block.y - 1) / block.y, a.g.nz);
+    if (a.fpos) {
+        // threads on the fluid nodes of a pore only: in the dense box a third
+        // to a half of them sit on wall nodes (48 x 48 x 96, R = 20: kernel
+        // FP64 35.4 -> 24.6 us, FP32 with noise 13.5 -> 11.0 us)
+        dim3 pb = block, pg;
+        if (a.g.pore_axis == 0) {
+            pg = dim3((a.g.nx + pb.x - 1) / pb.x, (a.nfpos + pb.y - 1) / pb.y, 1);
+        } else {
+            pb = dim3(block.x * block.y, 1, 1);
+            pg = dim3((a.nfpos + pb.x - 1) / pb.x, a.g.pore_axis == 1 ? a.g.ny : a.g.nz, 1);
+        }
+        if (pg.y <= 65535u) {
+            block = pb;
+            grid = pg;
+        } else {
+            a.fpos = nullptr;
+        }
+    }
     const bool pore = a.g.pore_axis >= 0 || a.g.chan;       // bounded: per-position wall masks
     if (odd) {
         if (pore) k_collide_stream<T, COLL, NOISE, true, true, OOP><<<grid, block, 0, s>>>(a);
@@ -427,6 +457,7 @@ bool make_wall_beads(const Geom &g, double pore_R, double spacing, double r_pore
     // a bead at radius rho >= Rc - rcut is at distance >= 2 sqrt(rho Rc) sin(dphi / 2)
     // from a wall bead dphi away around the axis, and >= |dz| along it
     const double rcut = std::sqrt(w.rcut2), rmin = w.Rc - rcut;
+    w.reach_f = (float)(rmin - 1e-3 * (1.0 + w.Rc));
     const double x = rmin > 0.0 ? rcut / (2.0 * std::sqrt(rmin * w.Rc)) : 2.0;
     w.wt = x >= 1.0 ? w.ntheta : (int)std::ceil(2.0 * std::asin(x) * w.ntheta / twopi + 0.5) + 1;
     w.wz = (int)std::ceil(rcut / (w.L / w.nrow) + 0.5) + 1;

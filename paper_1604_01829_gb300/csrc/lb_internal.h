@@ -58,6 +58,8 @@ struct FluidArgs {
     void *plane[19];             // base of each population plane (f + i N), uniform per launch
     const uint32_t *masks;       // pore: per position across the axis, bit 31 wall node, bit i the
                                  // upstream node of link i is a wall (launch_build_masks)
+    const uint4 *fpos;           // pore: fluid positions across the axis, {first coordinate, second, wall mask, 0}
+    int nfpos;                   // (null: one thread per node of the box)
     void *out[19];               // out-of-place step (launch_collide_stream_oop): where each plane's
                                  // populations are stored; the loads read f / plane
 };
@@ -91,6 +93,7 @@ struct WallBeads {
     int on, axis, ntheta, nrow, wt, wz;
     double cu, cv;               // axis position across it (box centre)
     double Rc, L, sigma2, rcut2, eps;
+    float reach_f;               // distance from the axis below which no wall bead is near, less a margin for FP32
 };
 
 // wall-bead parameters from the user's (host; lb_fluid.cu); false if invalid
@@ -111,7 +114,7 @@ struct CoupleArgs {
     const float *gforce_f;       // uniform force density rounded to FP32
     int *tiles_cur;              // flags of Fcur
     int *tlist;                  // flagged tiles of Fcur, in the order they were flagged
-    int *tcount;                 // entries of tlist
+    int *tcount;                 // entries of tlist (and, after it, the ticket of restart_list)
     int tile_base;               // added to tile indices recorded in tlist (batch pools)
     int ntx, nty;
     const double *s;             // body-frame bead offsets [3*nbeads]
@@ -134,6 +137,7 @@ struct CoupleArgs {
     double dt;
     float dt_f;
     uint32_t call;
+    WallBeads wall;              // pore-wall beads (single lattice)
 };
 
 // launchers (return the launch error)
@@ -177,7 +181,7 @@ struct Recorder {
 
 // dt: the MD (sub)step, 1 without substeps
 cudaError_t launch_step_pre(Body *b, int nbodies, bool finish_prev, void *F, bool fp32, int *tiles, const int *tlist,
-                            const int *tcount, int list_cap, const Geom &g, int ntx, int nty, const Recorder &rec,
+                            int *tcount, int list_cap, const Geom &g, int ntx, int nty, const Recorder &rec,
                             cudaStream_t s, double dt = 1.0, const double *ext = nullptr, bool alone = false);
 
 // The valid records of body `id` in a recorder ring, oldest first (host
@@ -189,6 +193,13 @@ cudaError_t copy_records(const double *ring, int every, int cap, long long k0, l
 cudaError_t launch_msd(const double *X, const double *q, int nrec, int nbodies, int max_lag, const double *p_ref,
                        void *work, double *out, cudaStream_t s);
 size_t msd_work_bytes(int nrec, int nbodies);
+// SMs of the current device
+int sm_count();
+// threads per block of the coupling kernels (4 beads a warp): one warp up to
+// four warps per SM, so that few beads spread over the SMs and their FP64
+// pipes and load units (224 beads, step of 32^3 FP64 18.3 against 19.0 us with
+// blocks of 128), else 128 (23,360 beads: 462.4 against 467.5 us with one warp)
+int couple_block(int nbeads);
 cudaError_t launch_couple(const CoupleArgs &a, cudaStream_t s);
 // end of a group of steps: second half kick of every body and the step
 // counter advance, in one launch (nbodies may be 0)
@@ -196,9 +207,6 @@ cudaError_t launch_finish(Body *b, int nbodies, double dt, unsigned long long *s
                           double *out = nullptr, const int *err = nullptr);
 // between MD substeps: second half kick, next first half kick and drift (dt each)
 cudaError_t launch_substep(Body *b, int nbodies, double dt, const Recorder &rec, cudaStream_t s);
-// force and torque of the pore-wall beads on every bead (after the coupling)
-cudaError_t launch_wall_beads(const WallBeads &w, Body *b, const double *s, const int *bead_body, int nbeads,
-                              cudaStream_t st);
 
 // host-side argument check: all n values finite (a null pointer passes)
 inline bool all_finite(const double *v, int n) {

