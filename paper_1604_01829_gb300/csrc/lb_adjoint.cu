@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(128) k_adj_couple(const AdjCouple a) {
     const int body = active ? a.bead_body[k] : 0;
     // kinematics of the step (translation-only or fixed bodies): FP64 storage
     // forms them here in FP64 as the FP64 coupling does; FP32 storage reads
-    // them as the body kernel prepared them for this step (k_adj_body_pre)
+    // them as the body kernel prepared them for this step (k_adj_body)
     Q Rm[9], Vp[3], wl[3];
     double Xp[3] = {0, 0, 0};
     const BodyAdj &BK = a.adj[body];
@@ -462,73 +462,88 @@ __global__ void __launch_bounds__(128) k_adj_couple(const AdjCouple a) {
     if (!fluid) lr[0] = lr[1] = lr[2] = Q(0);
     for (int off = 1; off < 8; off <<= 1)
         for (int q = 0; q < 3; ++q) lr[q] += __shfl_xor_sync(0xffffffffu, lr[q], off, 8);
-    if (active && c == 0) {
-        atomicAdd(a.lgam, (double)lg);
-        double lrel[3];
-        lrel[0] = (double)lr[0] + (double)(lv[1] * wl[2] - lv[2] * wl[1]);
-        lrel[1] = (double)lr[1] + (double)(lv[2] * wl[0] - lv[0] * wl[2]);
-        lrel[2] = (double)lr[2] + (double)(lv[0] * wl[1] - lv[1] * wl[0]);
-        for (int q = 0; q < 3; ++q)
-            a.dJds[3 * k + q] += (double)Rm[q] * lrel[0] + (double)Rm[3 + q] * lrel[1] + (double)Rm[6 + q] * lrel[2];
-        BodyAdj *BAw = a.adj + body;
-        for (int q = 0; q < 3; ++q) {
-            atomicAdd(&BAw->lXp[q], (double)lr[q]);
-            atomicAdd(&BAw->lVp[q], (double)lv[q]);
+    // the bead's own derivative, and its part of dJ/dgamma and of the body's
+    // adjoints: summed over the block's beads first (one atomic per value, body
+    // and block: with one body every bead's would go to the same address)
+    __shared__ double sum[16][7];
+    __shared__ int sbody[16];
+    const int slot = threadIdx.x >> 3, slots = blockDim.x >> 3;
+    if (c == 0) {
+        sbody[slot] = active ? body : -1;
+        if (active) {
+            double lrel[3];
+            lrel[0] = (double)lr[0] + (double)(lv[1] * wl[2] - lv[2] * wl[1]);
+            lrel[1] = (double)lr[1] + (double)(lv[2] * wl[0] - lv[0] * wl[2]);
+            lrel[2] = (double)lr[2] + (double)(lv[0] * wl[1] - lv[1] * wl[0]);
+            for (int q = 0; q < 3; ++q)
+                a.dJds[3 * k + q] += (double)Rm[q] * lrel[0] + (double)Rm[3 + q] * lrel[1] + (double)Rm[6 + q] * lrel[2];
+            for (int q = 0; q < 3; ++q) {
+                sum[slot][q] = (double)lr[q];
+                sum[slot][3 + q] = (double)lv[q];
+            }
+            sum[slot][6] = (double)lg;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < 7) {
+        const int q = threadIdx.x;
+        double acc = 0.0;
+        for (int i = 0; i < slots && sbody[i] >= 0; ++i) {
+            acc += sum[i][q];
+            const bool last = i + 1 == slots || sbody[i + 1] < 0;
+            if (q == 6) {
+                if (last) atomicAdd(a.lgam, acc);
+            } else if (last || sbody[i + 1] != sbody[i]) {
+                BodyAdj &W = a.adj[sbody[i]];
+                atomicAdd(q < 3 ? &W.lXp[q] : &W.lVp[q - 3], acc);
+                acc = 0.0;
+            }
         }
     }
 }
 
-// second half kick reversed (plus the objective's contribution)
-__global__ void k_adj_body_pre(const Body *bodies, BodyAdj *adj, int nb, int jb, int axis, double jw) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nb) return;
+// Between two reversed steps, one warp per body: the kick and drift of the
+// step whose coupling was reversed last (done, with the static parts of its
+// bodies), then the second half kick of the next one reversed, with the
+// objective's contribution, and that step's kinematics in FP32 as the body
+// prologue hands them to the FP32 coupling (bodies: taped before it).
+__global__ void k_adj_body(const Body *statics, bool done, const Body *bodies, BodyAdj *adj, int jb, int axis, double jw) {
+    const int b = blockIdx.x, lane = threadIdx.x, a = lane % 3;
     const Body &B = bodies[b];
     BodyAdj &A = adj[b];
-    // kick and drift of the step, then its kinematics in FP32 as the body
-    // prologue hands them to the FP32 coupling
-    double Rd[9];
-    quat_to_R(B.q, Rd);
-    const double w0[3] = {B.fixed == 2 ? 0.0 : B.w[0], B.fixed == 2 ? 0.0 : B.w[1], B.fixed == 2 ? 0.0 : B.w[2]};
-    for (int q = 0; q < 9; ++q) A.Rf[q] = (float)Rd[q];
-    for (int q = 0; q < 3; ++q) {
-        double vq = B.V[q], xq = B.X[q];
-        if (B.fixed == 2) {
-            vq += 0.5 * B.F_last[q] / B.mass;
-            xq += vq;
-        }
-        A.Vf[q] = (float)vq;
-        A.wlf[q] = (float)(Rd[3 * q] * w0[0] + Rd[3 * q + 1] * w0[1] + Rd[3 * q + 2] * w0[2]);
-        const double h = xq - 0.5, fl = floor(h);
-        A.Xi[q] = (int)fl;
-        A.Xf[q] = (float)(h - fl);
+    const int fixed = statics[b].fixed;
+    const double half_im = 0.5 * statics[b].inv_mass;
+    double lX = A.lX[a], lV = A.lV[a], lFl = A.lFl[a];
+    if (done) {
+        const double lXp = A.lXp[a], lvt = A.lVp[a] + lXp;
+        lX = fixed == 2 ? lXp : 0.0;
+        lV = fixed == 2 ? lvt : 0.0;
+        lFl = fixed == 2 ? lvt * half_im : 0.0;
     }
-    if (b == jb) A.lV[axis] += jw;
-    for (int q = 0; q < 3; ++q) {
-        A.lXp[q] = A.lX[q];
-        A.lFt[q] = A.lFl[q];
-        A.lVp[q] = 0.0;
-        if (B.fixed == 2) {
-            A.lVp[q] = A.lV[q];
-            A.lFt[q] += A.lV[q] / (2.0 * B.mass);
-        }
+    if (b == jb && a == axis) lV += jw;
+    double v = B.V[a], x = B.X[a];
+    if (fixed == 2) {
+        v += half_im * B.F_last[a];
+        x += v;
     }
-}
-
-// kick and drift reversed
-__global__ void k_adj_body_post(const Body *bodies, BodyAdj *adj, int nb) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nb) return;
-    const Body &B = bodies[b];
-    BodyAdj &A = adj[b];
-    for (int q = 0; q < 3; ++q) {
-        if (B.fixed == 2) {
-            const double lvt = A.lVp[q] + A.lXp[q];
-            A.lX[q] = A.lXp[q];
-            A.lV[q] = lvt;
-            A.lFl[q] = lvt / (2.0 * B.mass);
-        } else {
-            A.lX[q] = A.lV[q] = A.lFl[q] = 0.0;
-        }
+    const int l9 = lane < 9 ? lane : 0, i = l9 / 3, j = l9 - 3 * i;
+    const double R = rot_entry(B.q[0], B.q[1], B.q[2], B.q[3], i, j);
+    const double Rw = R * (fixed == 2 ? 0.0 : B.w[j]);
+    const double wl = __shfl_sync(0xffffffffu, Rw, 3 * a) + __shfl_sync(0xffffffffu, Rw, 3 * a + 1) +
+                      __shfl_sync(0xffffffffu, Rw, 3 * a + 2);
+    if (lane < 9) A.Rf[lane] = (float)R;
+    if (lane < 3) {
+        A.lX[a] = lX;
+        A.lV[a] = lV;
+        A.lFl[a] = lFl;
+        A.lXp[a] = lX;
+        A.lVp[a] = fixed == 2 ? lV : 0.0;
+        A.lFt[a] = fixed == 2 ? lFl + lV * half_im : lFl;
+        A.Vf[a] = (float)v;
+        A.wlf[a] = (float)wl;
+        const double h = x - 0.5, fl = floor(h);
+        A.Xi[a] = (int)fl;
+        A.Xf[a] = (float)(h - fl);
     }
 }
 
@@ -871,8 +886,17 @@ struct Run {
             }
             cudaEventRecord(ev[ev_used], s);
         }
+        // the bodies' reverse part (4-9 us of dependent FP64) needs the coupling
+        // of the step reversed before, the fluid's does not touch it: side by
+        // side, joined before this step's coupling
         const double jw = n >= nsteps - window ? 1.0 / window : 0.0;
-        lbk::k_adj_body_pre<<<(nb + 63) / 64, 64, 0, s>>>(bodies, w->adj, nb, jw != 0.0 ? body : -1, axis, jw);
+        cudaError_t e = cudaEventRecord(h->ev_fork, s);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(h->side, h->ev_fork, 0);
+        if (e != cudaSuccess) return fail_cuda(e, "adjoint fork");
+        lbk::k_adj_body<<<nb, 32, 0, h->side>>>(h->db, reversed > 0, bodies, w->adj, jw != 0.0 ? body : -1, axis, jw);
+        e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaEventRecord(h->ev_join, h->side);
+        if (e != cudaSuccess) return fail_cuda(e, "adjoint body launch");
         aa.fn = fn;
         aa.odd = ((n0 + n) & 1) != 0;
         aa.Fprev = Fprev;
@@ -884,7 +908,8 @@ struct Run {
         aa.lFp_out = w->lFp[cur ^ 1];
         if (h->fp32) lbk::k_adj_collide<float><<<grid, block, 0, s>>>(aa);
         else lbk::k_adj_collide<double><<<grid, block, 0, s>>>(aa);
-        cudaError_t e = cudaGetLastError();
+        e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(s, h->ev_join, 0);
         if (e != cudaSuccess) return fail_cuda(e, "adjoint collide launch");
         lbk::AdjCouple ac{};
         ac.g = h->g;
@@ -904,10 +929,10 @@ struct Run {
         ac.dJds = w->dJds;
         ac.lgam = w->lgam;
         ac.nbeads = nbeads;
-        const unsigned cg = (unsigned)((8LL * nbeads + 127) / 128);
-        if (h->fp32) lbk::k_adj_couple<float><<<cg, 128, 0, s>>>(ac);
-        else lbk::k_adj_couple<double><<<cg, 128, 0, s>>>(ac);
-        lbk::k_adj_body_post<<<(nb + 63) / 64, 64, 0, s>>>(bodies, w->adj, nb);
+        const int cb = lbk::couple_block(nbeads);
+        const unsigned cg = (unsigned)((8LL * nbeads + cb - 1) / cb);
+        if (h->fp32) lbk::k_adj_couple<float><<<cg, cb, 0, s>>>(ac);
+        else lbk::k_adj_couple<double><<<cg, cb, 0, s>>>(ac);
         e = cudaGetLastError();
         if (e != cudaSuccess) return fail_cuda(e, "adjoint coupling launch");
         if (timed) {
@@ -954,18 +979,16 @@ lb_status run_two_level(Run &R, int c) {
     // into the next entry (the last into the handle's array), so the tape is
     // written by the steps themselves.
     auto rerun = [&](int a0, int a1) -> lb_status {
+        std::vector<void *> f, F;
+        std::vector<Body *> bodies;
         for (int n = a0; n < a1; ++n) {
-            Tape &Tp = w->tape[n - a0];
-            const int curb = (int)((R.n0 + n) & 1);
-            cudaError_t ce = cudaMemcpyAsync(Tp.bodies, h->db, R.z.bbytes, cudaMemcpyDeviceToDevice, R.s);
-            if (ce != cudaSuccess) return R.fail_cuda(ce, "tape");
-            void *dst = n + 1 < a1 ? w->tape[n + 1 - a0].f : h->f;
-            lb_status st = lbk::ctx_step_oop(h, Tp.f, dst);
-            if (st != LB_OK) return st;
-            ce = cudaMemcpyAsync(Tp.Fnew, h->Fbuf[curb], R.z.Fbytes, cudaMemcpyDeviceToDevice, R.s);
-            if (ce != cudaSuccess) return R.fail_cuda(ce, "tape");
+            const Tape &Tp = w->tape[n - a0];
+            f.push_back(Tp.f);
+            F.push_back(Tp.Fnew);
+            bodies.push_back(Tp.bodies);
         }
-        return LB_OK;
+        f.push_back(h->f);
+        return lbk::ctx_tape_steps(h, a1 - a0, f.data(), bodies.data(), F.data(), R.z.Fbytes);
     };
     // A full segment re-runs the same steps on the same buffers whatever its
     // snapshot (entry 0 receives the snapshot's populations), so its launches

@@ -700,7 +700,7 @@ namespace {
 // step of a group (k = 0) has no fluid kernel of this group beside it, so its
 // clearing takes a full-GPU grid. The list of this buffer's tiles is left
 // empty for the step's coupling.
-lb_status launch_step_prologue(lb_ctx *h, int k, bool finish_prev, cudaStream_t st) {
+lb_status launch_step_prologue(lb_ctx *h, int k, bool finish_prev, cudaStream_t st, Body *snap = nullptr) {
     const int nb = (int)h->hb.size();
     const bool coupled = nb > 0 && !h->hbody_of.empty();
     const int cur = (int)((h->step + k) & 1);
@@ -710,7 +710,7 @@ lb_status launch_step_prologue(lb_ctx *h, int k, bool finish_prev, cudaStream_t 
     cudaError_t e = lbk::launch_step_pre(h->db, nb, finish_prev, coupled ? h->Fbuf[cur] : nullptr, h->fp32,
                                          coupled ? h->tiles[cur] : nullptr, h->tlist[cur], h->tcount[cur],
                                          h->list_cap, h->g, h->ntx, h->nty, rec, st, 1.0 / nsub, h->io_dmap,
-                                         k == 0);
+                                         k == 0, snap);
     if (e != cudaSuccess) return cuda_fail(h, e, "step_pre launch");
     return LB_OK;
 }
@@ -930,6 +930,48 @@ lb_status ctx_turn(lb_ctx *h, const void *src) {
     lb_status s = launch_step_prologue(h, 0, false, h->stream);
     if (s == LB_OK && !h->hbody_of.empty()) s = launch_step_coupling(h, 0, 0);
     h->f_src = nullptr;
+    return s;
+}
+
+// n steps (deterministic fluid) out of place for the adjoint's tape: step k
+// reads the populations at f[k] and stores the next at f[k + 1]; the bodies
+// before it go to bodies[k] (written by its prologue) and the spread force it
+// makes to F[k]. As in launch_steps the prologue of step k + 1 runs on the side
+// stream beside the fluid kernel of step k, and so does the copy of step k's
+// force (before the prologue of step k + 2 clears that buffer).
+lb_status ctx_tape_steps(lb_ctx *h, int n, void *const *f, Body *const *bodies, void *const *F, size_t Fbytes) {
+    LB_CUDA(h, cudaEventRecord(h->ev_fork, h->stream));
+    LB_CUDA(h, cudaStreamWaitEvent(h->side, h->ev_fork, 0));
+    lb_status s = launch_step_prologue(h, 0, false, h->side, bodies[0]);
+    for (int k = 0; k < n && s == LB_OK; ++k) {
+        const long long t = h->step + k;
+        const int cur = (int)(t & 1);
+        if (k == 0) {
+            LB_CUDA(h, cudaEventRecord(h->ev_join, h->side));
+            LB_CUDA(h, cudaStreamWaitEvent(h->stream, h->ev_join, 0));
+        }
+        h->f_src = f[k] != h->f ? f[k] : nullptr;
+        h->f_dst = f[k + 1] != h->f ? f[k + 1] : nullptr;
+        s = launch_step_coupling(h, k, 0);
+        const lbk::FluidArgs fa = fluid_args(h, cur, (uint32_t)k);
+        h->f_src = h->f_dst = nullptr;
+        if (s != LB_OK) break;
+        LB_CUDA(h, cudaEventRecord(h->ev_fork, h->stream));
+        LB_CUDA(h, cudaStreamWaitEvent(h->side, h->ev_fork, 0));
+        if (k + 1 < n) s = launch_step_prologue(h, k + 1, true, h->side, bodies[k + 1]);
+        if (s == LB_OK) s = timed_collide(h, fa, (t & 1) != 0);
+        if (s != LB_OK) break;
+        // the coupling of step k + 1 waits for the prologue, not for this copy
+        if (k + 1 < n) {
+            LB_CUDA(h, cudaEventRecord(h->ev_join, h->side));
+            LB_CUDA(h, cudaStreamWaitEvent(h->stream, h->ev_join, 0));
+        }
+        LB_CUDA(h, cudaMemcpyAsync(F[k], h->Fbuf[cur], Fbytes, cudaMemcpyDeviceToDevice, h->side));
+    }
+    LB_CUDA(h, cudaEventRecord(h->ev_join, h->side));
+    LB_CUDA(h, cudaStreamWaitEvent(h->stream, h->ev_join, 0));
+    if (s == LB_OK) s = finish_group(h, n);
+    h->step += n;
     return s;
 }
 

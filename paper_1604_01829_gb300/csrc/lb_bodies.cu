@@ -19,13 +19,14 @@ namespace {
 // flagged 4x4x4 tiles of this step's spread-force buffer.
 template <typename T>
 __global__ void k_step_pre(Body *bodies, int nb, int finish_prev, T *F, int *tiles, const int *tlist,
-                           int *tcount, Geom g, int ntx, int nty, Recorder rec, double dt, const double *ext) {
+                           int *tcount, Geom g, int ntx, int nty, Recorder rec, double dt, const double *ext, Body *snap) {
     const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     // one body per block, so the FP64 work of the bodies spreads over SMs
     if (threadIdx.x < 32 && blockIdx.x < nb) {
         Body *B = bodies + blockIdx.x;
-        if (finish_prev) body_update<true, true>(B, threadIdx.x, dt, ext, blockIdx.x, nb, rec);
-        else body_update<false, true>(B, threadIdx.x, dt, ext, blockIdx.x, nb, rec);
+        Body *sn = snap ? snap + blockIdx.x : nullptr;
+        if (finish_prev) body_update<true, true>(B, threadIdx.x, dt, ext, blockIdx.x, nb, rec, sn);
+        else body_update<false, true>(B, threadIdx.x, dt, ext, blockIdx.x, nb, rec, sn);
     }
     if (!tiles) return;
     // one thread per (listed tile, node of the tile): zero the force, drop the flag
@@ -120,7 +121,7 @@ int couple_block(int nbeads) { return nbeads <= 16 * sm_count() ? 32 : 128; }
 
 cudaError_t launch_step_pre(Body *b, int nbodies, bool finish_prev, void *F, bool fp32, int *tiles, const int *tlist,
                             int *tcount, int list_cap, const Geom &g, int ntx, int nty, const Recorder &rec,
-                            cudaStream_t s, double dt, const double *ext, bool alone) {
+                            cudaStream_t s, double dt, const double *ext, bool alone, Body *snap) {
     // one block per body, and for the tile clearing (grid-stride) at most a
     // quarter of the SMs' worth of blocks when the kernel runs beside the
     // fluid kernel of the previous step, whose blocks it would otherwise
@@ -135,8 +136,8 @@ cudaError_t launch_step_pre(Body *b, int nbodies, bool finish_prev, void *F, boo
     if (n > cap) n = cap;
     unsigned grid = (unsigned)((n + bs - 1) / bs);
     if (grid < (unsigned)nbodies) grid = (unsigned)nbodies;
-    if (fp32) k_step_pre<float><<<grid, bs, 0, s>>>(b, nbodies, finish_prev ? 1 : 0, (float *)F, tiles, tlist, tcount, g, ntx, nty, rec, dt, ext);
-    else k_step_pre<double><<<grid, bs, 0, s>>>(b, nbodies, finish_prev ? 1 : 0, (double *)F, tiles, tlist, tcount, g, ntx, nty, rec, dt, ext);
+    if (fp32) k_step_pre<float><<<grid, bs, 0, s>>>(b, nbodies, finish_prev ? 1 : 0, (float *)F, tiles, tlist, tcount, g, ntx, nty, rec, dt, ext, snap);
+    else k_step_pre<double><<<grid, bs, 0, s>>>(b, nbodies, finish_prev ? 1 : 0, (double *)F, tiles, tlist, tcount, g, ntx, nty, rec, dt, ext, snap);
     return cudaGetLastError();
 }
 

@@ -106,5 +106,6 @@ lb_status ctx_fail(lb_ctx *h, lb_status s, const std::string &m);
 // the prologue and coupling of the next step, reading the populations at src
 lb_status ctx_turn(lb_ctx *h, const void *src);
 lb_status ctx_step_oop(lb_ctx *h, const void *src, void *dst);
+lb_status ctx_tape_steps(lb_ctx *h, int n, void *const *f, Body *const *bodies, void *const *F, size_t Fbytes);
 void adj_free(lb_ctx *h);
 }  // namespace lbk

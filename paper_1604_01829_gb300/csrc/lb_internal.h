@@ -179,10 +179,12 @@ struct Recorder {
     uint32_t step_off;
 };
 
-// dt: the MD (sub)step, 1 without substeps
+// dt: the MD (sub)step, 1 without substeps; snap: the adjoint's copy of the
+// bodies before the step (body_update)
 cudaError_t launch_step_pre(Body *b, int nbodies, bool finish_prev, void *F, bool fp32, int *tiles, const int *tlist,
                             int *tcount, int list_cap, const Geom &g, int ntx, int nty, const Recorder &rec,
-                            cudaStream_t s, double dt = 1.0, const double *ext = nullptr, bool alone = false);
+                            cudaStream_t s, double dt = 1.0, const double *ext = nullptr, bool alone = false,
+                            Body *snap = nullptr);
 
 // The valid records of body `id` in a recorder ring, oldest first (host
 // arrays; lb_traj.cu).

@@ -21,9 +21,22 @@ __device__ __forceinline__ void quat_to_R(const double q[4], double R[9]) {
     R[6] = 2.0 * (x * z - y * w); R[7] = 2.0 * (y * z + x * w); R[8] = 1.0 - 2.0 * (x * x + y * y);
 }
 
+// entry (i, j) of quat_to_R
+__device__ __forceinline__ double rot_entry(double qw, double qx, double qy, double qz, int i, int j) {
+    if (i == j) {
+        const double u = i == 0 ? qy : qx, v = i == 2 ? qy : qz;
+        return 1.0 - 2.0 * (u * u + v * v);
+    }
+    const double u = i == 0 || j == 0 ? qx : qy, v = i == 2 || j == 2 ? qz : qy;
+    const double o = i + j == 1 ? qz : (i + j == 2 ? qy : qx);              // the third axis
+    const bool neg = j == i + 1 || (i == 2 && j == 0);                      // -w o for (0,1), (1,2), (2,0)
+    return 2.0 * (u * v + (neg ? -(o * qw) : o * qw));
+}
+
 // One body's update by one warp: the second half kick of the (sub)step that
 // has its coupling done (FINISH) and / or the first half kick and drift of the
-// next (START), over dt (1 without MD substeps, 1/n with n per LB step).
+// next (START), over dt (1 without MD substeps, 1/n with n per LB step). snap:
+// receives what the adjoint reads of the body's state between the two.
 //
 // Second half kick: totals F = beads + external and torque, V += dt F/(2M),
 // body-frame omega implicitly (6 fixed-point iterations), so that the two half
@@ -46,7 +59,7 @@ __device__ __forceinline__ void quat_to_R(const double q[4], double R[9]) {
 // substeps 54 -> 40 us, 64 boxes of 24^3 60 -> 47 us.
 template <bool FINISH, bool START>
 __device__ __forceinline__ void body_update(Body *B, int lane, double dt, const double *ext, int b, int nb,
-                                            const Recorder &rec) {
+                                            const Recorder &rec, Body *snap = nullptr) {
     constexpr unsigned FULL = 0xffffffffu;
     auto from = [&](double v, int src) { return __shfl_sync(FULL, v, src); };
     const int a = lane % 3, a1 = a == 2 ? 0 : a + 1, a2 = a == 0 ? 2 : a - 1;
@@ -86,6 +99,20 @@ __device__ __forceinline__ void body_update(Body *B, int lane, double dt, const 
         B->T_ext[a] = ext[3 * nb + 3 * b + a];
     }
     double X = B->X[a], q = B->q[lane & 3];
+    if (snap) {
+        if (lane < 3) {
+            snap->X[a] = X;
+            snap->V[a] = V;
+            snap->w[a] = w;
+            snap->F_last[a] = Fl;
+        }
+        if (lane < 4) snap->q[lane] = q;
+        if (lane == 0) {
+            snap->mass = B->mass;
+            snap->inv_mass = inv_mass;
+            snap->fixed = fixed;
+        }
+    }
     if (fixed != 1) {
         V += 0.5 * dt * Fl * inv_mass;
         X += dt * V;
@@ -136,16 +163,7 @@ __device__ __forceinline__ void body_update(Body *B, int lane, double dt, const 
     // rotation, lab = R body: R_ij of lane 3 i + j
     const double qw = from(q, 0), qx = from(q, 1), qy = from(q, 2), qz = from(q, 3);
     const int l9 = lane < 9 ? lane : 0, i = l9 / 3, j = l9 - 3 * i;
-    double R;
-    if (i == j) {
-        const double u = i == 0 ? qy : qx, v = i == 2 ? qy : qz;
-        R = 1.0 - 2.0 * (u * u + v * v);
-    } else {
-        const double u = i == 0 || j == 0 ? qx : qy, v = i == 2 || j == 2 ? qz : qy;
-        const double o = i + j == 1 ? qz : (i + j == 2 ? qy : qx);          // the third axis
-        const bool neg = j == i + 1 || (i == 2 && j == 0);                  // -w o for (0,1), (1,2), (2,0)
-        R = 2.0 * (u * v + (neg ? -(o * qw) : o * qw));
-    }
+    const double R = rot_entry(qw, qx, qy, qz, i, j);
     const double Rw = R * from(w, j);                       // lab omega: row sums of R_ij w_j
     const double wl = from(Rw, 3 * a) + from(Rw, 3 * a + 1) + from(Rw, 3 * a + 2);
     if (lane < 9) {
