@@ -102,20 +102,36 @@ LB_FIX_FN long long fix_in(double v, int cb, int &over) {
     return (int)hi < 0 ? -s : s;
 }
 
-// The double nearest (even) to V 2^(k - 61), |V| < 2^62; small: the smallest
-// upper half of |V| seen, 0 when a value is too small for this form.
-// ce = (1023 + k) << 20.
-LB_FIX_FN double fix_out(long long V, int ce, unsigned &small) {
+// The double nearest (even) to V 2^(k - 61), |V| < 2^62, by integer
+// instructions (~18): shift to bit 62, round, shift back. small: the smallest
+// upper half of |V| seen; 0: a value is too small for this form.
+LB_FIX_FN double fix_out(long long V, const FixParams &P, unsigned &small) {
     const unsigned sgn = (unsigned)((unsigned long long)V >> 32) & 0x80000000u;
     const unsigned long long A = (unsigned long long)(V < 0 ? -V : V);
     const unsigned ah = (unsigned)(A >> 32);
     small = small < ah ? small : ah;
-    const unsigned n = fix_clz(ah | 1u) - 1u;          // top bit to bit 62
+    const unsigned n = fix_clz(ah | 1u) - 1u;
     const unsigned long long w = A << n;
     const unsigned long long m = (w + (0x1FFu + (((unsigned)w >> 10) & 1u))) >> 10;
-    const unsigned h = (unsigned)(m >> 32) + (unsigned)ce - (n << 20) + sgn;
+    const unsigned h = (unsigned)(m >> 32) + (unsigned)P.ce - (n << 20) + sgn;
     return fix_double(((unsigned long long)h << 32) | (unsigned)m);
 }
+
+// The same by two additions on the FP64 pipe: the halves of V + 2^63 as the
+// low words of two doubles of fixed exponents, (2^84 + 2^32 (hi + 2^31)) and
+// (2^52 + lo) times 2^(k - 61); what was added is taken from the first
+// (exactly), and only the sum rounds. With every output by one form its pipe
+// is the bound (integer 65 % busy, or FP64 75 %): LB_FIX_OUT64 of the 19 take
+// this one.
+LB_FIX_FN double fix_out64(long long V, const FixParams &P) {
+    const unsigned hi = (unsigned)((unsigned long long)V >> 32) ^ 0x80000000u, lo = (unsigned)V;
+    const double a = fix_double(((unsigned long long)(unsigned)P.eh << 32) | hi);
+    const double b = fix_double(((unsigned long long)(unsigned)P.el << 32) | lo);
+    return (a - P.out) + b;
+}
+#ifndef LB_FIX_OUT64
+#define LB_FIX_OUT64 7
+#endif
 
 #ifdef __CUDACC__
 LB_FIX_FN float fix_rcp(float x) {
@@ -285,11 +301,12 @@ LB_FIX_FN bool collide_fix(const double (&f)[19], double (&o)[19], double Fx, do
     }
 
     unsigned small = 0xFFFFFFFFu;
-    o[0] = fix_out(v[0] + 12 * (q16 - q4), P.ce, small);
+    auto put = [&](int i, L V) { o[i] = i < LB_FIX_OUT64 ? fix_out64(V, P) : fix_out(V, P, small); };
+    put(0, v[0] + 12 * (q16 - q4));
     const L U = -2 * q16, V = q17 - q5, W = q6 - q18;
     auto pair2 = [&](int i, L E, L O) {
-        o[i] = fix_out(v[i] + E + O, P.ce, small);
-        o[i + 1] = fix_out(v[i + 1] + E - O, P.ce, small);
+        put(i, v[i] + E + O);
+        put(i + 1, v[i + 1] + E - O);
     };
     pair2(1, 2 * (U - 2 * V), 2 * (cF[0] - 2 * q10));
     pair2(3, 2 * (U + V + W), 2 * (cF[1] - 2 * q11));
@@ -363,6 +380,9 @@ inline FixParams fix_params(double rho0, double kT, const double rate[15]) {
     P.on = k > -600 && k < 600 && kT <= 0.01 * rho0 ? 1 : 0;
     P.cb = 1023 + k;
     P.ce = (1023 + k) * (1 << 20);
+    P.eh = (0x453 - 61 + k) * (1 << 20);
+    P.el = (0x433 - 61 + k) * (1 << 20);
+    P.out = std::ldexp(0x1p84 + 0x1p63 + 0x1p52, k - 61);
     P.fs = std::ldexp(1.0, 61 - k) / 12.0;
     static const long double b[15] = {2.0L / 3, 4.0L / 3, 4.0L / 9, 1.0L / 9, 1.0L / 9, 1.0L / 9, 2.0L / 3, 2.0L / 3,
                                       2.0L / 3, 2.0L / 9, 2.0L / 9, 2.0L / 9, 2.0L,     4.0L / 3, 4.0L / 9};

@@ -32,7 +32,8 @@ struct FixPair {
 };
 struct FixParams {
     int on;                      // 0: not usable for these parameters (FP64 arithmetic then)
-    int cb, ce;                  // exponent constants of the conversions
+    int cb, ce, eh, el;          // exponent constants of the conversions
+    double out;                  // what fix_out64 takes off
     double fs;                   // 2^(61 - k) / 12, k the exponent of the scaled unit
     FixPair ke[15];              // modes 4-18: c_k (1 - g_k) at 2^64
     FixPair ks[6];               // modes 4-9: c_k (1 + g_k) / 2 at 2^64
