@@ -37,6 +37,11 @@ lb_status cuda_fail(lb_ctx *h, cudaError_t e, const char *where) {
 #define LB_EAGER_NODES (1LL << 20)
 #endif
 
+// node count below which captured steps are chained launches (launch_chain)
+#ifndef LB_CHAIN_NODES
+#define LB_CHAIN_NODES (1LL << 20)
+#endif
+
 #define LB_CUDA(h, call)                                                  \
     do {                                                                  \
         cudaError_t e_ = (call);                                          \
@@ -436,7 +441,7 @@ lb_status lb_create(const lb_params *p, void *cuda_stream, lb_handle *out) {
     if ((s = dev_alloc(h, &h->f, es * 19 * (size_t)h->g.N)) != LB_OK ||
         (s = dev_alloc(h, &h->gforce, 3 * sizeof(double))) != LB_OK ||
         (s = dev_alloc(h, &h->gforce_f, 3 * sizeof(float))) != LB_OK ||
-        (s = dev_alloc(h, &h->step_dev, sizeof(unsigned long long))) != LB_OK ||
+        (s = dev_alloc(h, &h->step_dev, 2 * sizeof(unsigned long long))) != LB_OK ||
         (s = dev_alloc(h, &h->err_dev, sizeof(int))) != LB_OK) {
         g_create_error = h->err;
         lb_destroy(h);
@@ -449,7 +454,7 @@ lb_status lb_create(const lb_params *p, void *cuda_stream, lb_handle *out) {
         lb_destroy(h);
         return s;
     }
-    e = cudaMemsetAsync(h->step_dev, 0, sizeof(unsigned long long), h->stream);
+    e = cudaMemsetAsync(h->step_dev, 0, 2 * sizeof(unsigned long long), h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->err_dev, 0, sizeof(int), h->stream);
     if (e == cudaSuccess) e = lbk::launch_init(h->f, h->fp32, h->g.N, p->rho0, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
@@ -700,7 +705,8 @@ namespace {
 // step of a group (k = 0) has no fluid kernel of this group beside it, so its
 // clearing takes a full-GPU grid. The list of this buffer's tiles is left
 // empty for the step's coupling.
-lb_status launch_step_prologue(lb_ctx *h, int k, bool finish_prev, cudaStream_t st, Body *snap = nullptr) {
+lb_status launch_step_prologue(lb_ctx *h, int k, bool finish_prev, cudaStream_t st, Body *snap = nullptr,
+                               bool chain = false) {
     const int nb = (int)h->hb.size();
     const bool coupled = nb > 0 && !h->hbody_of.empty();
     const int cur = (int)((h->step + k) & 1);
@@ -710,13 +716,13 @@ lb_status launch_step_prologue(lb_ctx *h, int k, bool finish_prev, cudaStream_t 
     cudaError_t e = lbk::launch_step_pre(h->db, nb, finish_prev, coupled ? h->Fbuf[cur] : nullptr, h->fp32,
                                          coupled ? h->tiles[cur] : nullptr, h->tlist[cur], h->tcount[cur],
                                          h->list_cap, h->g, h->ntx, h->nty, rec, st, 1.0 / nsub, h->io_dmap,
-                                         k == 0, snap);
+                                         k == 0, snap, chain ? h->step_dev : nullptr);
     if (e != cudaSuccess) return cuda_fail(h, e, "step_pre launch");
     return LB_OK;
 }
 
 // The coupling of MD substep `sub` of step h->step + k on the main stream.
-lb_status launch_step_coupling(lb_ctx *h, int k, int sub) {
+lb_status launch_step_coupling(lb_ctx *h, int k, int sub, bool chain = false) {
     const int nbeads = (int)h->hbody_of.size();
     const long long t = h->step + k;
     const bool odd = (t & 1) != 0;
@@ -755,7 +761,7 @@ lb_status launch_step_coupling(lb_ctx *h, int k, int sub) {
     c.key0 = (uint32_t)h->p.seed;
     c.key1 = (uint32_t)(h->p.seed >> 32);
     c.instance = h->p.instance;
-    c.step_base = h->step_dev;
+    c.step_base = h->step_dev + (chain ? 1 : 0);
     c.step_off = (uint32_t)k;
     c.err = h->err_dev;
     c.ntiles = (long long)h->ntx * h->nty * h->ntz;
@@ -814,6 +820,64 @@ lb_status launch_steps(lb_ctx *h, int n) {
     return LB_OK;
 }
 
+// n steps of a lattice with beads as one chain of launches on the main stream:
+// a prologue, then per step the coupling (with MD substeps, the bodies'
+// updates and further couplings) and the fluid kernel, whose extra blocks do
+// the next step's prologue or, after the last step, the group's end. Two
+// launches a step and no second stream to fork and join, for the lattices whose
+// steps replay from graphs: there the launches and the gaps between them are
+// most of a step (32^3 FP64 17.8 -> 16.5 us, 64^3 16.9 -> 15.9, a 48 x 48 x 96
+// pore with two substeps 27.2 -> 25.9, thermal FP64 94 x 81 x 103 97.5 -> 88.0).
+// As programmatic dependent launches the same chain was slower (20.4, 15.6,
+// 26.7, 95.8 us): blocks that wait hold the slots of the kernel before.
+lb_status launch_chain(lb_ctx *h, int n) {
+    const int nb = (int)h->hb.size(), nsub = h->p.md_substeps;
+    const double dt = 1.0 / nsub;
+    const bool noise = h->p.collision == 1 && h->p.kT > 0.0;
+    lb_status s = launch_step_prologue(h, 0, false, h->stream, nullptr, true);
+    for (int k = 0; k < n && s == LB_OK; ++k) {
+        const long long t = h->step + k;
+        const int cur = (int)(t & 1), next = cur ^ 1;
+        for (int sub = 0; sub < nsub && s == LB_OK; ++sub) {
+            if (sub > 0) {
+                const lbk::Recorder rec{sub == nsub - 1 ? h->rec : nullptr, h->rec_every, h->rec_cap, h->step_dev + 1,
+                                        (uint32_t)k};
+                cudaError_t e = lbk::launch_substep(h->db, nb, dt, rec, h->stream);
+                if (e != cudaSuccess) return cuda_fail(h, e, "substep launch");
+            }
+            s = launch_step_coupling(h, k, sub, true);
+        }
+        if (s != LB_OK) return s;
+        lbk::FluidArgs a = fluid_args(h, cur, (uint32_t)k);
+        a.step_base = h->step_dev + 1;
+        lbk::StepExtra &x = a.ex;
+        const bool last = k + 1 == n;
+        x.mode = last ? 2 : 1;
+        // a block per body (up to 64), 32 for the clearing
+        x.body_blocks = std::min(nb, 64);
+        x.blocks = x.body_blocks + (last ? 0 : 32);
+        x.bodies = h->db;
+        x.nb = nb;
+        x.F = h->Fbuf[next];
+        x.tiles = h->tiles[next];
+        x.tlist = h->tlist[next];
+        x.tcount = h->tcount[next];
+        x.ntx = h->ntx;
+        x.nty = h->nty;
+        x.rec = lbk::Recorder{nsub == 1 ? h->rec : nullptr, h->rec_every, h->rec_cap, h->step_dev + 1, (uint32_t)(k + 1)};
+        x.dt = dt;
+        x.ext = h->io_dmap;
+        x.out = h->io_dmap ? h->io_dmap + 6 * h->hb.size() : nullptr;
+        x.err = h->err_dev;
+        x.step = h->step_dev;
+        x.by = (unsigned)n;
+        cudaError_t e = lbk::launch_collide_stream_chain(a, h->fp32, h->p.collision, noise, (t & 1) != 0, h->block,
+                                                         h->stream);
+        if (e != cudaSuccess) return cuda_fail(h, e, "chained collide_stream launch");
+    }
+    return s;
+}
+
 // end of a group of n steps: the last step's second half kick, counter advance
 lb_status finish_group(lb_ctx *h, int n) {
     cudaError_t e = lbk::launch_finish(h->db, (int)h->hb.size(), 1.0 / h->p.md_substeps, h->step_dev, (unsigned)n,
@@ -842,8 +906,13 @@ lb_status ensure_graph(lb_ctx *h, int n = 2) {
     if (slot) return LB_OK;
     cudaGraph_t graph = nullptr;
     LB_CUDA(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-    lb_status s = launch_steps(h, n);
-    if (s == LB_OK) s = finish_group(h, n);
+    lb_status s = LB_OK;
+    if (!h->hbody_of.empty() && h->g.N < LB_CHAIN_NODES && h->g.nz <= 65000) {
+        s = launch_chain(h, n);
+    } else {
+        s = launch_steps(h, n);
+        if (s == LB_OK) s = finish_group(h, n);
+    }
     cudaError_t e = cudaStreamEndCapture(h->stream, &graph);
     if (s != LB_OK) {
         if (graph) cudaGraphDestroy(graph);
@@ -887,16 +956,20 @@ lb_status step_groups(lb_ctx *h, int nsteps) {
     // the replayed graph (256^3: 0.4633 against 0.4672 ms; 128^3: 0.0769
     // against 0.0823), whatever the graph's length
     if (nsteps >= 4 && h->g.N >= LB_EAGER_NODES) return eager_steps(h, nsteps);
+    auto single = [&]() -> lb_status {
+        lb_status st = ensure_graph(h, 1);
+        if (st != LB_OK) return st;
+        LB_CUDA(h, cudaGraphLaunch(h->gexec1[h->step & 1], h->stream));
+        h->step += 1;
+        return LB_OK;
+    };
     if (nsteps < 4) {
-        for (int k = 0; k < nsteps; ++k) {
-            if ((s = ensure_graph(h, 1)) != LB_OK) return s;
-            LB_CUDA(h, cudaGraphLaunch(h->gexec1[h->step & 1], h->stream));
-            h->step += 1;
-        }
+        for (int k = 0; k < nsteps; ++k)
+            if ((s = single()) != LB_OK) return s;
         return LB_OK;
     }
     if (h->step & 1) {
-        if ((s = eager_steps(h, 1)) != LB_OK) return s;
+        if ((s = single()) != LB_OK) return s;
         --nsteps;
     }
     const int octets = nsteps / LB_GRAPH_STEPS;
@@ -912,7 +985,7 @@ lb_status step_groups(lb_ctx *h, int nsteps) {
         for (int r = 0; r < pairs; ++r) LB_CUDA(h, cudaGraphLaunch(h->gexec, h->stream));
         h->step += 2LL * pairs;
     }
-    if (nsteps & 1) return eager_steps(h, 1);
+    if (nsteps & 1) return single();
     return LB_OK;
 }
 }  // namespace

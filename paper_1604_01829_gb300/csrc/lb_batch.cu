@@ -396,7 +396,7 @@ __global__ void k_batch_pre(Body *bodies, int nb, int finish_prev, T *F, int *ti
         }
         if (l == 0) tiles[gt] = 0;
     }
-    restart_list(tcount);
+    restart_list(tcount, gridDim.x);
 }
 
 template <typename T>

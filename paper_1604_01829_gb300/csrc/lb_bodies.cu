@@ -19,7 +19,8 @@ namespace {
 // flagged 4x4x4 tiles of this step's spread-force buffer.
 template <typename T>
 __global__ void k_step_pre(Body *bodies, int nb, int finish_prev, T *F, int *tiles, const int *tlist,
-                           int *tcount, Geom g, int ntx, int nty, Recorder rec, double dt, const double *ext, Body *snap) {
+                           int *tcount, Geom g, int ntx, int nty, Recorder rec, double dt, const double *ext, Body *snap,
+                           unsigned long long *step) {
     const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     // one body per block, so the FP64 work of the bodies spreads over SMs
     if (threadIdx.x < 32 && blockIdx.x < nb) {
@@ -28,23 +29,10 @@ __global__ void k_step_pre(Body *bodies, int nb, int finish_prev, T *F, int *til
         if (finish_prev) body_update<true, true>(B, threadIdx.x, dt, ext, blockIdx.x, nb, rec, sn);
         else body_update<false, true>(B, threadIdx.x, dt, ext, blockIdx.x, nb, rec, sn);
     }
+    if (step && blockIdx.x == 0 && threadIdx.x == 0) step[1] = step[0];
     if (!tiles) return;
-    // one thread per (listed tile, node of the tile): zero the force, drop the flag
-    const long long total = 64LL * (*tcount);
-    for (long long i = t; i < total; i += (long long)gridDim.x * blockDim.x) {
-        const int tile = tlist[i >> 6];
-        const int l = (int)(i & 63);
-        const int tx = tile % ntx, ty = (tile / ntx) % nty, tz = tile / (ntx * nty);
-        const int x = 4 * tx + (l & 3), y = 4 * ty + ((l >> 2) & 3), z = 4 * tz + (l >> 4);
-        if (x < g.nx && y < g.ny && z < g.nz) {
-            const long long n = nidx(g, x, y, z);
-            F[n] = T(0);
-            F[g.N + n] = T(0);
-            F[2 * g.N + n] = T(0);
-        }
-        if (l == 0) tiles[tile] = 0;
-    }
-    restart_list(tcount);
+    clear_tiles(g, F, tiles, tlist, tcount, ntx, nty, t, (long long)gridDim.x * blockDim.x);
+    restart_list(tcount, gridDim.x);
 }
 
 // The end of a group of steps in one launch: the last step's second half
@@ -55,22 +43,7 @@ __global__ void k_step_pre(Body *bodies, int nb, int finish_prev, T *F, int *til
 __global__ void k_finish(Body *bodies, int nb, double dt, unsigned long long *step, unsigned int by, double *out,
                          const int *err) {
     const int b = blockIdx.x, lane = threadIdx.x;
-    if (b < nb) {
-        const Recorder none{};
-        body_update<true, false>(bodies + b, lane, dt, nullptr, b, nb, none);
-        if (out) {                       // each lane what it wrote itself (X and q are the prologue's)
-            const Body &B = bodies[b];
-            double *st = out + 6 * nb + 1 + 13 * b;
-            if (lane < 3) {
-                out[6 * b + lane] = B.F_tot[lane];
-                out[6 * b + 3 + lane] = B.T_tot[lane];
-                st[lane] = B.X[lane];
-                st[3 + lane] = B.V[lane];
-                st[10 + lane] = B.w[lane];
-            }
-            if (lane < 4) st[6 + lane] = B.q[lane];
-        }
-    }
+    if (b < nb) finish_body(bodies, b, nb, lane, dt, out);
     if (b == 0 && lane == 0) {
         *step += by;
         if (out) out[6 * nb] = err ? (double)*err : 0.0;
@@ -121,7 +94,8 @@ int couple_block(int nbeads) { return nbeads <= 16 * sm_count() ? 32 : 128; }
 
 cudaError_t launch_step_pre(Body *b, int nbodies, bool finish_prev, void *F, bool fp32, int *tiles, const int *tlist,
                             int *tcount, int list_cap, const Geom &g, int ntx, int nty, const Recorder &rec,
-                            cudaStream_t s, double dt, const double *ext, bool alone, Body *snap) {
+                            cudaStream_t s, double dt, const double *ext, bool alone, Body *snap,
+                            unsigned long long *step) {
     // one block per body, and for the tile clearing (grid-stride) at most a
     // quarter of the SMs' worth of blocks when the kernel runs beside the
     // fluid kernel of the previous step, whose blocks it would otherwise
@@ -136,8 +110,8 @@ cudaError_t launch_step_pre(Body *b, int nbodies, bool finish_prev, void *F, boo
     if (n > cap) n = cap;
     unsigned grid = (unsigned)((n + bs - 1) / bs);
     if (grid < (unsigned)nbodies) grid = (unsigned)nbodies;
-    if (fp32) k_step_pre<float><<<grid, bs, 0, s>>>(b, nbodies, finish_prev ? 1 : 0, (float *)F, tiles, tlist, tcount, g, ntx, nty, rec, dt, ext, snap);
-    else k_step_pre<double><<<grid, bs, 0, s>>>(b, nbodies, finish_prev ? 1 : 0, (double *)F, tiles, tlist, tcount, g, ntx, nty, rec, dt, ext, snap);
+    if (fp32) k_step_pre<float><<<grid, bs, 0, s>>>(b, nbodies, finish_prev ? 1 : 0, (float *)F, tiles, tlist, tcount, g, ntx, nty, rec, dt, ext, snap, step);
+    else k_step_pre<double><<<grid, bs, 0, s>>>(b, nbodies, finish_prev ? 1 : 0, (double *)F, tiles, tlist, tcount, g, ntx, nty, rec, dt, ext, snap, step);
     return cudaGetLastError();
 }
 

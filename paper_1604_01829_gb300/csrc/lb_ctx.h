@@ -27,7 +27,7 @@ struct lb_ctx {
     void *f_dst = nullptr;
     double *gforce = nullptr;               // device (3)
     float *gforce_f = nullptr;              // device (3), FP32 copy
-    unsigned long long *step_dev = nullptr; // device step counter
+    unsigned long long *step_dev = nullptr; // device step counter, and a chained group's start (launch_chain)
     int *err_dev = nullptr;                 // device error word of bounded waits
     int *err_host = nullptr;                // pinned host copy of it (read in the caller's synchronisation)
     uint32_t *dmask = nullptr;              // pore wall masks across the axis (launch_build_masks)

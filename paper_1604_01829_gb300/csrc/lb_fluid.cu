@@ -22,6 +22,7 @@
 #include <cmath>
 
 #include "lb_fix64.cuh"
+#include "lb_rigid.cuh"
 
 // Minimum resident blocks of 128 threads per SM requested for the FP32
 // collide kernels (caps their registers; FP64 kernels are not capped):
@@ -88,15 +89,26 @@ __device__ __forceinline__ uint32_t pore_section_index(const Geom &g, int x, int
 
 // ------------------------------------------------------- collide and stream
 
-template <typename T, int COLL, bool NOISE, bool ODD, bool PORE, bool OOP = false>
+template <typename T, int COLL, bool NOISE, bool ODD, bool PORE, bool OOP = false, bool CHAIN = false>
 __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (NOISE ? LB_CS_MINB_NOISE : LB_CS_MINB) : LB_CS_MINB_F64)
     k_collide_stream(const __grid_constant__ FluidArgs a) {
     using R = T;
     constexpr bool DEV = sizeof(T) == 4;
     const Geom &g = a.g;
+    int by = blockIdx.y, bz = blockIdx.z;
+    if (CHAIN) {
+        // the first planes (rows of a pore's grid) hold the extra blocks
+        int &plane = PORE && a.fpos ? by : bz;
+        if (plane < a.ex.planes) {
+            const int eb = blockIdx.x + gridDim.x * (PORE && a.fpos ? blockIdx.y : blockIdx.y + gridDim.y * blockIdx.z);
+            if (eb < a.ex.blocks) step_extra<T>(a.ex, g, eb);
+            return;
+        }
+        plane -= a.ex.planes;
+    }
     int x = blockIdx.x * blockDim.x + threadIdx.x;
-    int y = blockIdx.y * blockDim.y + threadIdx.y;
-    int z = blockIdx.z;
+    int y = by * blockDim.y + threadIdx.y;
+    int z = bz;
     uint32_t wmask = 0;                      // bit i: the upstream node x - c_i is a wall node
     if (PORE && a.fpos) {
         // one thread per fluid node: position j of the list across the axis,
@@ -210,7 +222,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (NOISE ? LB_CS_MINB_NOIS
     }
 }
 
-template <typename T, int COLL, bool NOISE, bool OOP = false>
+template <typename T, int COLL, bool NOISE, bool OOP = false, bool CHAIN = false>
 cudaError_t launch_cs_t(const FluidArgs &args, bool odd, dim3 block, cudaStream_t s) {
     FluidArgs a = args;
     dim3 grid((a.g.nx + block.x - 1) / block.x, (a.g.ny + block.y - 1) / block.y, a.g.nz);
@@ -225,20 +237,26 @@ cudaError_t launch_cs_t(const FluidArgs &args, bool odd, dim3 block, cudaStream_
             pb = dim3(block.x * block.y, 1, 1);
             pg = dim3((a.nfpos + pb.x - 1) / pb.x, a.g.pore_axis == 1 ? a.g.ny : a.g.nz, 1);
         }
-        if (pg.y <= 65535u) {
+        if (pg.y <= 65000u) {
             block = pb;
             grid = pg;
         } else {
             a.fpos = nullptr;
         }
     }
+    if (CHAIN) {
+        // the extra blocks in whole planes (rows) in front of the grid
+        const unsigned per = a.fpos ? grid.x : grid.x * grid.y;
+        a.ex.planes = (a.ex.blocks + per - 1) / per;
+        (a.fpos ? grid.y : grid.z) += a.ex.planes;
+    }
     const bool pore = a.g.pore_axis >= 0 || a.g.chan;       // bounded: per-position wall masks
     if (odd) {
-        if (pore) k_collide_stream<T, COLL, NOISE, true, true, OOP><<<grid, block, 0, s>>>(a);
-        else k_collide_stream<T, COLL, NOISE, true, false, OOP><<<grid, block, 0, s>>>(a);
+        if (pore) k_collide_stream<T, COLL, NOISE, true, true, OOP, CHAIN><<<grid, block, 0, s>>>(a);
+        else k_collide_stream<T, COLL, NOISE, true, false, OOP, CHAIN><<<grid, block, 0, s>>>(a);
     } else {
-        if (pore) k_collide_stream<T, COLL, NOISE, false, true, OOP><<<grid, block, 0, s>>>(a);
-        else k_collide_stream<T, COLL, NOISE, false, false, OOP><<<grid, block, 0, s>>>(a);
+        if (pore) k_collide_stream<T, COLL, NOISE, false, true, OOP, CHAIN><<<grid, block, 0, s>>>(a);
+        else k_collide_stream<T, COLL, NOISE, false, false, OOP, CHAIN><<<grid, block, 0, s>>>(a);
     }
     return cudaGetLastError();
 }
@@ -421,6 +439,18 @@ cudaError_t launch_collide_stream(const FluidArgs &a, bool fp32, int collision, 
     if (collision == 0) return launch_cs_t<double, 0, false>(a, odd, block, s);
     if (noise) return launch_cs_t<double, 1, true>(a, odd, block, s);
     return launch_cs_t<double, 1, false>(a, odd, block, s);
+}
+
+cudaError_t launch_collide_stream_chain(const FluidArgs &a, bool fp32, int collision, bool noise, bool odd, dim3 block,
+                                        cudaStream_t s) {
+    if (fp32) {
+        if (collision == 0) return launch_cs_t<float, 0, false, false, true>(a, odd, block, s);
+        if (noise) return launch_cs_t<float, 1, true, false, true>(a, odd, block, s);
+        return launch_cs_t<float, 1, false, false, true>(a, odd, block, s);
+    }
+    if (collision == 0) return launch_cs_t<double, 0, false, false, true>(a, odd, block, s);
+    if (noise) return launch_cs_t<double, 1, true, false, true>(a, odd, block, s);
+    return launch_cs_t<double, 1, false, false, true>(a, odd, block, s);
 }
 
 cudaError_t launch_collide_stream_oop(const FluidArgs &a, bool fp32, int collision, bool odd, dim3 block,

@@ -40,6 +40,61 @@ struct FixParams {
     FixPair kn[15];              // modes 4-18: noise amplitude over sqrt(rho) of the scaled unit, at 2^64
 };
 
+// Rigid bodies (FP64, array of structs; few bodies, one thread each).
+struct Body {
+    double X[3], V[3], q[4], w[3];   // centre, velocity, orientation (w,x,y,z), body-frame omega
+    double F_last[3], T_last[3];     // last step: lab-frame force, body-frame torque
+    double F_ext[3], T_ext[3];       // lab frame
+    double F_tot[3], T_tot[3];       // last step: lab-frame totals (beads + external)
+    double acc[6];                   // bead force / torque accumulators of the running step
+    double R[9];                     // rotation of the running step (row-major, lab = R body)
+    double wl[3];                    // lab-frame omega of the running step
+    double mass, I[3];
+    double inv_mass, inv_I[3];       // reciprocals, so the step divides nothing
+    // the running step's state in FP32 for the FP32 coupling: rotation,
+    // velocity, lab omega, and X - 1/2 split into floor (Xi) and fraction (Xf)
+    float Rf[9], Vf[3], wlf[3], Xf[3];
+    int Xi[3];
+    int fixed;
+    int inst;                        // instance of a batch (0 for a single lattice)
+};
+
+// Trajectory recorder: after the drift of step t, if (t + 1) % every == 0,
+// the step prologue writes every body's centre and orientation (7 doubles,
+// X then q) into record slot ((t + 1) / every - 1) % cap of `ring`
+// ([cap][nbodies][7]). ring == nullptr: off.
+struct Recorder {
+    double *ring;
+    int every, cap;
+    const unsigned long long *step_base;
+    uint32_t step_off;
+};
+
+// What the extra blocks of a chained fluid kernel (launch_collide_stream_chain)
+// do beside its fluid blocks: mode 1, the next step's prologue (every body's
+// second half kick of this step, first half kick and drift of the next, and
+// the clearing of the next step's spread-force tiles); mode 2, the end of a
+// group (second half kick, results to `out`, advance of the step counter).
+struct StepExtra {
+    int blocks, planes;          // extra blocks, and the grid planes (rows of a pore's grid) they lie in;
+    int body_blocks;             // the first of them for the bodies, the others for the clearing
+    int mode;
+    Body *bodies;
+    int nb;
+    void *F;
+    int *tiles;
+    const int *tlist;
+    int *tcount;
+    int ntx, nty;
+    Recorder rec;
+    double dt;
+    const double *ext;
+    double *out;
+    const int *err;
+    unsigned long long *step;
+    unsigned by;
+};
+
 // Everything the fused collide-and-stream kernel reads besides populations.
 struct FluidArgs {
     Geom g;
@@ -61,27 +116,9 @@ struct FluidArgs {
                                  // upstream node of link i is a wall (launch_build_masks)
     const uint4 *fpos;           // pore: fluid positions across the axis, {first coordinate, second, wall mask, 0}
     int nfpos;                   // (null: one thread per node of the box)
+    StepExtra ex;                // chained kernels
     void *out[19];               // out-of-place step (launch_collide_stream_oop): where each plane's
                                  // populations are stored; the loads read f / plane
-};
-
-// Rigid bodies (FP64, array of structs; few bodies, one thread each).
-struct Body {
-    double X[3], V[3], q[4], w[3];   // centre, velocity, orientation (w,x,y,z), body-frame omega
-    double F_last[3], T_last[3];     // last step: lab-frame force, body-frame torque
-    double F_ext[3], T_ext[3];       // lab frame
-    double F_tot[3], T_tot[3];       // last step: lab-frame totals (beads + external)
-    double acc[6];                   // bead force / torque accumulators of the running step
-    double R[9];                     // rotation of the running step (row-major, lab = R body)
-    double wl[3];                    // lab-frame omega of the running step
-    double mass, I[3];
-    double inv_mass, inv_I[3];       // reciprocals, so the step divides nothing
-    // the running step's state in FP32 for the FP32 coupling: rotation,
-    // velocity, lab omega, and X - 1/2 split into floor (Xi) and fraction (Xf)
-    float Rf[9], Vf[3], wlf[3], Xf[3];
-    int Xi[3];
-    int fixed;
-    int inst;                        // instance of a batch (0 for a single lattice)
 };
 
 // Repulsive pore-wall beads (Sec. 2.3): beads on the cylinder of radius Rc
@@ -145,6 +182,9 @@ struct CoupleArgs {
 cudaError_t launch_init(void *f, bool fp32, long long N, double rho0, cudaStream_t s);
 cudaError_t launch_collide_stream(const FluidArgs &a, bool fp32, int collision, bool noise, bool odd,
                                   dim3 block, cudaStream_t s);
+// the same with the extra blocks of a.ex in front of the fluid's
+cudaError_t launch_collide_stream_chain(const FluidArgs &a, bool fp32, int collision, bool noise, bool odd, dim3 block,
+                                        cudaStream_t s);
 // the same step out of place (deterministic fluid): loads from f / plane,
 // stores into out, in the AA layout of the next step; every slot of a fluid
 // node is written, the slots of wall nodes are not
@@ -169,23 +209,13 @@ cudaError_t launch_sample(const void *f, bool fp32, const Geom &g, bool odd, dou
 cudaError_t launch_moments(const void *f, bool fp32, const Geom &g, bool odd, double *partials,
                            int nblocks, double *out4, cudaStream_t s);
 
-// Trajectory recorder: after the drift of step t, if (t + 1) % every == 0,
-// the step prologue writes every body's centre and orientation (7 doubles,
-// X then q) into record slot ((t + 1) / every - 1) % cap of `ring`
-// ([cap][nbodies][7]). ring == nullptr: off.
-struct Recorder {
-    double *ring;
-    int every, cap;
-    const unsigned long long *step_base;
-    uint32_t step_off;
-};
-
 // dt: the MD (sub)step, 1 without substeps; snap: the adjoint's copy of the
-// bodies before the step (body_update)
+// bodies before the step (body_update); step: step[1] = step[0] (a chained
+// group's kernels count from step[1], which its end leaves alone)
 cudaError_t launch_step_pre(Body *b, int nbodies, bool finish_prev, void *F, bool fp32, int *tiles, const int *tlist,
                             int *tcount, int list_cap, const Geom &g, int ntx, int nty, const Recorder &rec,
                             cudaStream_t s, double dt = 1.0, const double *ext = nullptr, bool alone = false,
-                            Body *snap = nullptr);
+                            Body *snap = nullptr, unsigned long long *step = nullptr);
 
 // The valid records of body `id` in a recorder ring, oldest first (host
 // arrays; lb_traj.cu).

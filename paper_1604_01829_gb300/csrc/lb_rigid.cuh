@@ -199,13 +199,75 @@ __device__ __forceinline__ void body_update(Body *B, int lane, double dt, const 
 // kernel has read its length: the last block to arrive (count[1] is the
 // ticket, left at 0) resets it, in place of a memset node in the step's chain
 // (48 x 48 x 96 pore with two substeps 37 -> 28 us per step, 64^3 23 -> 17).
-__device__ __forceinline__ void restart_list(int *count) {
+__device__ __forceinline__ void restart_list(int *count, int blocks) {
     __syncthreads();
-    if (threadIdx.x != 0) return;
+    if (threadIdx.x != 0 || threadIdx.y != 0) return;
     __threadfence();
-    if (atomicAdd(count + 1, 1) == (int)gridDim.x - 1) {
+    if (atomicAdd(count + 1, 1) == blocks - 1) {
         count[0] = 0;
         count[1] = 0;
+    }
+}
+
+// The end of a group of steps for body b (one warp): its second half kick and,
+// with `out` (host-mapped), its totals (6 a body) and X, V, q, w (13 a body,
+// after the totals and the error word); each lane writes what it holds itself.
+__device__ __forceinline__ void finish_body(Body *bodies, int b, int nb, int lane, double dt, double *out) {
+    const Recorder none{};
+    body_update<true, false>(bodies + b, lane, dt, nullptr, b, nb, none);
+    if (!out) return;
+    const Body &B = bodies[b];           // X and q are the prologue's, the rest this lane's own
+    double *st = out + 6 * nb + 1 + 13 * b;
+    if (lane < 3) {
+        out[6 * b + lane] = B.F_tot[lane];
+        out[6 * b + 3 + lane] = B.T_tot[lane];
+        st[lane] = B.X[lane];
+        st[3 + lane] = B.V[lane];
+        st[10 + lane] = B.w[lane];
+    }
+    if (lane < 4) st[6 + lane] = B.q[lane];
+}
+
+// Zeroes the force on the nodes of the listed tiles and drops their flags:
+// thread t of n, one (tile, node of the tile) at a time.
+template <typename T>
+__device__ __forceinline__ void clear_tiles(const Geom &g, T *F, int *tiles, const int *tlist, const int *tcount,
+                                            int ntx, int nty, long long t, long long n) {
+    const long long total = 64LL * (*tcount);
+    for (long long i = t; i < total; i += n) {
+        const int tile = tlist[i >> 6];
+        const int l = (int)(i & 63);
+        const int tx = tile % ntx, ty = (tile / ntx) % nty, tz = tile / (ntx * nty);
+        const int x = 4 * tx + (l & 3), y = 4 * ty + ((l >> 2) & 3), z = 4 * tz + (l >> 4);
+        if (x < g.nx && y < g.ny && z < g.nz) {
+            const long long m = nidx(g, x, y, z);
+            F[m] = T(0);
+            F[g.N + m] = T(0);
+            F[2 * g.N + m] = T(0);
+        }
+        if (l == 0) tiles[tile] = 0;
+    }
+}
+
+// Extra block eb of a chained fluid kernel (StepExtra).
+template <typename T>
+__device__ __noinline__ void step_extra(const StepExtra &e, const Geom &g, int eb) {
+    const int n = blockDim.x * blockDim.y, t = threadIdx.x + blockDim.x * threadIdx.y;
+    const int lane = t & 31, warp = t >> 5, warps = n >> 5;
+    if (eb < e.body_blocks) {
+        for (int b = eb + e.body_blocks * warp; b < e.nb; b += e.body_blocks * warps) {
+            if (e.mode == 1) body_update<true, true>(e.bodies + b, lane, e.dt, e.ext, b, e.nb, e.rec);
+            else finish_body(e.bodies, b, e.nb, lane, e.dt, e.out);
+        }
+        if (e.mode == 2 && eb == 0 && t == 0) {
+            *e.step += e.by;
+            if (e.out) e.out[6 * e.nb] = e.err ? (double)*e.err : 0.0;
+        }
+    } else {                                   // mode 1
+        const int blocks = e.blocks - e.body_blocks;
+        clear_tiles(g, static_cast<T *>(e.F), e.tiles, e.tlist, e.tcount, e.ntx, e.nty,
+                    (long long)(eb - e.body_blocks) * n + t, (long long)blocks * n);
+        restart_list(e.tcount, blocks);
     }
 }
 
