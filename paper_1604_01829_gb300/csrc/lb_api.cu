@@ -226,6 +226,7 @@ lbk::FluidArgs fluid_args(const lb_ctx *h, int cur, uint32_t step_off) {
     for (int k = 10; k <= 18; ++k) a.pd.kg[k - 10] = (1.0 / 36.0) / bk[k] * rate(k);
     for (int k = 4; k <= 18; ++k) a.pd.kn[k - 4] = (1.0 / 36.0) / bk[k] * h->sig[k - 4] * 3.4641016151377544;
     a.fx = h->fx;
+    a.pk = lbk::coll_pairs(a.pd);
     a.pf.rho0 = (float)a.pd.rho0;
     a.pf.omega = (float)a.pd.omega;
     for (int k = 0; k < 6; ++k) {

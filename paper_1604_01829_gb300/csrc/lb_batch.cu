@@ -23,13 +23,15 @@
 #include "lb_fix64.cuh"
 #include "lb_couple.cuh"
 
-// register caps of the FP32 fluid kernel per parity (resident CTAs of 128
-// threads per SM: 65536 / (128 x cap), rounded down)
-#ifndef LB_BATCH_REGS_EVEN
-#define LB_BATCH_REGS_EVEN 64
+// register caps of the FP32 fluid kernel without and with noise (resident CTAs
+// of 128 threads per SM: 65536 / (128 x cap), rounded down): 256 uneven
+// instances without noise 624 us per launch at 56, 629 at 64, 632 at 72; 64
+// boxes of 24^3 with noise 28.7 / 28.5 / 28.7
+#ifndef LB_BATCH_REGS
+#define LB_BATCH_REGS 56
 #endif
-#ifndef LB_BATCH_REGS_ODD
-#define LB_BATCH_REGS_ODD 64
+#ifndef LB_BATCH_REGS_NOISE
+#define LB_BATCH_REGS_NOISE 64
 #endif
 // of the FP64 fluid kernel (fixed-point collision)
 #ifndef LB_BATCH_REGS_F64
@@ -70,6 +72,7 @@ struct BInst {
     float gf[3];
     CollParams<double> pd;
     CollParams<float> pf;
+    CollPairs pk;                // FP32 MRT
     FixParams fx;                // FP64 storage
 };
 
@@ -80,6 +83,7 @@ struct BatchArgs {
     int n, ntiles, chunk, order;
     CollParams<double> pd;       // collision constants shared by all instances (COMMON kernels)
     CollParams<float> pf;
+    CollPairs pk;
     FixParams fx;
     void *pool;
     const void *F;               // spread force of this step (pool, storage precision), nullptr without bodies
@@ -150,7 +154,7 @@ __device__ __forceinline__ void compact_odd_store(T *P, uint32_t base, uint32_t 
 }
 
 template <typename T, int COLL, bool NOISE, bool ODD, bool COMMON>
-__global__ void __maxnreg__(sizeof(T) == 4 ? (ODD ? LB_BATCH_REGS_ODD : LB_BATCH_REGS_EVEN) : LB_BATCH_REGS_F64)
+__global__ void __maxnreg__(sizeof(T) == 4 ? (NOISE ? LB_BATCH_REGS_NOISE : LB_BATCH_REGS) : LB_BATCH_REGS_F64)
     k_batch_collide(const __grid_constant__ BatchArgs a) {
     using R = T;
     constexpr bool DEV = sizeof(T) == 4;
@@ -235,7 +239,8 @@ __global__ void __maxnreg__(sizeof(T) == 4 ? (ODD ? LB_BATCH_REGS_ODD : LB_BATCH
         uint32_t step = 0;
         if (NOISE) step = (uint32_t)(*a.step_base) + a.step_off;
         const uint2 key = make_uint2(I.key0, I.key1);
-        if constexpr (DEV) collide<R, true, COLL, NOISE>(f, Fx, Fy, Fz, COMMON ? a.pf : I.pf, key, I.instance, n, step);
+        if constexpr (DEV)
+            collide_f32<COLL, NOISE, true>(f, Fx, Fy, Fz, COMMON ? a.pf : I.pf, COMMON ? a.pk : I.pk, key, I.instance, n, step);
         else collide_node_f64<COLL, NOISE>(f, Fx, Fy, Fz, COMMON ? a.fx : I.fx, COMMON ? a.pd : I.pd, key, I.instance, n,
                                            step, load);
         // re-read the plane layout for the stores instead of keeping 19 plane
@@ -588,6 +593,7 @@ void fill_coll(const lb_params &p, BInst &I) {
         const double sig = (p.collision == 1 && p.kT > 0.0) ? std::sqrt(3.0 * p.kT * bk[k] * (1.0 - g * g)) : 0.0;
         I.pd.kn[k - 4] = (1.0 / 36.0) / bk[k] * sig * 3.4641016151377544;
     }
+    I.pk = lbk::coll_pairs(I.pd);
     if (p.precision == 64) {
         double rates[15];
         for (int k = 4; k <= 18; ++k) rates[k - 4] = p.collision == 0 ? 1.0 - 1.0 / p.tau : rate(k);
@@ -960,6 +966,7 @@ lb_status launch_step(lb_batch_ctx *h, int k, bool finish_prev, bool record, boo
     a.ntiles = h->ntiles;
     a.pd = h->hinst[0].pd;
     a.fx = h->hinst[0].fx;
+    a.pk = h->hinst[0].pk;
     a.pf = h->hinst[0].pf;
     const int res = h->resident[odd ? 1 : 0];
     int grid = h->sms * std::min(h->bpsm, res > 0 ? res : h->bpsm);

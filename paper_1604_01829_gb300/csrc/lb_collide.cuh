@@ -103,28 +103,18 @@ __device__ __forceinline__ void collide(R (&f)[19], R Fx, R Fy, R Fz, const Coll
     R q13 = a.kg[3] * m13, q14 = a.kg[4] * m14, q15 = a.kg[5] * m15;
     R q16 = a.kg[6] * m16, q17 = a.kg[7] * m17, q18 = a.kg[8] * m18;
 
-    if (NOISE) {
+    if constexpr (NOISE) {
+        static_assert(sizeof(R) == 8, "FP32 with noise: collide_mrt_f32");
         // 15 non-conserved modes, variance 3 rho kT b_k (1 - g_k^2); kn_k holds
-        // c_k sqrt(3 kT b_k (1 - g_k^2)) sqrt(12) (times 2^-32 in FP32). The
+        // c_k sqrt(3 kT b_k (1 - g_k^2)) sqrt(12). The
         // variates are 16-bit: two Philox calls give 16 half-words, mode 4 + j
         // takes half-word j (high half of word j/2 for even j, else the low
-        // half), xi = sqrt(12) ((h + 1/2) 2^-16 - 1/2). In FP32 the half-word
-        // and a 1/2 below it become the mantissa of y = 1 + (h + 1/2) 2^-16 in
-        // [1, 2), and (y - 3/2) 2^32 = xi 2^32 / sqrt(12) is exact in one FMA
-        // (no integer-to-float conversion).
+        // half), xi = sqrt(12) ((h + 1/2) 2^-16 - 1/2).
         const uint4 r0 = philox4x32_10(make_uint4(node, step, instance, 0u), key);
         const uint4 r1 = philox4x32_10(make_uint4(node, step, instance, 1u), key);
-        R sr;
-        if constexpr (sizeof(R) == 4) asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(sr) : "f"(rho));
-        else sr = sqrt(rho);
-        auto hi = [&](R &q, int k, uint32_t v) {
-            if constexpr (sizeof(R) == 8) q += (sr * a.kn[k]) * centred16_d(v >> 16);
-            else q = fmaf(sr * a.kn[k], fmaf(__uint_as_float(((v >> 9) & 0x7FFF80u) | 0x3F800040u), 0x1p32f, -0x1.8p32f), q);
-        };
-        auto lo = [&](R &q, int k, uint32_t v) {
-            if constexpr (sizeof(R) == 8) q += (sr * a.kn[k]) * centred16_d(v & 0xFFFFu);
-            else q = fmaf(sr * a.kn[k], fmaf(__uint_as_float(((v << 7) & 0x7FFF80u) | 0x3F800040u), 0x1p32f, -0x1.8p32f), q);
-        };
+        const R sr = sqrt(rho);
+        auto hi = [&](R &q, int k, uint32_t v) { q += (sr * a.kn[k]) * centred16_d(v >> 16); };
+        auto lo = [&](R &q, int k, uint32_t v) { q += (sr * a.kn[k]) * centred16_d(v & 0xFFFFu); };
         hi(q4, 0, r0.x); lo(q5, 1, r0.x); hi(q6, 2, r0.y); lo(q7, 3, r0.y);
         hi(q8, 4, r0.z); lo(q9, 5, r0.z); hi(q10, 6, r0.w); lo(q11, 7, r0.w);
         hi(q12, 8, r1.x); lo(q13, 9, r1.x); hi(q14, 10, r1.y); lo(q15, 11, r1.y);
@@ -180,11 +170,144 @@ __device__ __forceinline__ void collide(R (&f)[19], R Fx, R Fy, R Fz, const Coll
     }
 }
 
-template <int COLL, bool NOISE>
-__device__ __forceinline__ void collide_fp32(float (&f)[19], float Fx, float Fy, float Fz,
-                                             const CollParams<float> &a, const FluidArgs &fa, uint32_t node,
-                                             uint32_t step) {
-    collide<float, true, COLL, NOISE>(f, Fx, Fy, Fz, a, make_uint2(fa.key0, fa.key1), fa.instance, node, step);
+// The MRT collision in FP32 on deviations, two values per instruction
+// (fma.rn.f32x2 and its kin): the planes xy and xz, the axes y and z, and the
+// modes they mix into share every formula but a sign, so links (7, 11), (9, 13),
+// (3, 5) and (15, 17), components (y, z) and modes (5, 6), (7, 9), (11, 12),
+// (14, -15), (17, 18) go in pairs: ~140 FP32 instructions instead of ~240, in a
+// kernel that waits for memory at the occupancy its registers allow and, on a
+// lattice that stays in L2, is bound by issue. Measured against the scalar
+// form: 256^3 with noise 436.9 -> 427.5 us per launch, 64 batched boxes of 24^3
+// with noise 30.9 -> 28.5, 256 uneven instances without 640 -> 629 (624 at 56
+// registers); one lattice without noise 86.7 -> 88.0 (150 x 97 x 203: the pairs
+// spill at the 64 registers that suit it), so that keeps the scalar form.
+template <bool NOISE>
+__device__ __forceinline__ void collide_mrt_f32(float (&f)[19], float Fx, float Fy, float Fz, const CollPairs &a,
+                                                uint2 key, uint32_t instance, uint32_t node, uint32_t step) {
+    auto add = [](float2 x, float2 y) { return __fadd2_rn(x, y); };
+    auto mul = [](float2 x, float2 y) { return __fmul2_rn(x, y); };
+    auto fma = [](float2 x, float2 y, float2 z) { return __ffma2_rn(x, y, z); };
+    auto two = [](float x) { return make_float2(x, x); };
+    auto sub = [](float2 x, float2 y) { return __ffma2_rn(y, make_float2(-1.f, -1.f), x); };
+    auto pr = [](float x, float y) { return make_float2(x, y); };
+
+    const float2 p1 = pr(f[7], f[11]), o1 = pr(f[8], f[12]), p2 = pr(f[9], f[13]), o2 = pr(f[10], f[14]);
+    const float2 py = pr(f[3], f[5]), oy = pr(f[4], f[6]), pz = pr(f[15], f[17]), oz = pr(f[16], f[18]);
+    const float2 s1 = add(p1, o1), d1 = sub(p1, o1), s2 = add(p2, o2), d2 = sub(p2, o2);
+    const float2 sY = add(py, oy), dY = sub(py, oy), sZ = add(pz, oz), dZ = sub(pz, oz);
+    const float sx = f[1] + f[2], dx = f[1] - f[2];
+    const float2 Sp = add(s1, s2), m79 = sub(s1, s2);                     // (Sxy, Sxz), (m7, m9)
+    const float2 dp = add(d1, d2), dm = sub(d1, d2);
+    const float Syz = sZ.x + sZ.y, m8 = sZ.x - sZ.y;
+    const float2 dz = pr(dZ.x + dZ.y, dZ.x - dZ.y);
+    const float Sxx = Sp.x + Sp.y, Sd = Sxx + Syz, Sa = sY.x + sY.y, Sax = sx + Sa;
+    const float m0 = f[0] + Sax + Sd;
+    const float rho = a.rho0 + m0;
+    const float tx = dp.x + dp.y, jx = dx + tx;
+    const float2 tyz = add(dm, dz), jyz = add(dY, tyz);
+    const float m10 = fmaf(-2.f, dx, tx), m13 = dp.x - dp.y;
+    const float2 m1112 = fma(dY, two(-2.f), tyz), m1415 = sub(dz, dm);    // (m14, -m15)
+    const float2 A = pr(fmaf(2.f, sx, -Sa), sY.x - sY.y), B = pr(fmaf(-2.f, Syz, Sxx), Sp.x - Sp.y);
+    const float2 m56 = add(A, B), m1718 = sub(B, A);
+    const float m4 = Sd - f[0], m16 = fmaf(-2.f, Sax, f[0] + Sd);
+
+    const float ir = __fdividef(1.0f, rho);
+    const float2 Fyz = pr(Fy, Fz);
+    const float ux = fmaf(0.5f, Fx, jx) * ir;
+    const float2 uyz = mul(fma(Fyz, two(0.5f), jyz), two(ir));
+    // equilibrium stress rho u u and Guo source (uF + Fu; ks holds its 2)
+    const float rux = rho * ux;
+    const float2 ruyz = mul(two(rho), uyz), eyz = mul(ruyz, uyz);
+    const float exx = rux * ux, et = eyz.x + eyz.y;
+    const float2 e56 = pr(fmaf(2.f, exx, -et), eyz.x - eyz.y), e79 = mul(two(rux), uyz);
+    const float e8 = ruyz.x * uyz.y;
+    const float2 g = mul(uyz, Fyz);
+    const float gx = ux * Fx, gt = g.x + g.y;
+    const float2 g56 = pr(fmaf(2.f, gx, -gt), g.x - g.y), g79 = fma(two(ux), Fyz, mul(uyz, two(Fx)));
+    const float g8 = fmaf(uyz.x, Fz, uyz.y * Fy);
+    float q4 = fmaf(a.ke4, exx + et, fmaf(a.km4, m4, a.ks4 * (gx + gt)));
+    float2 q56 = fma(a.ke56, e56, fma(a.km56, m56, mul(a.ks56, g56)));
+    float2 q79 = fma(a.ke79, e79, fma(a.km79, m79, mul(a.ks79, g79)));
+    float q8 = fmaf(a.ke8, e8, fmaf(a.km8, m8, a.ks8 * g8));
+    float q10 = a.kg10 * m10, q13 = a.kg13 * m13, q16 = a.kg16 * m16;
+    float2 q1112 = mul(a.kg1112, m1112), q1415 = mul(a.kg1415, m1415), q1718 = mul(a.kg1718, m1718);
+
+    if (NOISE) {
+        // 15 non-conserved modes, variance 3 rho kT b_k (1 - g_k^2); kn_k holds
+        // c_k sqrt(3 kT b_k (1 - g_k^2)) sqrt(12) 2^-32. Mode 4 + j takes
+        // half-word j of two Philox calls (high half of word j/2 for even j,
+        // else the low half), xi = sqrt(12) ((h + 1/2) 2^-16 - 1/2): the
+        // half-word and a 1/2 below it become the mantissa of y = 1 + (h + 1/2)
+        // 2^-16 in [1, 2), and (y - 3/2) 2^32 is exact in one FMA (no
+        // integer-to-float conversion).
+        const uint4 r0 = philox4x32_10(make_uint4(node, step, instance, 0u), key);
+        const uint4 r1 = philox4x32_10(make_uint4(node, step, instance, 1u), key);
+        float sr;
+        asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(sr) : "f"(rho));
+        auto hi = [](uint32_t v) { return __uint_as_float(((v >> 9) & 0x7FFF80u) | 0x3F800040u); };
+        auto lo = [](uint32_t v) { return __uint_as_float(((v << 7) & 0x7FFF80u) | 0x3F800040u); };
+        auto n1 = [&](float &q, float k, float y) { q = fmaf(sr * k, fmaf(y, 0x1p32f, -0x1.8p32f), q); };
+        auto n2 = [&](float2 &q, float2 k, float y, float z) {
+            q = fma(mul(two(sr), k), fma(pr(y, z), two(0x1p32f), two(-0x1.8p32f)), q);
+        };
+        n1(q4, a.kn4, hi(r0.x));
+        n2(q56, a.kn56, lo(r0.x), hi(r0.y));
+        n2(q79, a.kn79, lo(r0.y), lo(r0.z));
+        n1(q8, a.kn8, hi(r0.z));
+        n1(q10, a.kn10, hi(r0.w));
+        n2(q1112, a.kn1112, lo(r0.w), hi(r1.x));
+        n1(q13, a.kn13, lo(r1.x));
+        n2(q1415, a.kn1415, hi(r1.y), lo(r1.y));
+        n1(q16, a.kn16, hi(r1.z));
+        n2(q1718, a.kn1718, lo(r1.z), hi(r1.w));
+    }
+
+    // back to populations (as collide)
+    constexpr float c0 = 1.0f / 36.0f, c1 = 1.0f / 12.0f;
+    const float q0 = c0 * m0, q1 = c1 * (jx + Fx);
+    const float2 q23 = mul(add(jyz, Fyz), two(c1));
+    f[0] = 12.f * (q0 - q4 + q16);
+    const float U = fmaf(-2.f, q16, q0);
+    const float2 VW = sub(q1718, q56);                                    // (V, -W)
+    {
+        const float E = fmaf(-2.f, VW.x, U), O = fmaf(-2.f, q10, q1);
+        f[1] = 2.f * (E + O);
+        f[2] = 2.f * (E - O);
+    }
+    {
+        const float UV = U + VW.x;
+        const float2 E = pr(UV - VW.y, UV + VW.y), O = fma(q1112, two(-2.f), q23);
+        const float2 u = mul(two(2.f), add(E, O)), v = mul(two(2.f), sub(E, O));
+        f[3] = u.x; f[5] = u.y;
+        f[4] = v.x; f[6] = v.y;
+    }
+    const float Ed = q0 + q4 + q16;
+    const float2 S = add(q56, q1718);
+    const float T = Ed + S.x, T3 = fmaf(-2.f, S.x, Ed);
+    const float2 T12 = pr(T + S.y, T - S.y), Ep = add(T12, q79), Em = sub(T12, q79);
+    const float P = q1 + q10;
+    const float2 QR = add(q23, q1112), Pc = pr(P + q13, P - q13), G = sub(QR, q1415);
+    const float2 O1 = add(Pc, G), O2 = sub(Pc, G);
+    const float2 a7 = add(Ep, O1), a8 = sub(Ep, O1), a9 = add(Em, O2), a10 = sub(Em, O2);
+    f[7] = a7.x; f[11] = a7.y;
+    f[8] = a8.x; f[12] = a8.y;
+    f[9] = a9.x; f[13] = a9.y;
+    f[10] = a10.x; f[14] = a10.y;
+    const float2 H = add(QR, q1415);                                      // (Q + q14, R - q15)
+    const float2 O3 = pr(H.x + H.y, H.x - H.y), E3 = pr(T3 + q8, T3 - q8);
+    const float2 a15 = add(E3, O3), a16 = sub(E3, O3);
+    f[15] = a15.x; f[17] = a15.y;
+    f[16] = a16.x; f[18] = a16.y;
+}
+
+// Collision of one FP32 node: MRT in pairs (PAIRS, and always with noise), or
+// as it stands.
+template <int COLL, bool NOISE, bool PAIRS>
+__device__ __forceinline__ void collide_f32(float (&f)[19], float Fx, float Fy, float Fz, const CollParams<float> &pf,
+                                            const CollPairs &pk, uint2 key, uint32_t instance, uint32_t node,
+                                            uint32_t step) {
+    if constexpr (COLL == 1 && (PAIRS || NOISE)) collide_mrt_f32<NOISE>(f, Fx, Fy, Fz, pk, key, instance, node, step);
+    else collide<float, true, COLL, false>(f, Fx, Fy, Fz, pf, key, instance, node, step);
 }
 
 }  // namespace lbk

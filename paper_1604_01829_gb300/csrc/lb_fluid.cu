@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (NOISE ? LB_CS_MINB_NOIS
     if (NOISE) step = (uint32_t)(*a.step_base) + a.step_off;
 
     const uint2 key = make_uint2(a.key0, a.key1);
-    if constexpr (sizeof(R) == 4) collide<R, DEV, COLL, NOISE>(f, Fx, Fy, Fz, a.pf, key, a.instance, (uint32_t)n, step);
+    if constexpr (DEV) collide_f32<COLL, NOISE, false>(f, Fx, Fy, Fz, a.pf, a.pk, key, a.instance, (uint32_t)n, step);
     else collide_node_f64<COLL, NOISE>(f, Fx, Fy, Fz, a.fx, a.pd, key, a.instance, (uint32_t)n, step, load);
 
     // odd step: f*_i goes to the downstream node n + c_i, the upstream node of

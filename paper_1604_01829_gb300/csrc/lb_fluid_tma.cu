@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kThreads, LB_TMA_MINB)
             }
             uint32_t step = 0;
             if (NOISE) step = (uint32_t)(*a.step_base) + a.step_off;
-            collide_fp32<COLL, NOISE>(f, Fx, Fy, Fz, a.pf, a, n, step);
+            collide_f32<COLL, NOISE, false>(f, Fx, Fy, Fz, a.pf, a.pk, make_uint2(a.key0, a.key1), a.instance, n, step);
             if (!ODD) {
 #pragma unroll
                 for (int i = 0; i < 19; ++i) A[(size_t)opp(i) * N32 + n] = f[i];

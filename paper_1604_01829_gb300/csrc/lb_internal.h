@@ -25,6 +25,35 @@ struct CollParams {
                                  //   applied to a centred uniform variate in (-1/2, 1/2) (FP32: times 2^-32)
 };
 
+// The MRT constants of the FP32 collision, paired as its two-wide arithmetic
+// reads them (lb_collide.cuh): {5, 6} is the value of mode 5 and of mode 6.
+// ks holds twice CollParams::ks for modes 4-6; kn of mode 15 is negated, as
+// the collision carries -m_15.
+struct alignas(8) CollPairs {
+    float2 ke56, km56, ks56, ke79, km79, ks79, kg1112, kg1415, kg1718;
+    float2 kn56, kn79, kn1112, kn1415, kn1718;
+    float rho0, ke4, km4, ks4, ke8, km8, ks8, kg10, kg13, kg16, kn4, kn8, kn10, kn13, kn16;
+};
+
+inline CollPairs coll_pairs(const CollParams<double> &d) {
+    CollPairs p{};
+    auto two = [](double a, double b) { return make_float2((float)a, (float)b); };
+    const double n = 2.3283064365386963e-10;       // 2^-32 (CollParams::kn in FP32)
+    p.ke56 = two(d.ke[1], d.ke[2]); p.km56 = two(d.km[1], d.km[2]); p.ks56 = two(2 * d.ks[1], 2 * d.ks[2]);
+    p.ke79 = two(d.ke[3], d.ke[5]); p.km79 = two(d.km[3], d.km[5]); p.ks79 = two(d.ks[3], d.ks[5]);
+    p.kg1112 = two(d.kg[1], d.kg[2]); p.kg1415 = two(d.kg[4], d.kg[5]); p.kg1718 = two(d.kg[7], d.kg[8]);
+    p.kn56 = two(n * d.kn[1], n * d.kn[2]); p.kn79 = two(n * d.kn[3], n * d.kn[5]);
+    p.kn1112 = two(n * d.kn[7], n * d.kn[8]); p.kn1415 = two(n * d.kn[10], -n * d.kn[11]);
+    p.kn1718 = two(n * d.kn[13], n * d.kn[14]);
+    p.rho0 = (float)d.rho0;
+    p.ke4 = (float)d.ke[0]; p.km4 = (float)d.km[0]; p.ks4 = (float)(2 * d.ks[0]);
+    p.ke8 = (float)d.ke[4]; p.km8 = (float)d.km[4]; p.ks8 = (float)d.ks[4];
+    p.kg10 = (float)d.kg[0]; p.kg13 = (float)d.kg[3]; p.kg16 = (float)d.kg[6];
+    p.kn4 = (float)(n * d.kn[0]); p.kn8 = (float)(n * d.kn[4]); p.kn10 = (float)(n * d.kn[6]);
+    p.kn13 = (float)(n * d.kn[9]); p.kn16 = (float)(n * d.kn[12]);
+    return p;
+}
+
 // A 64-bit factor as h 2^32 + l with l signed, and the constants of the
 // fixed-point evaluation of the FP64 collision (lb_fix64.cuh).
 struct FixPair {
@@ -101,7 +130,6 @@ struct FluidArgs {
     void *f;                     // populations: double[19][N] (FP64) or float[19][N] deviations
     CollParams<double> pd;
     CollParams<float> pf;
-    FixParams fx;                // FP64 storage
     const double *gforce;        // device: uniform force density (3)
     const float *gforce_f;       // device: the same, rounded to FP32
     const void *Fn;              // device: spread bead force [3][N] in the storage precision, or nullptr
@@ -114,11 +142,16 @@ struct FluidArgs {
     void *plane[19];             // base of each population plane (f + i N), uniform per launch
     const uint32_t *masks;       // pore: per position across the axis, bit 31 wall node, bit i the
                                  // upstream node of link i is a wall (launch_build_masks)
+    void *out[19];               // out-of-place step (launch_collide_stream_oop): where each plane's
+                                 // populations are stored; the loads read f / plane
+    // below: not read by the FP32 kernels of large lattices without noise, whose
+    // 64 registers depend on the offsets above (held bodies in 150 x 97 x 203:
+    // step 96.8 us with these members in the middle, 96.4 here)
     const uint4 *fpos;           // pore: fluid positions across the axis, {first coordinate, second, wall mask, 0}
     int nfpos;                   // (null: one thread per node of the box)
     StepExtra ex;                // chained kernels
-    void *out[19];               // out-of-place step (launch_collide_stream_oop): where each plane's
-                                 // populations are stored; the loads read f / plane
+    CollPairs pk;                // FP32 MRT
+    FixParams fx;                // FP64 storage
 };
 
 // Repulsive pore-wall beads (Sec. 2.3): beads on the cylinder of radius Rc
