@@ -1,0 +1,141 @@
+"""Branches of the step on the CUDA path against the oracle: the fixed-point
+FP64 collision inside and outside its range, the chained launches of small
+lattices (body updates and tile clearing in extra blocks of the fluid kernel)
+over group lengths, body counts, substeps and pore axes, force sums of blocks
+that hold several bodies, fast rotations, and results read from host-mapped
+memory after calls that make them stale.
+
+Tolerances as in test_gpu_parity.py: TOL = 1e-12 (FP64) and 1e-5 (FP32) of
+w_i rho0 for populations. Populations within TOL give a velocity within TOL / 3
+(sum of w_i |c_i| per component); bead forces are gamma u with u ~ 0.01 and more,
+so they and what they drive (bodies heavier than 10, at most 29 steps) are held
+to 100 TOL, a body's totals relative to its largest bead force times the bead
+count, since a few beads can cancel."""
+import numpy as np
+import pytest
+
+from helpers import Pair, perturbed_populations
+from paper_1604_01829_gb300 import workloads as Wl
+
+pytestmark = pytest.mark.gpu
+
+TOL = {64: 1e-12, 32: 1e-5}
+MRT = dict(collision=1, gamma_shear=-0.45, gamma_bulk=-0.2, gamma_odd=0.3, gamma_even=-0.1)
+
+
+@pytest.mark.parametrize("rho0", [1.0, 6.004, 1e-3, 0.4])
+@pytest.mark.parametrize("kT", [0.0, 1e-4, 0.02])
+@pytest.mark.parametrize("force", [0.0, 1e-5, 0.6])
+def test_fp64_collision_in_and_out_of_the_fixed_point_range(rho0, kT, force):
+    """Nodes with negative, oversized, tiny and vanishing populations, high speeds
+    and low densities beside ordinary ones; kT = 0.02 rho0 and |F| = 0.6 rho0 leave
+    the range for every node."""
+    params = dict(MRT) if kT else dict(collision=0, tau=0.8)
+    P = Pair(18, 7, 6, precision=64, rho0=rho0, kT=kT * rho0, seed=5, body_force=(0.0, 0.3 * force * rho0, force * rho0),
+             **params)
+    f = perturbed_populations(P.N, rho0=rho0, seed=9)
+    rng = np.random.default_rng(2)
+    at = rng.permutation(P.N)
+    f[rng.integers(1, 19, 40), at[:40]] *= -0.5                    # negative
+    f[rng.integers(7, 19, 40), at[40:80]] += 0.2 * rho0             # beyond 1/16
+    f[0, at[80:100]] += 0.4 * rho0                                  # beyond 1/2
+    f[rng.integers(1, 19, 40), at[100:140]] = 1e-12 * rho0          # far below the grid's steps
+    f[rng.integers(1, 19, 40), at[140:180]] = 0.0
+    f[1, at[180:200]] += 0.11 * rho0                                # fast
+    f[:, at[200:210]] *= 0.2                                        # thin
+    P.set_populations(f)
+    P.step(1)
+    assert P.pop_error() <= 1e-12 * (1 + force)
+
+
+def _beads(rng, n):
+    return rng.uniform(-2.0, 2.0, (n, 3))
+
+
+def _force_errors(P, b):
+    g, o = P.gpu.lb_forces(b, per_bead=True), P.orc.body(b)
+    pb = P.orc.bead_forces(b)
+    scale = np.abs(pb).max() * len(pb)
+    return max(np.abs(g[0] - o["F"]).max() / scale, np.abs(g[1] - o["T"]).max() / (3 * scale),
+               np.abs(g[2] - pb).max() / np.abs(pb).max())
+
+
+@pytest.mark.parametrize("precision", [64, 32])
+@pytest.mark.parametrize("nbodies,nbeads,substeps", [(1, 1, 1), (1, 300, 2), (5, 7, 1), (70, 3, 3), (130, 2, 1)])
+def test_chained_steps(precision, nbodies, nbeads, substeps):
+    rng = np.random.default_rng(nbodies)
+    P = Pair(21, 18, 19, precision=precision, kT=1e-4, seed=3, gamma_bead=0.05, md_substeps=substeps, compensate_force=1, **MRT)
+    P.set_populations(perturbed_populations(P.N, amp=0.005, u_amp=0.01, seed=4))
+    for b in range(nbodies):
+        P.add_body(_beads(rng, nbeads), rng.random(3) * (21, 18, 19), rng.standard_normal(4), mass=20.0, inertia=(30, 35, 42),
+                   F_ext=1e-3 * rng.standard_normal(3), T_ext=1e-3 * rng.standard_normal(3), fixed=b % 3 if nbodies > 1 else 0)
+    for n in (1, 2, 8, 5, 13):                                     # single, short, octet, odd start, mixed
+        P.step(n)
+    assert P.pop_error() <= TOL[precision]
+    for b in range(nbodies):
+        e = P.body_errors(b)
+        assert max(e["X"], e["V"], e["q"], e["w"], _force_errors(P, b)) <= 100 * TOL[precision]
+
+
+@pytest.mark.parametrize("precision", [64, 32])
+@pytest.mark.parametrize("axis", [0, 1, 2])
+def test_chained_pore_steps(precision, axis):
+    n = [19, 20, 21]
+    P = Pair(*n, precision=precision, pore=(8.0, axis), gamma_bead=0.05, body_force=(1e-5, 1e-5, 1e-5), **MRT)
+    P.set_populations(perturbed_populations(P.N, amp=0.005, u_amp=0.01, seed=6))
+    P.add_body(Wl.sphere_raspberry(2.0), np.array(n) / 2 + 0.3, mass=33.0, inertia=(50, 50, 50), F_ext=(1e-3, 0, 2e-3))
+    P.step(11)
+    assert P.pop_error() <= TOL[precision]
+    e = P.body_errors(0)
+    assert max(e["X"], e["V"], e["q"], e["w"]) <= 100 * TOL[precision]
+
+
+@pytest.mark.parametrize("speed", [1e-9, 0.3, 0.99, 1.01, 3.0])
+def test_fast_rotation(speed):
+    """Half angles on both sides of 1/2, where the power series ends."""
+    P = Pair(16, 16, 16, precision=64, gamma_bead=0.01, collision=0, tau=0.9)
+    w = speed * np.array([0.6, -0.48, 0.64])
+    P.add_body(Wl.fibonacci_sphere(12, 2.0), [8.2, 7.9, 8.1], mass=40.0, inertia=(60, 80, 110), w=w, F_ext=(1e-4, 0, 0))
+    P.step(6)
+    e = P.body_errors(0)
+    assert max(e["X"], e["V"], e["q"], e["w"]) <= 1e-11
+    assert P.pop_error() <= 1e-11                                  # speeds of 3 w per unit of population
+
+
+def test_mapped_results_follow_the_state():
+    from paper_1604_01829_gb300 import lb
+    kw = dict(precision=64, gamma_bead=0.05, collision=0, tau=0.9)
+    h = lb.LB(16, 16, 16, **kw)
+    h.lb_add_raspberry(Wl.sphere_raspberry(2.0), [8.2, 7.9, 8.1], mass=33.0, inertia=(50, 50, 50), F_ext=(1e-3, 0, 0))
+    h.lb_step(5)
+    F, T = h.lb_forces_all()
+    assert np.array_equal(F, h.lb_forces(0)[0]) and np.array_equal(T, h.lb_forces(0)[1])
+    data, at5 = h.lb_checkpoint_save(), h.lb_get_body(0)
+    h.lb_set_body_state(0, X=(3.0, 4.0, 5.0))
+    assert np.array_equal(h.lb_get_body(0)["X"], [3.0, 4.0, 5.0]) and np.array_equal(h.lb_get_body(0)["V"], at5["V"])
+    h.lb_step(4)
+    assert np.abs(h.lb_get_body(0)["X"] - [3.0, 4.0, 5.0]).max() < 0.1
+    h.lb_checkpoint_load(data)
+    assert all(np.array_equal(h.lb_get_body(0)[k], at5[k]) for k in at5)
+    assert np.array_equal(h.lb_forces_all()[0], F)
+
+    B = lb.LBBatch([dict(nx=16, ny=16, nz=16 + k, **kw) for k in range(3)])
+    for k in range(3):
+        B.lb_batch_add_raspberry(k, Wl.sphere_raspberry(2.0), [8.2, 7.9, 8.1], mass=33.0, inertia=(50, 50, 50),
+                                 F_ext=(1e-3, 0, 1e-4 * k))
+    before = B.lb_batch_get_body(2)["X"]
+    assert np.array_equal(before, [8.2, 7.9, 8.1])
+    for n in (1, 8, 3, 10):
+        B.lb_batch_step(n)
+    data = B.lb_batch_checkpoint_save()
+    got = [(B.lb_batch_get_body(k), B.lb_batch_forces(k)) for k in range(3)]
+    B.lb_batch_autotune(2)
+    for k in range(3):
+        body, (F, T) = B.lb_batch_get_body(k), B.lb_batch_forces(k)
+        assert all(np.array_equal(body[q], got[k][0][q]) for q in body)
+        assert np.array_equal(F, got[k][1][0]) and np.array_equal(T, got[k][1][1])
+    B.lb_batch_step(6)
+    assert not np.array_equal(B.lb_batch_get_body(1)["X"], got[1][0]["X"])
+    B.lb_batch_checkpoint_load(data)
+    assert np.array_equal(B.lb_batch_get_body(1)["X"], got[1][0]["X"])
+    assert np.array_equal(B.lb_batch_forces(1)[0], got[1][1][0])
