@@ -36,6 +36,10 @@
 #ifndef LB_CS_MINB_NOISE
 #define LB_CS_MINB_NOISE 7
 #endif
+// slices between a block's own and the one it fetches, per SM (fetch_plane)
+#ifndef LB_AHEAD
+#define LB_AHEAD 8
+#endif
 #ifndef LB_CS_MINB_F64
 #define LB_CS_MINB_F64 4
 #endif
@@ -89,11 +93,35 @@ __device__ __forceinline__ uint32_t pore_section_index(const Geom &g, int x, int
 
 // ------------------------------------------------------- collide and stream
 
-template <typename T, int COLL, bool NOISE, bool ODD, bool PORE, bool OOP = false, bool CHAIN = false>
-__global__ void __launch_bounds__(128, sizeof(T) == 4 ? (NOISE ? LB_CS_MINB_NOISE : LB_CS_MINB) : LB_CS_MINB_F64)
+// One thread's part (plane i) of a block's fetch into L2: the box is cut into
+// as many slices as the grid has blocks, and the block fetches the slice `ahead`
+// slices after its own (whole 128-byte lines of that slice). A block's loads
+// wait ~1 us for memory at 7 or 8 blocks per SM, and while it computes and
+// stores it loads nothing: with the next blocks' populations on their way to L2
+// the memory stays busy. Per step, before and after: 256^3 with noise 424 ->
+// 377 us (the copy rate), with 64 ellipsoids 456 -> 430, without noise 398 ->
+// 380, BGK 413 -> 377, 128^3 58.4 -> 53.4, 112^3 43.2 -> 41.2, held bodies in
+// 150 x 97 x 203 96.4 -> 90.2. Slices ahead, as blocks per SM: 256^3 with noise
+// 408 at 2, 383 at 4, 377 at 6 to 8, 380 at 10; with bodies 430 at 8, 456 at 16.
+// One thread per plane: the copies are queued, not waited for.
+__device__ __forceinline__ void fetch_plane(const FluidArgs &a, int i) {
+    const unsigned long long b = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z) + a.ahead;
+    const unsigned long long n0 = (b * a.slice) >> 32, n1 = ((b + 1) * a.slice) >> 32;
+    if (n1 > (unsigned long long)a.g.N) return;
+    const unsigned long long p = reinterpret_cast<unsigned long long>(a.plane[0]) + 4 * (unsigned long long)i * a.g.N;
+    const unsigned long long p0 = (p + 4 * n0) & ~127ull, p1 = (p + 4 * n1) & ~127ull;
+    if (p1 > p0) fetch_l2(reinterpret_cast<const void *>(p0), (unsigned)(p1 - p0));
+}
+
+// FORM 1: a chained kernel with extra blocks in front (launch_chain); 2: one
+// that fetches ahead (fetch_plane).
+template <typename T, int COLL, bool NOISE, bool ODD, bool PORE, bool OOP = false, int FORM = 0>
+__global__ void __launch_bounds__(128, sizeof(T) == 8 ? LB_CS_MINB_F64
+                                           : NOISE || (COLL == 0 && FORM == 2) ? LB_CS_MINB_NOISE
+                                                                             : LB_CS_MINB)
     k_collide_stream(const __grid_constant__ FluidArgs a) {
     using R = T;
-    constexpr bool DEV = sizeof(T) == 4;
+    constexpr bool DEV = sizeof(T) == 4, CHAIN = FORM == 1;
     const Geom &g = a.g;
     int by = blockIdx.y, bz = blockIdx.z;
     if (CHAIN) {
@@ -105,6 +133,10 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (NOISE ? LB_CS_MINB_NOIS
             return;
         }
         plane -= a.ex.planes;
+    }
+    if constexpr (FORM == 2) {
+        const unsigned i = threadIdx.x + blockDim.x * threadIdx.y;
+        if (i < 19) fetch_plane(a, i);
     }
     int x = blockIdx.x * blockDim.x + threadIdx.x;
     int y = by * blockDim.y + threadIdx.y;
@@ -222,7 +254,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (NOISE ? LB_CS_MINB_NOIS
     }
 }
 
-template <typename T, int COLL, bool NOISE, bool OOP = false, bool CHAIN = false>
+template <typename T, int COLL, bool NOISE, bool OOP = false, int FORM = 0>
 cudaError_t launch_cs_t(const FluidArgs &args, bool odd, dim3 block, cudaStream_t s) {
     FluidArgs a = args;
     dim3 grid((a.g.nx + block.x - 1) / block.x, (a.g.ny + block.y - 1) / block.y, a.g.nz);
@@ -244,19 +276,34 @@ cudaError_t launch_cs_t(const FluidArgs &args, bool odd, dim3 block, cudaStream_
             a.fpos = nullptr;
         }
     }
-    if (CHAIN) {
+    if (FORM == 1) {
         // the extra blocks in whole planes (rows) in front of the grid
         const unsigned per = a.fpos ? grid.x : grid.x * grid.y;
         a.ex.planes = (a.ex.blocks + per - 1) / per;
         (a.fpos ? grid.y : grid.z) += a.ex.planes;
     }
     const bool pore = a.g.pore_axis >= 0 || a.g.chan;       // bounded: per-position wall masks
+    // A periodic FP32 box larger than L2 fetches ahead. FP64 waits for its
+    // arithmetic and was slower with it (94 x 81 x 103 with noise 73.6 -> 79.8
+    // us, 128^3 174 -> 189); BGK then takes 72 registers and no spills to speak
+    // of (256^3 416 -> 376), MRT without noise 64 as before (held bodies 93.2 at
+    // 72, 90.1 at 64).
+    if constexpr (sizeof(T) == 4 && !OOP && FORM == 0) {
+        if (!pore && 76 * a.g.N >= LB_AHEAD_BYTES) {
+            const unsigned long long blocks = (unsigned long long)grid.x * grid.y * grid.z;
+            a.slice = ((unsigned long long)a.g.N << 32) / blocks;
+            a.ahead = LB_AHEAD * sm_count();
+            if (odd) k_collide_stream<T, COLL, NOISE, true, false, false, 2><<<grid, block, 0, s>>>(a);
+            else k_collide_stream<T, COLL, NOISE, false, false, false, 2><<<grid, block, 0, s>>>(a);
+            return cudaGetLastError();
+        }
+    }
     if (odd) {
-        if (pore) k_collide_stream<T, COLL, NOISE, true, true, OOP, CHAIN><<<grid, block, 0, s>>>(a);
-        else k_collide_stream<T, COLL, NOISE, true, false, OOP, CHAIN><<<grid, block, 0, s>>>(a);
+        if (pore) k_collide_stream<T, COLL, NOISE, true, true, OOP, FORM><<<grid, block, 0, s>>>(a);
+        else k_collide_stream<T, COLL, NOISE, true, false, OOP, FORM><<<grid, block, 0, s>>>(a);
     } else {
-        if (pore) k_collide_stream<T, COLL, NOISE, false, true, OOP, CHAIN><<<grid, block, 0, s>>>(a);
-        else k_collide_stream<T, COLL, NOISE, false, false, OOP, CHAIN><<<grid, block, 0, s>>>(a);
+        if (pore) k_collide_stream<T, COLL, NOISE, false, true, OOP, FORM><<<grid, block, 0, s>>>(a);
+        else k_collide_stream<T, COLL, NOISE, false, false, OOP, FORM><<<grid, block, 0, s>>>(a);
     }
     return cudaGetLastError();
 }
@@ -444,13 +491,13 @@ cudaError_t launch_collide_stream(const FluidArgs &a, bool fp32, int collision, 
 cudaError_t launch_collide_stream_chain(const FluidArgs &a, bool fp32, int collision, bool noise, bool odd, dim3 block,
                                         cudaStream_t s) {
     if (fp32) {
-        if (collision == 0) return launch_cs_t<float, 0, false, false, true>(a, odd, block, s);
-        if (noise) return launch_cs_t<float, 1, true, false, true>(a, odd, block, s);
-        return launch_cs_t<float, 1, false, false, true>(a, odd, block, s);
+        if (collision == 0) return launch_cs_t<float, 0, false, false, 1>(a, odd, block, s);
+        if (noise) return launch_cs_t<float, 1, true, false, 1>(a, odd, block, s);
+        return launch_cs_t<float, 1, false, false, 1>(a, odd, block, s);
     }
-    if (collision == 0) return launch_cs_t<double, 0, false, false, true>(a, odd, block, s);
-    if (noise) return launch_cs_t<double, 1, true, false, true>(a, odd, block, s);
-    return launch_cs_t<double, 1, false, false, true>(a, odd, block, s);
+    if (collision == 0) return launch_cs_t<double, 0, false, false, 1>(a, odd, block, s);
+    if (noise) return launch_cs_t<double, 1, true, false, 1>(a, odd, block, s);
+    return launch_cs_t<double, 1, false, false, 1>(a, odd, block, s);
 }
 
 cudaError_t launch_collide_stream_oop(const FluidArgs &a, bool fp32, int collision, bool odd, dim3 block,

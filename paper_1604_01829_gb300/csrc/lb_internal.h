@@ -125,6 +125,12 @@ struct StepExtra {
 };
 
 // Everything the fused collide-and-stream kernel reads besides populations.
+// bytes of populations from which the FP32 fluid kernels fetch ahead into L2:
+// below, the lattice (or batch) stays in its 129 MB from step to step
+#ifndef LB_AHEAD_BYTES
+#define LB_AHEAD_BYTES (100LL << 20)
+#endif
+
 struct FluidArgs {
     Geom g;
     void *f;                     // populations: double[19][N] (FP64) or float[19][N] deviations
@@ -152,6 +158,8 @@ struct FluidArgs {
     StepExtra ex;                // chained kernels
     CollPairs pk;                // FP32 MRT
     FixParams fx;                // FP64 storage
+    unsigned ahead;              // fetching kernels: slices between a block's own and the one it fetches into L2
+    unsigned long long slice;    // nodes per block, times 2^32
 };
 
 // Repulsive pore-wall beads (Sec. 2.3): beads on the cylinder of radius Rc
