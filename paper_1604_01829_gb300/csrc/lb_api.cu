@@ -417,9 +417,14 @@ lb_status lb_create(const lb_params *p, void *cuda_stream, lb_handle *out) {
                      : (k == 0 ? p->gamma_bulk : (k <= 5 ? p->gamma_shear : (k <= 11 ? p->gamma_odd : p->gamma_even)));
         h->fx = lbk::fix_params(p->rho0, p->kT, rates);
     }
-    // block shape: x fastest, 128 threads
+    // block shape: x fastest, 128 threads; a wider box takes the row length (128,
+    // 64 or 32) that leaves the fewest threads beyond its edge
     int bx = ((p->nx + 31) / 32) * 32;
-    if (bx > 128) bx = 128;
+    if (bx > 128) {
+        bx = 128;
+        for (int c = 64; c >= 32; c /= 2)
+            if ((p->nx + c - 1) / c * c < (p->nx + bx - 1) / bx * bx) bx = c;
+    }
     h->block = dim3(bx, 128 / bx, 1);
 
     if (cuda_stream) h->stream = (cudaStream_t)cuda_stream;
