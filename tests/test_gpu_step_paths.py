@@ -1,9 +1,9 @@
 """Branches of the step on the CUDA path against the oracle: the fixed-point
 FP64 collision inside and outside its range, the chained launches of small
 lattices (body updates and tile clearing in extra blocks of the fluid kernel)
-over group lengths, body counts, substeps and pore axes, force sums of blocks
-that hold several bodies, fast rotations, and results read from host-mapped
-memory after calls that make them stale.
+over group lengths, body counts, substeps and pore axes, fluid kernels that fetch
+ahead into L2, rows cut into blocks, fast rotations, and results read from
+host-mapped memory after calls that make them stale.
 
 Tolerances as in test_gpu_parity.py: TOL = 1e-12 (FP64) and 1e-5 (FP32) of
 w_i rho0 for populations. Populations within TOL give a velocity within TOL / 3
@@ -14,7 +14,7 @@ count, since a few beads can cancel."""
 import numpy as np
 import pytest
 
-from helpers import Pair, perturbed_populations
+from helpers import Pair, W19, perturbed_populations
 from paper_1604_01829_gb300 import workloads as Wl
 
 pytestmark = pytest.mark.gpu
@@ -46,6 +46,57 @@ def test_fp64_collision_in_and_out_of_the_fixed_point_range(rho0, kT, force):
     P.set_populations(f)
     P.step(1)
     assert P.pop_error() <= 1e-12 * (1 + force)
+
+
+@pytest.mark.parametrize("size", [(150, 97, 97), (33, 211, 205), (4100, 19, 18), (2, 840, 841)])
+@pytest.mark.parametrize("case", ["noise", "mrt", "bgk"])
+def test_fetching_ahead(size, case):
+    """FP32 boxes just above the size from which the fluid kernel fetches ahead,
+    with rows that are no multiple of its lines or blocks."""
+    params = dict(MRT, kT=1e-4, seed=2) if case == "noise" else (dict(MRT) if case == "mrt" else dict(collision=0, tau=0.8))
+    P = Pair(*size, precision=32, body_force=(1e-5, 0, 2e-5), **params)
+    P.set_populations(perturbed_populations(P.N, amp=0.005, u_amp=0.01, seed=8))
+    P.step(3)
+    assert P.pop_error() <= TOL[32]
+
+
+@pytest.mark.parametrize("tile,order", [(128, 0), (64, 0), (256, 1), (128, 2)])
+def test_batch_fetching_ahead(tile, order):
+    """A batch above that size: instances of odd sizes, a pore among them, against
+    the oracle."""
+    from oracle import oracle as O
+    from paper_1604_01829_gb300 import lb
+    sizes = [(61, 43, 67), (67, 71, 59), (64, 64, 64), (71, 67, 73), (33, 95, 101)]
+    pars = [dict(nx=n[0], ny=n[1], nz=n[2], precision=32, body_force=(0, 1e-5, 1e-5), **MRT) for n in sizes]
+    B = lb.LBBatch(pars)
+    B.lb_batch_set_pore(3, 30.0, 2)
+    B.lb_batch_set_schedule(tile, 4, order)
+    orcs = []
+    for k, n in enumerate(sizes):
+        f = perturbed_populations(n[0] * n[1] * n[2], amp=0.005, u_amp=0.01, seed=k)
+        B.lb_batch_set_populations(k, f)
+        o = O.OracleLB(*n, body_force=(0, 1e-5, 1e-5), **MRT)
+        if k == 3:
+            o.set_pore(30.0, 2)
+        o.set_populations(f)
+        orcs.append(o)
+    B.lb_batch_step(3)
+    for k, o in enumerate(orcs):
+        o.step(3)
+        fluid = o.mask == 0 if k == 3 else slice(None)
+        d = B.lb_batch_get_populations(k)[:, fluid] - o.populations()[:, fluid]
+        assert np.max(np.abs(d) / W19[:, None]) <= TOL[32]
+
+
+@pytest.mark.parametrize("precision", [64, 32])
+@pytest.mark.parametrize("nx", [129, 150, 190, 224])
+def test_rows_split_without_waste(nx, precision):
+    """Rows longer than a block, cut into 128, 64 or 32 threads."""
+    P = Pair(nx, 7, 5, precision=precision, gamma_bead=0.05, **MRT)
+    P.set_populations(perturbed_populations(P.N, amp=0.005, u_amp=0.01, seed=nx))
+    P.add_body(Wl.fibonacci_sphere(12, 1.5), [nx - 0.7, 6.8, 0.2], mass=30.0, inertia=(40, 40, 40), F_ext=(1e-3, 0, 0))
+    P.step(5)
+    assert P.pop_error() <= TOL[precision]
 
 
 def _beads(rng, n):
