@@ -69,7 +69,7 @@ struct FixParams {
     FixPair kn[15];              // modes 4-18: noise amplitude over sqrt(rho) of the scaled unit, at 2^64
 };
 
-// Rigid bodies (FP64, array of structs; few bodies, one thread each).
+// Rigid bodies (FP64, array of structs; few bodies, one warp each in the step).
 struct Body {
     double X[3], V[3], q[4], w[3];   // centre, velocity, orientation (w,x,y,z), body-frame omega
     double F_last[3], T_last[3];     // last step: lab-frame force, body-frame torque
