@@ -1178,6 +1178,13 @@ extern "C" lb_status lb_adjoint_drag_ex(lb_handle h, int nsteps, int window, int
     lb_status st = lbk::ctx_upload(h);
     if (st == LB_OK) st = lbk::ctx_apply_external(h);
     if (st != LB_OK) return st;
+    // the sweep's lb_step calls declare the mapped results fresh, and every
+    // re-run segment writes them again: whichever way this call ends, they are
+    // not those of the state it leaves
+    struct Stale {
+        lb_ctx *h;
+        ~Stale() { h->out_fresh = false; }
+    } stale{h};
 
     int nsnap, ntape, c = 0, S = 0;
     if (schedule == LB_ADJ_TWO_LEVEL) {

@@ -320,10 +320,8 @@ namespace lbk {
 // host-side hooks used by the adjoint driver (lb_adjoint.cu)
 lb_status ctx_upload(lb_ctx *h) { return upload_bodies(h); }
 // the device body records take the host's external forces now (the adjoint
-// steps with kernels of its own, which do not read the mapped staging), and
-// the mapped totals are stale once it has run
+// steps with kernels of its own, which do not read the mapped staging)
 lb_status ctx_apply_external(lb_ctx *h) {
-    h->out_fresh = false;
     if (!h->io_map || h->hb.empty()) return LB_OK;
     lb_status s = pull_bodies(h);
     if (s != LB_OK) return s;

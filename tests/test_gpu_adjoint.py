@@ -241,3 +241,27 @@ def test_calibration_recovers_the_parameter_of_a_target_drag(param, p_true, p0):
     assert abs(p / p_true - 1) < 1e-6, hist
     assert abs(xi / target - 1) < 1e-6
     assert len(hist) <= 8
+
+
+@pytest.mark.parametrize("precision", [64, 32])
+@pytest.mark.parametrize("schedule,snapshots", [(0, 0), (0, 1), (0, 5), (1, 1), (1, 3), (1, 30)])
+def test_handle_reads_as_after_plain_steps(precision, schedule, snapshots):
+    """What the handle reports after the adjoint is the state after nsteps: the
+    bodies and totals read back equal a handle's that only stepped, to the
+    tolerances of a forward run (the sweep's re-run and plain steps sum the
+    bodies' forces by atomics, in any order)."""
+    g, _ = _pair(precision, dict(MRT))
+    twin, _ = _pair(precision, dict(MRT))
+    before = twin.lb_get_body(0)["X"]
+    g.lb_adjoint_drag_ex(30, 10, body=0, axis=2, schedule=schedule, snapshots=snapshots)
+    twin.lb_step(30)
+    tol = 1e-12 if precision == 64 else 1e-5
+    a, b = g.lb_get_body(0), twin.lb_get_body(0)
+    assert np.abs(b["X"] - before).max() > 100 * tol
+    for k in a:
+        assert np.abs(a[k] - b[k]).max() <= tol * max(1.0, np.abs(b[k]).max())
+    for x, y in zip(g.lb_forces_all(), twin.lb_forces_all()):
+        assert np.abs(x - y).max() <= tol
+    g.lb_step(3)
+    twin.lb_step(3)
+    assert np.abs(g.lb_get_body(0)["X"] - twin.lb_get_body(0)["X"]).max() <= tol * np.abs(b["X"]).max()
