@@ -34,6 +34,7 @@ namespace lbk {
 #define LB_FIX_FN inline
 #endif
 
+// v = h 2^32 + l, l signed; v below 2^63 - 2^31 (from there on h would be 2^31)
 LB_FIX_FN FixPair fix_split(long long v) {
     FixPair p;
     p.l = (int)v;

@@ -438,11 +438,13 @@ __global__ void __launch_bounds__(32 * kWarps) k_msd_angle(const Limbs *fix, con
                         }
                         z = t2 + (t1 >> 28);
                     }
-                    if (z < 0) z = 0;
-                    // k by Horner's rule in u = z/2 - 1/2, |u| <= 1/2: the inner seven
-                    // steps (below 2^-14, and times u^12 at the end) in 32 bits
-                    const long long half = z << 8, u = half - (1LL << 62);   // z/2 and u at 2^63
-                    const int u32 = (int)(u >> 31);
+                    z = max(0LL, min(z, 1LL << 55));             // 2 may be passed by a rounding error
+                    // k by Horner's rule in u = z/2 - 1/2, |u| <= 1/2 (both ends are
+                    // reached: z = 0 and a right angle): the inner seven steps (below
+                    // 2^-14, and times u^12 at the end) in 32 bits
+                    const long long half = z << 7;                           // z/2 at 2^62
+                    const long long u = (half - (1LL << 61)) << 1;           // at 2^63
+                    const int u32 = (int)min(u >> 31, 0x7FFFFFFFLL);         // at 2^32
                     int ki = kAsinSq32[6];
 #pragma unroll
                     for (int j = 5; j >= 0; --j) ki = kAsinSq32[j] + __mulhi(ki, u32);
@@ -450,7 +452,7 @@ __global__ void __launch_bounds__(32 * kWarps) k_msd_angle(const Limbs *fix, con
                     const FixPair up = fix_split(u);
 #pragma unroll
                     for (int j = 11; j >= 0; --j) k = kAsinSq[j] + (fix_mul(fix_split(k), up) << 1);
-                    const long long B = fix_mul(fix_split(k), fix_split(half));   // z k at 2^62
+                    const long long B = fix_mul(fix_split(k), fix_split(half)) << 1;   // z k at 2^62
                     if (!far) {
                         accr[q] += (U128)(unsigned long long)z * (unsigned long long)B;
                     } else if (z >= (1LL << 46)) {

@@ -1,0 +1,61 @@
+"""The squared angle of lb_msd_trajectory (column 6) between reference vectors
+that stand at a chosen angle: records alternate between two orientations a
+rotation apart, so that every odd lag's average is that one pair's value.
+
+The expected value is the angle of the rotation itself, about the x axis with
+the reference vector along z. Tolerance: the vectors come from quaternions and
+rotation matrices rounded in FP64 (an angle error of up to 4e-16 each) and
+the evaluation is good to 2^-52 relative: 2 theta (8e-16) + 2e-16 theta^2
+< 6e-15 for theta up to pi."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+TOL = 6e-15
+
+
+def _squared_angles(qa, qb, lags=5, nrec=64):
+    from paper_1604_01829_gb300 import lb
+    q = np.zeros((1, nrec, 4))
+    q[0, 0::2], q[0, 1::2] = qa, qb
+    return lb.lb_msd_trajectory(np.zeros((1, nrec, 3)) + 1.0, q, lags, p_ref=(0, 0, 1))[0, :, 6]
+
+
+def _about_x(angle):
+    return [np.cos(angle / 2), np.sin(angle / 2), 0.0, 0.0]
+
+
+@pytest.mark.parametrize("qb", [(0.5, 0.5, 0.5, 0.5), (np.sqrt(0.5), np.sqrt(0.5), 0, 0), (np.sqrt(0.5), 0, -np.sqrt(0.5), 0)])
+def test_quarter_turns(qb):
+    got = _squared_angles((1, 0, 0, 0), qb)
+    assert np.abs(got[0::2] - np.pi ** 2 / 4).max() <= TOL
+    assert np.abs(got[1::2]).max() <= TOL
+
+
+@pytest.mark.parametrize("off", [1e-16, 1e-13, 1e-12, 1e-11, 1e-10, 2e-10, 2.4e-10, 3e-10, 1e-9, 1e-6])
+@pytest.mark.parametrize("side", [-1, 1])
+def test_angles_close_to_a_right_angle(off, side):
+    angle = np.pi / 2 + side * off
+    got = _squared_angles((1, 0, 0, 0), _about_x(angle))
+    assert np.abs(got[0::2] - angle ** 2).max() <= TOL
+    assert np.abs(got[1::2]).max() <= TOL
+
+
+def test_random_perpendicular_pairs():
+    """Pairs of rotations whose reference vectors are perpendicular to rounding, in any direction."""
+    from paper_1604_01829_gb300 import lb
+    rng = np.random.default_rng(4)
+    nb = 400
+    q = np.zeros((nb, 2, 4))
+    for b in range(nb):
+        p, r = rng.standard_normal((2, 3))
+        p /= np.linalg.norm(p)
+        r -= p * (p @ r)
+        r /= np.linalg.norm(r)
+        for k, v in enumerate((p, r)):                    # the rotation that takes z to v
+            h = np.array([1.0 + v[2], -v[1], v[0], 0.0])
+            q[b, k] = h / np.linalg.norm(h)
+    got = lb.lb_msd_trajectory(np.zeros((nb, 2, 3)), q, 1, p_ref=(0, 0, 1))[:, 0, 6]
+    # the frames built above are perpendicular to a few roundings, more for p or r close to -z
+    assert np.abs(got - np.pi ** 2 / 4).max() <= 1e-12
