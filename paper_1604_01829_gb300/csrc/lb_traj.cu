@@ -429,14 +429,17 @@ __global__ void __launch_bounds__(32 * kWarps) k_msd_angle(const Limbs *fix, con
                         z = 0;
                     }
                     if (far) {                   // the supplement's squared chord, from the sum of the vectors
-                        long long t1 = 0, t2 = 0;
+                        // to nearest: s = sqrt(z) passes z's error on over 2 s, and the low
+                        // product left out would be 12 units
+                        long long t0 = 0, t1 = 0, t2 = 0;
 #pragma unroll
                         for (int c = 0; c < 3; ++c) {
-                            const int e0 = v[c].l + a[c].l, e1 = v[c].h + a[c].h;
+                            const int e0 = v[c].l + a[c].l, e1 = v[c].h + a[c].h;    // e0 < 2^30
+                            t0 += (long long)e0 * e0;
                             t1 += (long long)e1 * e0;
                             t2 += (long long)e1 * e1;
                         }
-                        z = t2 + (t1 >> 28);
+                        z = t2 + ((t1 + (t0 >> 30) + (1LL << 27)) >> 28);
                     }
                     z = max(0LL, min(z, 1LL << 55));             // 2 may be passed by a rounding error
                     // k by Horner's rule in u = z/2 - 1/2, |u| <= 1/2 (both ends are
@@ -462,7 +465,7 @@ __global__ void __launch_bounds__(32 * kWarps) k_msd_angle(const Limbs *fix, con
                         long long r = fix_sqrt(zz + (fix_mul(fix_split(zz), fix_split(B)) << 2));
                         if (low) r >>= 2;
                         const FixPair th = fix_split(7244019458077122842LL - r);   // pi 2^61
-                        a2 = fix_mul(th, th) >> 4;                           // theta^2 at 2^54
+                        a2 = (fix_mul(th, th) + 8) >> 4;                     // theta^2 at 2^54
                     } else {
                         auto val = [](Limbs x) { return fma((double)x.h, 0x1p29, (double)x.l); };
                         const double w0[3] = {val(a[0]), val(a[1]), val(a[2])};
