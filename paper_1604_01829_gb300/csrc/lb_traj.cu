@@ -459,12 +459,13 @@ __global__ void __launch_bounds__(32 * kWarps) k_msd_angle(const Limbs *fix, con
                     if (!far) {
                         accr[q] += (U128)(unsigned long long)z * (unsigned long long)B;
                     } else if (z >= (1LL << 46)) {
-                        // theta = pi - s, s^2 = z (1 + z k), s from an integer square root
-                        const bool low = z < (1LL << 50);                    // below 2^-4: 16 s^2
-                        const long long zz = z << (low ? 11 : 7);             // at 2^61 (2^65)
-                        long long r = fix_sqrt(zz + (fix_mul(fix_split(zz), fix_split(B)) << 2));
-                        if (low) r >>= 2;
-                        const FixPair th = fix_split(7244019458077122842LL - r);   // pi 2^61
+                        // theta = pi - s, s^2 = z (1 + z k), s from an integer square root of
+                        // 4^j s^2 in [1/4, 1.24): m = 7 + 2 j odd, z's top bit to bit 59 or 60
+                        const int m = (__clzll(z) - 4) | 1;
+                        const long long zz = z << m;                         // 4^j z at 2^61
+                        const long long r = fix_sqrt(zz + (fix_mul(fix_split(zz), fix_split(B)) << 2));
+                        // pi 2^61 less s at 2^61 (j = -1 from z = 1 on)
+                        const FixPair th = fix_split(7244019458077122842LL - (m < 7 ? r << 1 : r >> ((m - 7) >> 1)));
                         a2 = (fix_mul(th, th) + 8) >> 4;                     // theta^2 at 2^54
                     } else {
                         auto val = [](Limbs x) { return fma((double)x.h, 0x1p29, (double)x.l); };

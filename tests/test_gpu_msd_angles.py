@@ -87,3 +87,14 @@ def test_angles_beyond_a_right_angle_are_not_biased():
         th = np.arctan2(np.sqrt((cr * cr).sum(1)), (a * b).sum(1))
         ref = float((th * th).mean())
         assert abs(got - ref) <= 2 * 2.0 ** -52 * ref
+
+
+@pytest.mark.parametrize("side", [1 - 1e-9, 1.0, 1 + 1e-9])
+@pytest.mark.parametrize("power", range(-10, 2))
+def test_supplements_at_every_scaling_switch(power, side):
+    """Squared chords of the supplement on both sides of each power of two,
+    where the square root's argument is scaled anew (below 2^-8: FP64). Half a
+    unit of 2^-54 in the chord's square is 2^-55 / s in theta."""
+    s = 2 * np.arcsin(0.5 * np.sqrt(side * 2.0 ** power))
+    got = _squared_angles((1, 0, 0, 0), _about_x(np.pi - s))
+    assert np.abs(got[0::2] - (np.pi - s) ** 2).max() <= TOL + 2 * np.pi * 2.0 ** -55 / s
