@@ -371,8 +371,8 @@ __device__ __forceinline__ void collide_node_f64(double (&f)[19], double Fx, dou
 
 // The fixed-point constants of a parameter set. rate[k - 4]: the relaxation
 // rate g_k of mode k = 4..18 (BGK: 1 - 1/tau for all). Not usable (on = 0)
-// when the noise could leave the range above (kT > 0.01 rho0) or the scaled
-// exponents the doubles'.
+// when the noise could leave the range above (kT > 0.01 rho0), the scaled
+// exponents the doubles', or a factor of the equilibrium fix_split's.
 inline FixParams fix_params(double rho0, double kT, const double rate[15]) {
     FixParams P{};
     int e = 0;
@@ -388,8 +388,12 @@ inline FixParams fix_params(double rho0, double kT, const double rate[15]) {
     static const long double b[15] = {2.0L / 3, 4.0L / 3, 4.0L / 9, 1.0L / 9, 1.0L / 9, 1.0L / 9, 2.0L / 3, 2.0L / 3,
                                       2.0L / 3, 2.0L / 9, 2.0L / 9, 2.0L / 9, 2.0L,     4.0L / 3, 4.0L / 9};
     for (int q = 0; q < 15; ++q) {
-        const long double c = 1.0L / 36 / b[q], g = rate[q];
-        P.ke[q] = fix_split(std::llrint(std::ldexp(c * (1 - g), 64)));
+        const long double c = 1.0L / 36 / b[q], g = rate[q], ke = std::ldexp(c * (1 - g), 64);
+        if (ke >= 0x1p63L - 0x1p31L) {         // c = 1/4 and g within 2^-31 of -1: beyond fix_split's range
+            P.on = 0;
+            return P;
+        }
+        P.ke[q] = fix_split(std::llrint(ke));
         if (q < 6) P.ks[q] = fix_split(std::llrint(std::ldexp(c * (1 + g) / 2, 64)));
         if (P.on) {
             const long double kn = c * std::sqrt(36.0L * kT * b[q] * (1 - g * g));

@@ -190,3 +190,25 @@ def test_mapped_results_follow_the_state():
     B.lb_batch_checkpoint_load(data)
     assert np.array_equal(B.lb_batch_get_body(1)["X"], got[1][0]["X"])
     assert np.array_equal(B.lb_batch_forces(1)[0], got[1][1][0])
+
+
+@pytest.mark.parametrize("gap", [2.0 ** -50, 1e-12, 2.0 ** -33, 2.0 ** -31, 2.0 ** -30, 1e-8])
+@pytest.mark.parametrize("case", ["bgk", "mrt", "noise"])
+def test_fp64_rates_close_to_minus_one(gap, case):
+    """Rates down to the closest to -1 that are accepted (tau - 1/2 = gap / 4),
+    where the weight of the equilibrium moments is 1/2 and its fixed-point form
+    ends; single lattices and batches."""
+    from paper_1604_01829_gb300 import lb
+    g = -1.0 + gap
+    params = (dict(collision=0, tau=0.5 + 0.25 * gap) if case == "bgk"
+              else dict(MRT, gamma_shear=g, kT=1e-4 if case == "noise" else 0.0, seed=3))
+    P = Pair(13, 7, 6, precision=64, body_force=(0.0, 1e-5, 0.0), **params)
+    f = perturbed_populations(P.N, seed=11)
+    P.set_populations(f)
+    P.step(1)
+    assert P.pop_error() <= TOL[64]
+    B = lb.LBBatch([dict(nx=13, ny=7, nz=6, precision=64, body_force=(0.0, 1e-5, 0.0), **params)])
+    B.lb_batch_set_populations(0, f)
+    B.lb_batch_step(1)
+    o = P.orc.populations()
+    assert np.max(np.abs(B.lb_batch_get_populations(0) - o) / W19[:, None]) <= TOL[64]
