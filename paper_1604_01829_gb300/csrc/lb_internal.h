@@ -263,8 +263,9 @@ cudaError_t launch_step_pre(Body *b, int nbodies, bool finish_prev, void *F, boo
 cudaError_t copy_records(const double *ring, int every, int cap, long long k0, long long step, int nb, int id,
                          int max_records, long long *steps, double *X, double *q, int *count, cudaStream_t s);
 
-// MSD analysis of recorded trajectories (lb_traj.cu); all pointers device
-cudaError_t launch_msd(const double *X, const double *q, int nrec, int nbodies, int max_lag, const double *p_ref,
+// MSD analysis of recorded trajectories (lb_traj.cu); all pointers device, q is
+// overwritten
+cudaError_t launch_msd(const double *X, double *q, int nrec, int nbodies, int max_lag, const double *p_ref,
                        void *work, double *out, cudaStream_t s);
 size_t msd_work_bytes(int nrec, int nbodies);
 // SMs of the current device

@@ -124,6 +124,9 @@ __global__ void __launch_bounds__(kThreads) k_msd_scan(int nrec, double *work) {
 // 64 times the rate. Measured for that case: 0.54 ms (k_msd_disp, 12 warp
 // instructions per 32 pairs and column) and 1.69 ms (k_msd_angle, bound by
 // its ~330, the polynomial mostly), the whole call 15.8 -> 2.85 ms.
+// The integer columns take the place of what they come from: X's three that of
+// the quaternions (read last by k_msd_prep), the others that of the work
+// columns, so the analysis needs no more memory than in FP64.
 constexpr int kFixCols = 12;       // X (3), body-frame trajectory (3), angles (3), p-hat (3)
 constexpr int kFixBits = 56;       // |value| < 2^56 about the middle of a column's range
 constexpr int kRun = 15;           // consecutive origins per lane and tile (odd: no bank conflicts)
@@ -137,30 +140,29 @@ struct Limbs {
     int l, h;
 };
 
-__device__ __forceinline__ Limbs limbs(long long v) {
-    Limbs o;
-    o.l = (int)((unsigned)v & 0x1FFFFFFFu);
-    o.h = (int)(v >> 29);
-    return o;
+// its two words as the bits of a double (of the column that it replaces)
+__device__ __forceinline__ double limbs(long long v) {
+    return __hiloint2double((int)(v >> 29), (int)((unsigned)v & 0x1FFFFFFFu));
 }
 
-// One block per (column, body): the column as integers about the middle of
-// its range, value = fix 2^unit; bad[body] is set where a value is not finite
-// or the scale is extreme (the FP64 kernel then takes the body).
-__global__ void __launch_bounds__(kThreads) k_msd_fix(const double *X, const double *work, int nrec, Limbs *fix,
-                                                    int *unit, int *bad) {
+// integer column c of body b (nrec values)
+__device__ __forceinline__ double *fix_column(double *q, double *work, int b, int c, int nrec) {
+    return c < 3 ? q + ((long long)b * 4 + c) * nrec : work + ((long long)b * kW + (c < 9 ? c : c - 9)) * nrec;
+}
+__device__ __forceinline__ const Limbs *fix_column(const double *q, const double *work, int b, int c, int nrec) {
+    return reinterpret_cast<const Limbs *>(fix_column(const_cast<double *>(q), const_cast<double *>(work), b, c, nrec));
+}
+
+// One block per (column, body): the exponent of the column's largest value, its
+// scale; bad[b] is set where a value is not finite or the scale is extreme (the
+// FP64 kernel then takes the body).
+__global__ void __launch_bounds__(kThreads) k_msd_scale(const double *X, const double *work, int nrec, int *unit,
+                                                      int *bad) {
     const int c = blockIdx.x, b = blockIdx.y;
-    const double *src;
-    long long st = 1;
-    if (c < 3) {
-        src = X + (long long)b * nrec * 3 + c;
-        st = 3;
-    } else {
-        src = work + ((long long)b * kW + (c < 9 ? c : c - 9)) * nrec;
-    }
-    Limbs *dst = fix + ((long long)b * kFixCols + c) * nrec;
+    const double *src = c < 3 ? X + (long long)b * nrec * 3 + c
+                              : work + ((long long)b * kW + (c < 9 ? c : c - 9)) * nrec;
+    const long long st = c < 3 ? 3 : 1;
     __shared__ double smax[kThreads];
-    __shared__ long long slo[kThreads], shi[kThreads];
     const int t = threadIdx.x;
     double m = 0.0;
     bool fine = true;
@@ -175,30 +177,40 @@ __global__ void __launch_bounds__(kThreads) k_msd_fix(const double *X, const dou
         if (t < w && smax[t + w] > smax[t]) smax[t] = smax[t + w];
         __syncthreads();
     }
+    if (t != 0) return;
     m = smax[0];
-    if (!fine || (m > 0.0 && m < 0x1p-400)) {
-        if (t == 0) bad[b] = 1;
-        return;
-    }
+    if (!fine || (m > 0.0 && m < 0x1p-400)) bad[b] = 1;
+    int e = 0;
+    frexp(m, &e);                                  // m < 2^e
+    unit[b * kFixCols + c] = e;
+}
+
+// One block per (column, body), the last one per body all of p-hat: the column
+// as integers about the middle of its range, value = fix 2^unit.
+__global__ void __launch_bounds__(kThreads) k_msd_fix(const double *X, double *q, double *work, int nrec, int *unit,
+                                                    const int *bad) {
+    const int c = blockIdx.x, b = blockIdx.y, t = threadIdx.x;
+    if (bad[b]) return;
+    double *dst = fix_column(q, work, b, c, nrec);
     if (c >= 9) {
         // p-hat: components of a unit vector at 2^56, the last rounding errors
         // of its length taken out (p - p off / 2, off = |p|^2 - 1 exactly)
-        const double *p = work + (long long)b * kW * nrec;
         for (int k = t; k < nrec; k += kThreads) {
             long long v[3];
             __int128 sum = -((__int128)1 << 112);
             for (int r = 0; r < 3; ++r) {
-                v[r] = __double2ll_rn(p[(long long)r * nrec + k] * 0x1p56);
+                v[r] = __double2ll_rn(dst[(long long)r * nrec + k] * 0x1p56);
                 sum += (__int128)v[r] * v[r];
             }
-            const long long mine = c == 9 ? v[0] : (c == 10 ? v[1] : v[2]);
-            dst[k] = limbs(mine - (long long)((__int128)mine * (long long)sum >> 113));
+            for (int r = 0; r < 3; ++r)
+                dst[(long long)r * nrec + k] = limbs(v[r] - (long long)((__int128)v[r] * (long long)sum >> 113));
         }
-        if (t == 0) unit[b * kFixCols + c] = -56;
         return;
     }
-    int e = 0;
-    frexp(m, &e);                                  // m < 2^e
+    const double *src = c < 3 ? X + (long long)b * nrec * 3 + c : dst;
+    const long long st = c < 3 ? 3 : 1;
+    __shared__ long long slo[kThreads], shi[kThreads];
+    const int e = unit[b * kFixCols + c];
     const double up = ldexp(1.0, 61 - e);
     long long lo = 0x7FFFFFFFFFFFFFFFLL, hi = -0x7FFFFFFFFFFFFFFFLL;
     for (int k = t; k < nrec; k += kThreads) {
@@ -223,7 +235,7 @@ __global__ void __launch_bounds__(kThreads) k_msd_fix(const double *X, const dou
     while ((half >> sh) >= (1LL << kFixBits) - 1) ++sh;
     const long long rnd = sh ? 1LL << (sh - 1) : 0;
     for (int k = t; k < nrec; k += kThreads) dst[k] = limbs((__double2ll_rn(src[k * st] * up) - mid + rnd) >> sh);
-    if (t == 0) unit[b * kFixCols + c] = e - 61 + sh;
+    if (t == 0) unit[b * kFixCols + c] = e - 61 + sh;          // read above by every thread, before the barriers
 }
 
 typedef unsigned __int128 U128;
@@ -246,11 +258,11 @@ __device__ __forceinline__ double to_double(U128 v) {
 // takes 8 lags, each lane 15 consecutive origins per tile and a sliding
 // window of 8 later records in registers (a quarter load per pair).
 constexpr int kLags = 8;
-__global__ void __launch_bounds__(32 * kWarps) k_msd_disp(const Limbs *fix, const int *unit, const int *bad,
-                                                         int nrec, int max_lag, double *out) {
+__global__ void __launch_bounds__(32 * kWarps) k_msd_disp(const double *fq, const double *work, const int *unit,
+                                                         const int *bad, int nrec, int max_lag, double *out) {
     const int c = blockIdx.y, b = blockIdx.z;
     if (bad[b]) return;
-    const Limbs *x = fix + ((long long)b * kFixCols + c) * nrec;
+    const Limbs *x = fix_column(fq, work, b, c, nrec);
     __shared__ Limbs s0[kTile], s1[kTile + kLags * kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int lb0 = blockIdx.x * kLags * kWarps + 1;      // first lag of the block
@@ -350,12 +362,12 @@ __constant__ long long kAsinSq[12] = {
 };
 __constant__ int kAsinSq32[7] = {1058753029, 642436037, 387510425, 203554602, 123855014, 139058146, 85944151};
 
-__global__ void __launch_bounds__(32 * kWarps) k_msd_angle(const Limbs *fix, const int *bad, int nrec, int max_lag,
-                                                         double *out) {
+__global__ void __launch_bounds__(32 * kWarps) k_msd_angle(const double *fq, const double *work, const int *bad,
+                                                         int nrec, int max_lag, double *out) {
     constexpr int LG = 4;                                 // lags per warp
     const int b = blockIdx.y;
     if (bad[b]) return;
-    const Limbs *x = fix + ((long long)b * kFixCols + 9) * nrec;
+    const Limbs *x = fix_column(fq, work, b, 9, nrec);
     __shared__ Limbs s0[3][kTile], s1[3][kTile + LG * kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int lb0 = blockIdx.x * LG * kWarps + 1, l0 = lb0 + warp * LG;
@@ -549,26 +561,26 @@ __global__ void __launch_bounds__(kThreads) k_msd_lags(const double *X, int nrec
 }  // namespace
 
 size_t msd_work_bytes(int nrec, int nbodies) {
-    const size_t n = (size_t)nrec * nbodies;
-    return n * kW * sizeof(double) + n * kFixCols * sizeof(Limbs) + (size_t)nbodies * (kFixCols + 1) * sizeof(int);
+    return (size_t)nrec * nbodies * kW * sizeof(double) + (size_t)nbodies * (kFixCols + 1) * sizeof(int);
 }
 
-cudaError_t launch_msd(const double *X, const double *q, int nrec, int nbodies, int max_lag, const double *p_ref,
+cudaError_t launch_msd(const double *X, double *q, int nrec, int nbodies, int max_lag, const double *p_ref,
                        void *work, double *out, cudaStream_t s) {
     const size_t n = (size_t)nrec * nbodies;
+    const unsigned nb = (unsigned)nbodies;
     double *w = static_cast<double *>(work);
-    Limbs *fix = reinterpret_cast<Limbs *>(w + n * kW);
-    int *unit = reinterpret_cast<int *>(fix + n * kFixCols), *bad = unit + (size_t)nbodies * kFixCols;
+    int *unit = reinterpret_cast<int *>(w + n * kW), *bad = unit + (size_t)nbodies * kFixCols;
     cudaError_t e = cudaMemsetAsync(bad, 0, sizeof(int) * nbodies, s);
     if (e != cudaSuccess) return e;
     k_msd_prep<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(X, q, nrec, nbodies, p_ref, w);
-    k_msd_scan<<<dim3(6, (unsigned)nbodies), kThreads, 0, s>>>(nrec, w);
-    k_msd_fix<<<dim3(kFixCols, (unsigned)nbodies), kThreads, 0, s>>>(X, w, nrec, fix, unit, bad);
+    k_msd_scan<<<dim3(6, nb), kThreads, 0, s>>>(nrec, w);
+    k_msd_scale<<<dim3(kFixCols, nb), kThreads, 0, s>>>(X, w, nrec, unit, bad);
+    k_msd_fix<<<dim3(10, nb), kThreads, 0, s>>>(X, q, w, nrec, unit, bad);
     const unsigned gd = (unsigned)((max_lag + kLags * kWarps - 1) / (kLags * kWarps));
-    k_msd_disp<<<dim3(gd, 9, (unsigned)nbodies), 32 * kWarps, 0, s>>>(fix, unit, bad, nrec, max_lag, out);
+    k_msd_disp<<<dim3(gd, 9, nb), 32 * kWarps, 0, s>>>(q, w, unit, bad, nrec, max_lag, out);
     const unsigned ga = (unsigned)((max_lag + 4 * kWarps - 1) / (4 * kWarps));
-    k_msd_angle<<<dim3(ga, (unsigned)nbodies), 32 * kWarps, 0, s>>>(fix, bad, nrec, max_lag, out);
-    k_msd_lags<<<dim3((unsigned)std::min(max_lag, std::max(8, 2048 / nbodies)), (unsigned)nbodies), kThreads, 0, s>>>(X, nrec, max_lag, w, bad, out);
+    k_msd_angle<<<dim3(ga, nb), 32 * kWarps, 0, s>>>(q, w, bad, nrec, max_lag, out);
+    k_msd_lags<<<dim3((unsigned)std::min(max_lag, std::max(8, 2048 / nbodies)), nb), kThreads, 0, s>>>(X, nrec, max_lag, w, bad, out);
     return cudaGetLastError();
 }
 
