@@ -66,9 +66,10 @@ __global__ void k_msd_prep(const double *X, const double *q, int nrec, int nb, c
     double p[3];
     for (int r = 0; r < 3; ++r) p[r] = (ak[0][r] * p_ref[0] + ak[1][r] * p_ref[1] + ak[2][r] * p_ref[2]) / pn;
     // a quaternion that is not a unit one to rounding: the length is taken out
-    // (the squared chord of k_msd_angle scales with it)
-    const double off = fma(p[0], p[0], fma(p[1], p[1], fma(p[2], p[2], -1.0)));
-    const double len = fabs(off) > 0x1p-50 ? sqrt(dot3(p, p)) : 1.0;
+    // (the squared chord of k_msd_angle scales with it), unless it has none in
+    // FP64 (the vector is 0, or its square under- or overflows)
+    const double off = fma(p[0], p[0], fma(p[1], p[1], fma(p[2], p[2], -1.0))), n2 = dot3(p, p);
+    const double len = fabs(off) > 0x1p-50 && n2 > 0.0 && n2 < 0x1p1023 ? sqrt(n2) : 1.0;
     for (int r = 0; r < 3; ++r) w[(long long)r * nrec] = p[r] / len;
     if (k == 0) {
         for (int c = 3; c < kW; ++c) w[(long long)c * nrec] = 0.0;
@@ -154,8 +155,8 @@ __device__ __forceinline__ const Limbs *fix_column(const double *q, const double
 }
 
 // One block per (column, body): the exponent of the column's largest value, its
-// scale; bad[b] is set where a value is not finite or the scale is extreme (the
-// FP64 kernel then takes the body).
+// scale; bad[b] is set where a value is not finite, the scale is extreme or a
+// reference vector has no length (the FP64 kernel then takes the body).
 __global__ void __launch_bounds__(kThreads) k_msd_scale(const double *X, const double *work, int nrec, int *unit,
                                                       int *bad) {
     const int c = blockIdx.x, b = blockIdx.y;
@@ -169,6 +170,10 @@ __global__ void __launch_bounds__(kThreads) k_msd_scale(const double *X, const d
     for (int k = t; k < nrec; k += kThreads) {
         const double v = fabs(src[k * st]);
         fine = fine && v < 0x1p400;
+        if (c == 9) {                              // p-hat: a unit vector
+            const double p1 = src[k + (long long)nrec], p2 = src[k + 2LL * nrec];
+            fine = fine && fabs(fma(v, v, fma(p1, p1, fma(p2, p2, -1.0)))) < 0x1p-40;
+        }
         if (v > m) m = v;
     }
     smax[t] = m;
@@ -512,7 +517,7 @@ __global__ void __launch_bounds__(32 * kWarps) k_msd_angle(const double *fq, con
 }
 
 // The same averages in FP64 (blocks over lags and bodies), for the bodies
-// that k_msd_fix marked: non-finite values spread to the lags they take part
+// that k_msd_scale marked: non-finite values spread to the lags they take part
 // in.
 __global__ void __launch_bounds__(kThreads) k_msd_lags(const double *X, int nrec, int max_lag, const double *work,
                                                      const int *bad, double *out) {

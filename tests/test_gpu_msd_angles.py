@@ -98,3 +98,17 @@ def test_supplements_at_every_scaling_switch(power, side):
     s = 2 * np.arcsin(0.5 * np.sqrt(side * 2.0 ** power))
     got = _squared_angles((1, 0, 0, 0), _about_x(np.pi - s))
     assert np.abs(got[0::2] - (np.pi - s) ** 2).max() <= TOL + 2 * np.pi * 2.0 ** -55 / s
+
+
+@pytest.mark.parametrize("qb", [(0, 0.5, 0.5, 0), (0, 0.5 * (1 - 2.0 ** -40), 0.5, 0), (0, 3e100, 1e90, 0)])
+def test_quaternions_that_leave_no_unit_vector(qb):
+    """Quaternions far from unit length whose matrix takes the reference vector
+    to 0, nearly to 0 or beyond the squares' range: the angle is the
+    arctangent's of the vectors as they are (0 between a vector and 0)."""
+    w, x, y, z = qb
+    p = np.array([2 * (x * z + y * w), 2 * (y * z - x * w), 1 - 2 * (x * x + y * y)])
+    with np.errstate(over="ignore", invalid="ignore"):
+        th = np.arctan2(np.hypot(p[0], p[1]), p[2])        # against (0, 0, 1)
+    got = _squared_angles((1, 0, 0, 0), qb)
+    assert np.abs(got[0::2] - th ** 2).max() <= TOL
+    assert np.abs(got[1::2]).max() <= TOL
