@@ -134,6 +134,7 @@ constexpr int kRun = 15;           // consecutive origins per lane and tile (odd
 constexpr int kTile = 32 * kRun;   // origins per tile
 constexpr int kTilesPerSum = 8;    // tiles until the 128-bit sums (< 2^114 a term, 3840 terms) are taken off
 constexpr int kWarps = 8;
+constexpr int kExact = -0x7FFFFFFF;    // a column of X that its integers hold exactly (k_msd_near)
 
 // a value v of a column as h 2^29 + l, 0 <= l < 2^29: the difference of two is
 // (h1 - h0) 2^29 + (l1 - l0), two subtractions without a carry
@@ -235,12 +236,22 @@ __global__ void __launch_bounds__(kThreads) k_msd_fix(const double *X, double *q
     }
     lo = slo[0];
     hi = shi[0];
-    const long long mid = lo / 2 + hi / 2, half = (hi - lo) / 2 + 2;
+    const long long half = (hi - lo) / 2 + 2;
     int sh = 0;
-    while ((half >> sh) >= (1LL << kFixBits) - 1) ++sh;
-    const long long rnd = sh ? 1LL << (sh - 1) : 0;
-    for (int k = t; k < nrec; k += kThreads) dst[k] = limbs((__double2ll_rn(src[k * st] * up) - mid + rnd) >> sh);
-    if (t == 0) unit[b * kFixCols + c] = e - 61 + sh;          // read above by every thread, before the barriers
+    while ((half >> sh) >= (1LL << kFixBits) - 3) ++sh;
+    const long long low = (1LL << sh) - 1, mid = (lo / 2 + hi / 2) & ~low, rnd = (low + 1) >> 1;
+    bool coarse = false;
+    for (int k = t; k < nrec; k += kThreads) {
+        const double v = src[k * st] * up;
+        const long long r = __double2ll_rn(v);
+        coarse |= v != rint(v) || (r & low);
+        dst[k] = limbs((r - mid + rnd) >> sh);
+    }
+    coarse = __syncthreads_or(coarse);
+    if (t != 0) return;
+    unit[b * kFixCols + c] = e - 61 + sh;
+    // X: the exponent of the column's range, where its grid is coarser than a value (p-hat has no use for the place)
+    if (c < 3) unit[b * kFixCols + 9 + c] = coarse ? 64 - __clzll(hi - lo) + e - 61 : kExact;
 }
 
 typedef unsigned __int128 U128;
@@ -516,6 +527,53 @@ __global__ void __launch_bounds__(32 * kWarps) k_msd_angle(const double *fq, con
         out[((long long)b * max_lag + (l - 1)) * LB_MSD_COLS + 6] = total / (double)(nrec - l);
 }
 
+// X's averages that a column's grid is too coarse for, again in FP64. The grid
+// is 2^-57 of the column's range: where every record takes part in a lag, the
+// average is at least 1/n of the range squared and the grid's errors (random,
+// and summed over n pairs) stay below the rounding of an FP64 evaluation. A lag
+// beyond half the trajectory leaves out the records in its middle, and the
+// rest may have moved by far less than the range: an average below 2^(2 s - 8)
+// / n, 2^s the range, is recomputed from the values themselves. (The other
+// columns are running sums, whose own rounding in such a trajectory is larger
+// than the grid.) Nothing to do where the integers are exact, as they are for
+// values away from 0 by more than 1/8 of their range.
+__global__ void __launch_bounds__(kThreads) k_msd_near(const double *X, int nrec, int max_lag, const int *unit,
+                                                     const int *bad, double *out) {
+    const int b = blockIdx.y;
+    const int *span = unit + b * kFixCols + 9;
+    if (bad[b] || (span[0] == kExact && span[1] == kExact && span[2] == kExact)) return;
+    const double *Xb = X + (long long)b * nrec * 3;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __shared__ double red[3][kThreads / 32];
+    for (int l = blockIdx.x + 1; l <= max_lag; l += gridDim.x) {
+        const int n = nrec - l;
+        double *o = out + ((long long)b * max_lag + (l - 1)) * LB_MSD_COLS;
+        int need = 0;                        // the same in every thread: written below, after a barrier
+        for (int a = 0; a < 3; ++a)
+            if (span[a] != kExact && o[a] < ldexp(1.0, 2 * span[a] - 8) / (double)n) need |= 1 << a;
+        if (!need) continue;
+        double acc[3] = {0.0, 0.0, 0.0};
+        for (int t = threadIdx.x; t < n; t += kThreads) {
+            const double *x0 = Xb + (long long)t * 3, *x1 = Xb + (long long)(t + l) * 3;
+            for (int a = 0; a < 3; ++a) {
+                const double d = x1[a] - x0[a];
+                acc[a] += d * d;
+            }
+        }
+        for (int a = 0; a < 3; ++a) {
+            for (int k = 16; k > 0; k >>= 1) acc[a] += __shfl_down_sync(0xffffffffu, acc[a], k);
+            if (lane == 0) red[a][warp] = acc[a];
+        }
+        __syncthreads();
+        if (threadIdx.x < 3 && (need >> threadIdx.x & 1)) {
+            double v = 0.0;
+            for (int w = 0; w < kThreads / 32; ++w) v += red[threadIdx.x][w];
+            o[threadIdx.x] = v / (double)n;
+        }
+        __syncthreads();                     // red is reused
+    }
+}
+
 // The same averages in FP64 (blocks over lags and bodies), for the bodies
 // that k_msd_scale marked: non-finite values spread to the lags they take part
 // in.
@@ -585,7 +643,9 @@ cudaError_t launch_msd(const double *X, double *q, int nrec, int nbodies, int ma
     k_msd_disp<<<dim3(gd, 9, nb), 32 * kWarps, 0, s>>>(q, w, unit, bad, nrec, max_lag, out);
     const unsigned ga = (unsigned)((max_lag + 4 * kWarps - 1) / (4 * kWarps));
     k_msd_angle<<<dim3(ga, nb), 32 * kWarps, 0, s>>>(q, w, bad, nrec, max_lag, out);
-    k_msd_lags<<<dim3((unsigned)std::min(max_lag, std::max(8, 2048 / nbodies)), nb), kThreads, 0, s>>>(X, nrec, max_lag, w, bad, out);
+    const dim3 gl((unsigned)std::min(max_lag, std::max(8, 2048 / nbodies)), nb);
+    k_msd_near<<<gl, kThreads, 0, s>>>(X, nrec, max_lag, unit, bad, out);
+    k_msd_lags<<<gl, kThreads, 0, s>>>(X, nrec, max_lag, w, bad, out);
     return cudaGetLastError();
 }
 
