@@ -528,8 +528,10 @@ typedef struct {
     int project_final;       /* 1: end with every bead on its nearest surface point  */
     int pair_search;         /* 0: automatic (per-bead neighbour lists kept over many steps
                                 where they fit in shared memory: up to about 2640 beads in
-                                FP32, 2048 in FP64; larger shells: the cell list when it fits,
-                                else all pairs); 1: all pairs; 2: cell list
+                                FP32, 2048 in FP64; the longer lists of crowded shells, more
+                                than about 2.4 beads per unit area at the default sigma, in
+                                device memory, 1 GB at most; larger shells: the cell list when
+                                it fits, else all pairs); 1: all pairs; 2: cell list
                                 (cells at least as wide as the WCA range, rebuilt every
                                 step; a step with a bead outside the box 1.25 a + 1
                                 around the centre tests all pairs). The results agree

@@ -61,6 +61,11 @@ struct ShellArgs {
     int max_cells;            // largest grid (shared-memory extent)
     int *err;                 // index checks of checked builds (LB_CHECKS): bit 2 on failure
     R rl2, move2;             // neighbour lists: (range + skin)^2 and the squared move that outdates them
+    // lists of crowded shells in device memory: [nshells][list_rows][max_count],
+    // the longest list of each shell
+    uint16_t *glist;
+    const int *list_len;
+    int list_rows;
 };
 
 __device__ __forceinline__ float rdiv(float a, float b) { return __fdividef(a, b); }
@@ -358,7 +363,14 @@ __global__ void __launch_bounds__(kShellThreads) k_relax_shells(const ShellArgs<
 // was built, in index order, and stays complete until some bead has moved by
 // skin / 2; the pairs outside the range add nothing, so every step sums what
 // the all-pairs search sums, in the same order. A list longer than kListLen
-// is not kept: its bead tests all pairs.
+// is not kept: its bead tests all pairs. Crowded shells (LONG: more than
+// kCrowded beads expected within rl of a bead) have longer lists in device
+// memory, read through L1: at kListLen most of their beads would test all
+// pairs. Per step, with short lists, long ones and the cell list: FP32 2000
+// beads at three a unit area 279 / 18.7 / 117 us, 900 there 59 / 8.3 / 59, 200
+// at six 18.6 / 7.4 / -; FP64 2000 at three 7204 / 724 / 4818. A shell that
+// flies apart rebuilds its lists every step whatever their length (2000 at six,
+// dt^2 times the forces ~0.01: 661 / 401 / 332).
 //
 // One block per shell, positions in two shared buffers (one barrier a step),
 // velocities, list references and surface roots in registers. Bound by the
@@ -370,6 +382,8 @@ __global__ void __launch_bounds__(kShellThreads) k_relax_shells(const ShellArgs<
 // one shell of 2400 beads 117 -> 14.8 us (cell list); FP64, the 203 shells:
 // 1134 -> 98 us (its divisions on the FP64 pipe).
 constexpr int kListLen = 32;
+constexpr double kCrowded = 24.0;
+constexpr size_t kLongBytes = 1ull << 30;           // device memory for long lists at most
 #ifndef LB_LIST_SKIN
 #define LB_LIST_SKIN 0.15
 #endif
@@ -378,13 +392,16 @@ constexpr int kListLen = 32;
 template <typename R>
 constexpr int list_threads() { return sizeof(R) == 8 ? 512 : 1024; }
 
-template <typename R, int BPT>
+template <typename R, int BPT, bool LONG>
 __global__ void __launch_bounds__(list_threads<R>()) k_relax_list(const ShellArgs<R> a) {
     extern __shared__ unsigned char smem_raw[];
     R *pos = reinterpret_cast<R *>(smem_raw);                          // [2][3][max_count]
-    uint16_t *list = reinterpret_cast<uint16_t *>(pos + 6 * (size_t)a.max_count);   // [kListLen][max_count]
     const int M = a.max_count;
     const int s = blockIdx.x;
+    uint16_t *list;                                                    // [cap][max_count]
+    if constexpr (LONG) list = a.glist + (size_t)s * a.list_rows * M;
+    else list = reinterpret_cast<uint16_t *>(pos + 6 * (size_t)M);
+    const int cap = LONG ? a.list_len[s] : kListLen;
     const int n = a.count[s];
     double *X = a.xyz + 3 * a.offset[s];
     const R ax = (R)a.axes[3 * s], ay = (R)a.axes[3 * s + 1], az = (R)a.axes[3 * s + 2];
@@ -418,13 +435,13 @@ __global__ void __launch_bounds__(list_threads<R>()) k_relax_list(const ShellArg
                 for (int j = 0; j < n; ++j) {
                     const R dx = xi[b] - px[j], dy = yi[b] - py[j], dz = zi[b] - pz[j];
                     if (dx * dx + dy * dy + dz * dz < a.rl2 && j != i) {
-                        if (k < kListLen) list[(size_t)k * M + i] = (uint16_t)j;
+                        if (k < cap) list[(size_t)k * M + i] = (uint16_t)j;
                         ++k;
                     }
                 }
                 // padded to whole groups of four with the bead itself
-                for (int q = k; q < ((k + 3) & ~3) && q < kListLen; ++q) list[(size_t)q * M + i] = (uint16_t)i;
-                len[b] = k <= kListLen ? k : -1;
+                for (int q = k; q < ((k + 3) & ~3) && q < cap; ++q) list[(size_t)q * M + i] = (uint16_t)i;
+                len[b] = k <= cap ? k : -1;
                 rx[b] = xi[b];
                 ry[b] = yi[b];
                 rz[b] = zi[b];
@@ -507,13 +524,37 @@ size_t list_smem(size_t rsize, int max_count) {
     return 6 * rsize * (size_t)max_count + sizeof(uint16_t) * kListLen * (size_t)max_count;
 }
 
-template <typename R, int BPT>
+// surface area by Thomsen's formula (within 1.1 %)
+double ellipsoid_area(const double *a) {
+    const double p = 1.6075, x = std::pow(a[0] * a[1], p) + std::pow(a[0] * a[2], p) + std::pow(a[1] * a[2], p);
+    return 4.0 * 3.141592653589793 * std::pow(x / 3.0, 1.0 / p);
+}
+
+// The longest list to keep for a shell of n beads: a spherical cap of chord
+// radius rl has the area pi rl^2, so n pi rl^2 / area beads lie within rl of an
+// evenly spread bead; half as many again, and a few, for uneven spreads. A
+// value of this shell alone: shells relaxed together are relaxed as each alone.
+int list_rows(const double *axes, int n, double sigma) {
+    const double rl = (kWcaCut + LB_LIST_SKIN) * sigma, near = n * 3.141592653589793 * rl * rl / ellipsoid_area(axes);
+    if (n <= kListLen || !(near > kCrowded)) return kListLen;
+    return (int)std::min((n + 3.0) / 4.0, 0.375 * near + 5.0) * 4;
+}
+
+template <typename R, int BPT, bool LONG>
 cudaError_t launch_list_t(const ShellArgs<R> &a, int nshells, int threads, cudaStream_t s) {
-    const size_t smem = list_smem(sizeof(R), a.max_count);
-    cudaError_t e = cudaFuncSetAttribute(k_relax_list<R, BPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = LONG ? 6 * sizeof(R) * (size_t)a.max_count : list_smem(sizeof(R), a.max_count);
+    cudaError_t e = cudaFuncSetAttribute(k_relax_list<R, BPT, LONG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
     if (e != cudaSuccess) return e;
-    k_relax_list<R, BPT><<<nshells, threads, smem, s>>>(a);
+    k_relax_list<R, BPT, LONG><<<nshells, threads, smem, s>>>(a);
     return cudaGetLastError();
+}
+
+template <typename R, bool LONG>
+cudaError_t launch_list(const ShellArgs<R> &a, int bpt, int nshells, int threads, cudaStream_t s) {
+    if (bpt == 1) return launch_list_t<R, 1, LONG>(a, nshells, threads, s);
+    if (bpt == 2) return launch_list_t<R, 2, LONG>(a, nshells, threads, s);
+    return launch_list_t<R, 4, LONG>(a, nshells, threads, s);
 }
 
 size_t shell_smem(size_t rsize, int max_count, int max_cells, bool cells) {
@@ -554,9 +595,7 @@ cudaError_t launch_shells(ShellArgs<R> a, const lb_shell_params &p, int nshells,
         const double skin = LB_LIST_SKIN * p.sigma, rl = kWcaCut * p.sigma + skin;
         a.rl2 = (R)(rl * rl);
         a.move2 = (R)(0.98 * 0.25 * skin * skin);
-        if (bpt == 1) return launch_list_t<R, 1>(a, nshells, threads, s);
-        if (bpt == 2) return launch_list_t<R, 2>(a, nshells, threads, s);
-        return launch_list_t<R, 4>(a, nshells, threads, s);
+        return a.glist ? launch_list<R, true>(a, bpt, nshells, threads, s) : launch_list<R, false>(a, bpt, nshells, threads, s);
     }
     if (cells) {
         if (bpt == 1) return launch_shells_t<R, 1, true>(a, nshells, threads, s);
@@ -642,12 +681,29 @@ extern "C" lb_status lb_relax_shells(int nshells, const double *axes, const int 
     const bool lists = p->pair_search == 0 && max_count <= list_cap && lbk::list_smem(rsize, max_count) <= (size_t)optin;
     const bool cells = p->pair_search == 2 || (p->pair_search == 0 && !lists && cells_fit);
 
+    // longer lists where a shell is crowded (without them, as without their
+    // memory: lists of kListLen)
+    std::vector<int> rows(nshells, lbk::kListLen);
+    int max_rows = lbk::kListLen;
+    if (lists)
+        for (int s = 0; s < nshells; ++s) {
+            rows[s] = lbk::list_rows(axes + 3 * s, counts[s], p->sigma);
+            max_rows = std::max(max_rows, rows[s]);
+        }
+    const size_t long_bytes = sizeof(uint16_t) * (size_t)nshells * max_rows * max_count;
+    bool longer = max_rows > lbk::kListLen && long_bytes <= lbk::kLongBytes;
+
     cudaStream_t st = (cudaStream_t)cuda_stream;
     const size_t nd = (size_t)3 * nshells + (size_t)3 * total + (size_t)3 * nshells;
-    const size_t bytes = nd * sizeof(double) + (size_t)nshells * (sizeof(long long) + sizeof(int) + 3 * sizeof(int)) +
+    const size_t bytes = nd * sizeof(double) + (size_t)nshells * (sizeof(long long) + sizeof(int) + 4 * sizeof(int)) +
                          sizeof(int);
     void *d = nullptr;
-    e = cudaMalloc(&d, bytes);
+    e = cudaMalloc(&d, bytes + (longer ? long_bytes : 0));
+    if (e == cudaErrorMemoryAllocation && longer) {
+        cudaGetLastError();
+        longer = false;
+        e = cudaMalloc(&d, bytes);
+    }
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
         return fail(LB_ERR_OOM, "device allocation for the shells failed");
@@ -657,7 +713,9 @@ extern "C" lb_status lb_relax_shells(int nshells, const double *axes, const int 
     long long *doff = reinterpret_cast<long long *>(dbox + 3 * nshells);
     int *dcount = reinterpret_cast<int *>(doff + nshells);
     int *dgrid = dcount + nshells;
-    int *derr = dgrid + 3 * nshells;             // index checks of checked builds
+    int *drows = dgrid + 3 * nshells;
+    int *derr = drows + nshells;                 // index checks of checked builds
+    uint16_t *dlong = longer ? reinterpret_cast<uint16_t *>(derr + 1) : nullptr;
     std::vector<double> out((size_t)3 * total);
     e = cudaMemcpyAsync(daxes, axes, 3 * nshells * sizeof(double), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(dxyz, xyz, 3 * total * sizeof(double), cudaMemcpyHostToDevice, st);
@@ -665,17 +723,21 @@ extern "C" lb_status lb_relax_shells(int nshells, const double *axes, const int 
     if (e == cudaSuccess) e = cudaMemcpyAsync(dcount, counts, nshells * sizeof(int), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(dbox, box.data(), 3 * nshells * sizeof(double), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(dgrid, grid.data(), 3 * nshells * sizeof(int), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess && longer)
+        e = cudaMemcpyAsync(drows, rows.data(), nshells * sizeof(int), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(derr, 0, sizeof(int), st);
     if (e == cudaSuccess) {
         if (p->precision == 64) {
             lbk::ShellArgs<double> a{};
             a.axes = daxes; a.count = dcount; a.offset = doff; a.xyz = dxyz; a.max_count = max_count;
             a.cgrid = dgrid; a.cbox = dbox; a.max_cells = cells ? max_cells : 1; a.err = derr;
+            a.glist = dlong; a.list_len = drows; a.list_rows = max_rows;
             e = lbk::launch_shells<double>(a, *p, nshells, cells, lists, st);
         } else {
             lbk::ShellArgs<float> a{};
             a.axes = daxes; a.count = dcount; a.offset = doff; a.xyz = dxyz; a.max_count = max_count;
             a.cgrid = dgrid; a.cbox = dbox; a.max_cells = cells ? max_cells : 1; a.err = derr;
+            a.glist = dlong; a.list_len = drows; a.list_rows = max_rows;
             e = lbk::launch_shells<float>(a, *p, nshells, cells, lists, st);
         }
     }

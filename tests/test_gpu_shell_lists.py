@@ -68,3 +68,50 @@ def test_many_shells_equal_each_alone():
     together = lb.lb_relax_shells(axes, starts, steps=60, precision=32)
     for s in (0, 11, 29):
         assert np.array_equal(lb.lb_relax_shells([axes[s]], [starts[s]], steps=60, precision=32)[0], together[s])
+
+
+@pytest.mark.parametrize("precision", [64, 32])
+@pytest.mark.parametrize("n,density", [(32, 6.0), (33, 6.0), (200, 6.0), (255, 2.3), (255, 2.6), (900, 6.0), (1100, 3.0), (2000, 6.0),
+                                       (4, 100.0), (600, 100.0)])
+def test_crowded_shells(n, density, precision):
+    """Both sides of the density from which lists are longer (24 beads in the list
+    radius: 2.4 a unit area), up to lists of every other bead: as all pairs."""
+    from paper_1604_01829_gb300 import lb, workloads as W
+    a = np.sqrt(n / density / (4 * np.pi))
+    X0 = W.spread_shell_start(a, a, a, n, seed=n)
+    # small steps: 20 of them stay far from the chaos of a shell that blows up
+    dt = 1e-6 if density < 50 else 1e-12
+    got = [lb.lb_relax_shells([(a, a, a)], [X0], steps=20, dt=dt, eta=1.0 / dt, precision=precision, project_final=False,
+                              pair_search=s)[0] for s in (0, 1)]
+    assert np.abs(got[0] - got[1]).max() <= TOL[precision]
+
+
+@pytest.mark.parametrize("precision", [64, 32])
+def test_crowded_and_loose_shells_together(precision):
+    """Shells with short and long lists in one call as each alone: bit for bit in
+    FP32, in FP64 to the rounding of kernels that carry 1 or 2 beads a thread."""
+    from paper_1604_01829_gb300 import lb, workloads as W
+    axes, starts = [], []
+    for n, density in ((300, 1.0), (300, 6.0), (40, 3.0), (700, 2.0), (700, 3.5)):
+        a = np.sqrt(n / density / (4 * np.pi))
+        axes.append((a, a, a))
+        starts.append(W.spread_shell_start(a, a, a, n, seed=n))
+    kw = dict(steps=30, dt=1e-6, eta=1e6, precision=precision)
+    together = lb.lb_relax_shells(axes, starts, **kw)
+    for s in range(5):
+        alone = lb.lb_relax_shells([axes[s]], [starts[s]], **kw)[0]
+        assert np.abs(alone - together[s]).max() <= (1e-12 if precision == 64 else 0.0)
+
+
+@pytest.mark.parametrize("precision", [64, 32])
+def test_a_clump_on_a_loose_shell(precision):
+    """45 beads within one list radius of each other on a shell of one bead a unit
+    area: more than a list holds, the others' lists do."""
+    from paper_1604_01829_gb300 import lb, workloads as W
+    a = 6.0
+    X0 = W.spread_shell_start(a, a, a, 400, seed=3)
+    rng = np.random.default_rng(5)
+    X0[100:145] = X0[7] + 0.4 * rng.standard_normal((45, 3))
+    got = [lb.lb_relax_shells([(a, a, a)], [X0], steps=20, dt=1e-8, eta=1e8, precision=precision, project_final=False,
+                              pair_search=s)[0] for s in (0, 1)]
+    assert np.abs(got[0] - got[1]).max() <= TOL[precision]
