@@ -879,6 +879,12 @@ lb_status launch_chain(lb_ctx *h, int n) {
                                                          h->stream);
         if (e != cudaSuccess) return cuda_fail(h, e, "chained collide_stream launch");
     }
+#ifdef LB_CHECKS
+    // the last fluid kernel's own index checks count too (other builds' fluid
+    // kernels write no error word here)
+    if (s == LB_OK && h->io_dmap)
+        LB_CUDA(h, lbk::launch_error_word(h->io_dmap + 12 * h->hb.size(), h->err_dev, h->stream));
+#endif
     return s;
 }
 

@@ -50,6 +50,8 @@ __global__ void k_finish(Body *bodies, int nb, double dt, unsigned long long *st
     }
 }
 
+__global__ void k_error_word(double *out, const int *err) { *out = (double)*err; }
+
 // Between two MD substeps of one LB step: the finished substep's second half
 // kick, the next substep's first half kick and drift (and the trajectory
 // record after the last substep's drift).
@@ -127,6 +129,11 @@ cudaError_t launch_couple(const CoupleArgs &a, cudaStream_t s) {
 cudaError_t launch_finish(Body *b, int nbodies, double dt, unsigned long long *step, unsigned int by, cudaStream_t s,
                           double *out, const int *err) {
     k_finish<<<nbodies > 0 ? nbodies : 1, 32, 0, s>>>(b, nbodies > 0 ? nbodies : 0, dt, step, by, out, err);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_error_word(double *out, const int *err, cudaStream_t s) {
+    k_error_word<<<1, 1, 0, s>>>(out, err);
     return cudaGetLastError();
 }
 

@@ -280,6 +280,9 @@ cudaError_t launch_couple(const CoupleArgs &a, cudaStream_t s);
 // counter advance, in one launch (nbodies may be 0)
 cudaError_t launch_finish(Body *b, int nbodies, double dt, unsigned long long *step, unsigned int by, cudaStream_t s,
                           double *out = nullptr, const int *err = nullptr);
+// checked builds: *out = *err once every kernel queued before has run (the extra
+// blocks of a chained group's last fluid kernel run beside it)
+cudaError_t launch_error_word(double *out, const int *err, cudaStream_t s);
 // between MD substeps: second half kick, next first half kick and drift (dt each)
 cudaError_t launch_substep(Body *b, int nbodies, double dt, const Recorder &rec, cudaStream_t s);
 
