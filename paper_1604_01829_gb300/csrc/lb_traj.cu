@@ -168,6 +168,7 @@ __global__ void __launch_bounds__(kThreads) k_msd_scale(const double *X, const d
     const int t = threadIdx.x;
     double m = 0.0;
     bool fine = true;
+#pragma unroll 4
     for (int k = t; k < nrec; k += kThreads) {
         const double v = fabs(src[k * st]);
         fine = fine && v < 0x1p400;
@@ -219,6 +220,7 @@ __global__ void __launch_bounds__(kThreads) k_msd_fix(const double *X, double *q
     const int e = unit[b * kFixCols + c];
     const double up = ldexp(1.0, 61 - e);
     long long lo = 0x7FFFFFFFFFFFFFFFLL, hi = -0x7FFFFFFFFFFFFFFFLL;
+#pragma unroll 4
     for (int k = t; k < nrec; k += kThreads) {
         const long long v = __double2ll_rn(src[k * st] * up);
         if (v < lo) lo = v;
@@ -378,9 +380,11 @@ __constant__ long long kAsinSq[12] = {
 };
 __constant__ int kAsinSq32[7] = {1058753029, 642436037, 387510425, 203554602, 123855014, 139058146, 85944151};
 
+// LG lags per warp; block z of gridDim.z takes every gridDim.z-th tile and
+// leaves its sums in part (one block: the average in out)
+template <int LG>
 __global__ void __launch_bounds__(32 * kWarps) k_msd_angle(const double *fq, const double *work, const int *bad,
-                                                         int nrec, int max_lag, double *out) {
-    constexpr int LG = 4;                                 // lags per warp
+                                                         int nrec, int max_lag, double *part, double *out) {
     const int b = blockIdx.y;
     if (bad[b]) return;
     const Limbs *x = fix_column(fq, work, b, 9, nrec);
@@ -422,7 +426,7 @@ __global__ void __launch_bounds__(32 * kWarps) k_msd_angle(const double *fq, con
         }
     };
     int tiles = 0;
-    for (int t0 = 0; t0 + lb0 < nrec; t0 += kTile) {
+    for (int t0 = blockIdx.z * kTile; t0 + lb0 < nrec; t0 += gridDim.z * kTile) {
         for (int c = 0; c < 3; ++c) {
             const Limbs *xc = x + (long long)c * nrec;
             for (int i = threadIdx.x; i < kTile; i += 32 * kWarps) s0[c][i] = t0 + i < nrec ? xc[t0 + i] : Limbs{0, 0};
@@ -436,7 +440,8 @@ __global__ void __launch_bounds__(32 * kWarps) k_msd_angle(const double *fq, con
             long long A0[LG], A1[LG], A2[LG];
 #pragma unroll
             for (int q = 0; q < LG; ++q) A0[q] = A1[q] = A2[q] = 0;
-            for (int i = 0; i < kRun; ++i) {
+            const int run = min(kRun, nrec - t0 - l0);        // of lane 0, which has the most pairs
+            for (int i = 0; i < run; ++i) {
                 const Limbs a[3] = {s0[0][at0 + i], s0[1][at0 + i], s0[2][at0 + i]};
 #pragma unroll
                 for (int q = 0; q < LG; ++q) {
@@ -523,8 +528,11 @@ __global__ void __launch_bounds__(32 * kWarps) k_msd_angle(const double *fq, con
     if (l0 > max_lag) return;
     take();
     const int l = l0 + lane;
-    if (lane < LG && l <= max_lag)
-        out[((long long)b * max_lag + (l - 1)) * LB_MSD_COLS + 6] = total / (double)(nrec - l);
+    if (lane < LG && l <= max_lag) {
+        const long long at = (long long)b * max_lag + (l - 1);
+        if (gridDim.z > 1) part[(long long)blockIdx.z * gridDim.y * max_lag + at] = total;
+        else out[at * LB_MSD_COLS + 6] = total / (double)(nrec - l);
+    }
 }
 
 // X's averages that a column's grid is too coarse for, again in FP64. The grid
@@ -537,11 +545,20 @@ __global__ void __launch_bounds__(32 * kWarps) k_msd_angle(const double *fq, con
 // columns are running sums, whose own rounding in such a trajectory is larger
 // than the grid.) Nothing to do where the integers are exact, as they are for
 // values away from 0 by more than 1/8 of their range.
+// Before that, the angle's average from the sums of `parts` blocks (parts > 1).
 __global__ void __launch_bounds__(kThreads) k_msd_near(const double *X, int nrec, int max_lag, const int *unit,
-                                                     const int *bad, double *out) {
+                                                     const int *bad, const double *part, int parts, double *out) {
     const int b = blockIdx.y;
     const int *span = unit + b * kFixCols + 9;
-    if (bad[b] || (span[0] == kExact && span[1] == kExact && span[2] == kExact)) return;
+    if (bad[b]) return;
+    if (parts > 1)
+        for (int l = 1 + blockIdx.x + gridDim.x * threadIdx.x; l <= max_lag; l += gridDim.x * kThreads) {
+            const long long at = (long long)b * max_lag + (l - 1);
+            double v = 0.0;
+            for (int z = 0; z < parts; ++z) v += part[(long long)z * gridDim.y * max_lag + at];
+            out[at * LB_MSD_COLS + 6] = v / (double)(nrec - l);
+        }
+    if (span[0] == kExact && span[1] == kExact && span[2] == kExact) return;
     const double *Xb = X + (long long)b * nrec * 3;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     __shared__ double red[3][kThreads / 32];
@@ -623,8 +640,25 @@ __global__ void __launch_bounds__(kThreads) k_msd_lags(const double *X, int nrec
 
 }  // namespace
 
+// k_msd_angle: four lags a warp (32 a block) and one block per body and lags
+// when these fill the SMs twice; else one lag a warp and the tiles split over
+// blocks until they do, so that few bodies or few lags are not a few blocks'
+// serial work (one body: calls of 4000 records x 80 lags 716 -> 320 us, 606 in
+// FP64; 500 x 10 305 -> 270, 271; 16 bodies 4000 x 400 1135 -> 932, 4426)
+static int angle_parts(int nrec, int nbodies, int max_lag, bool &wide) {
+    const long long want = 2LL * sm_count(), nb = nbodies;
+    wide = nb * ((max_lag + 4 * kWarps - 1) / (4 * kWarps)) >= want;
+    const long long blocks = nb * ((max_lag + kWarps - 1) / kWarps);
+    const long long tiles = (nrec - 2) / kTile + 1;
+    return wide ? 1 : (int)std::max(1LL, std::min(tiles, want / blocks));
+}
+
+// the sums that angle_parts' blocks leave: parts x 8 lags x blocks at most
+static size_t part_doubles() { return 2 * (size_t)sm_count() * kWarps; }
+
 size_t msd_work_bytes(int nrec, int nbodies) {
-    return (size_t)nrec * nbodies * kW * sizeof(double) + (size_t)nbodies * (kFixCols + 1) * sizeof(int);
+    return ((size_t)nrec * nbodies * kW + part_doubles()) * sizeof(double) +
+           (size_t)nbodies * (kFixCols + 1) * sizeof(int);
 }
 
 cudaError_t launch_msd(const double *X, double *q, int nrec, int nbodies, int max_lag, const double *p_ref,
@@ -632,7 +666,8 @@ cudaError_t launch_msd(const double *X, double *q, int nrec, int nbodies, int ma
     const size_t n = (size_t)nrec * nbodies;
     const unsigned nb = (unsigned)nbodies;
     double *w = static_cast<double *>(work);
-    int *unit = reinterpret_cast<int *>(w + n * kW), *bad = unit + (size_t)nbodies * kFixCols;
+    double *part = w + n * kW;
+    int *unit = reinterpret_cast<int *>(part + part_doubles()), *bad = unit + (size_t)nbodies * kFixCols;
     cudaError_t e = cudaMemsetAsync(bad, 0, sizeof(int) * nbodies, s);
     if (e != cudaSuccess) return e;
     k_msd_prep<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(X, q, nrec, nbodies, p_ref, w);
@@ -641,10 +676,14 @@ cudaError_t launch_msd(const double *X, double *q, int nrec, int nbodies, int ma
     k_msd_fix<<<dim3(10, nb), kThreads, 0, s>>>(X, q, w, nrec, unit, bad);
     const unsigned gd = (unsigned)((max_lag + kLags * kWarps - 1) / (kLags * kWarps));
     k_msd_disp<<<dim3(gd, 9, nb), 32 * kWarps, 0, s>>>(q, w, unit, bad, nrec, max_lag, out);
-    const unsigned ga = (unsigned)((max_lag + 4 * kWarps - 1) / (4 * kWarps));
-    k_msd_angle<<<dim3(ga, nb), 32 * kWarps, 0, s>>>(q, w, bad, nrec, max_lag, out);
+    bool wide = false;
+    const int parts = angle_parts(nrec, nbodies, max_lag, wide);
+    const unsigned lags = wide ? 4 * kWarps : kWarps;
+    const dim3 ga((max_lag + lags - 1) / lags, nb, (unsigned)parts);
+    if (wide) k_msd_angle<4><<<ga, 32 * kWarps, 0, s>>>(q, w, bad, nrec, max_lag, part, out);
+    else k_msd_angle<1><<<ga, 32 * kWarps, 0, s>>>(q, w, bad, nrec, max_lag, part, out);
     const dim3 gl((unsigned)std::min(max_lag, std::max(8, 2048 / nbodies)), nb);
-    k_msd_near<<<gl, kThreads, 0, s>>>(X, nrec, max_lag, unit, bad, out);
+    k_msd_near<<<gl, kThreads, 0, s>>>(X, nrec, max_lag, unit, bad, part, parts, out);
     k_msd_lags<<<gl, kThreads, 0, s>>>(X, nrec, max_lag, w, bad, out);
     return cudaGetLastError();
 }

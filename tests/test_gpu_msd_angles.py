@@ -112,3 +112,28 @@ def test_quaternions_that_leave_no_unit_vector(qb):
     got = _squared_angles((1, 0, 0, 0), qb)
     assert np.abs(got[0::2] - th ** 2).max() <= TOL
     assert np.abs(got[1::2]).max() <= TOL
+
+
+@pytest.mark.parametrize("nb,nrec,lags", [(1, 481, 1), (1, 482, 9), (1, 4000, 5), (1, 4400, 400), (3, 1700, 33), (2, 3900, 3899), (40, 600, 64), (20, 4000, 20)])
+def test_few_bodies_and_lags(nb, nrec, lags):
+    """Tiles split over blocks, one or four lags a warp: small and large angles
+    together, against FP64's own evaluation. Its arctangents and unit vectors are
+    good to 4e-16 + 2^-52 relative, sums of n terms to (log2 n + 8) 2^-52."""
+    from paper_1604_01829_gb300 import lb
+    rng = np.random.default_rng(nrec + lags)
+    q = np.zeros((nb, nrec, 4))
+    q[..., 0] = 1.0
+    q[:, 1:, 1:] = np.cumsum(0.3 * rng.standard_normal((nb, nrec - 1, 3)), axis=1)
+    q /= np.linalg.norm(q, axis=2, keepdims=True)
+    got = lb.lb_msd_trajectory(np.zeros((nb, nrec, 3)), q, lags, p_ref=(0, 0, 1))[:, :, 6]
+    w, x, y, z = np.moveaxis(q, 2, 0)
+    p = np.stack([2 * (x * z + y * w), 2 * (y * z - x * w), 1 - 2 * (x * x + y * y)], axis=2)
+    for l in {1, 2, lags // 2 + 1, max(1, lags - 1), lags}:
+        if l > lags:
+            continue
+        a, b = p[:, :-l], p[:, l:]
+        th = np.arctan2(np.linalg.norm(np.cross(a, b), axis=2), (a * b).sum(2))
+        n = nrec - l
+        ref = (th * th).mean(axis=1)
+        bound = 2 * th.mean(axis=1) * 4e-16 + (np.log2(n) + 10) * 2.0 ** -52 * ref
+        assert np.all(np.abs(got[:, l - 1] - ref) <= bound + 4 * np.finfo(float).eps ** 2)
