@@ -494,6 +494,7 @@ struct lb_batch_ctx {
     std::vector<long long> flag_start;      // n + 1
     std::vector<long long> nfluid;
     long long Ntot = 0, Ttot = 0, Ftot = 0;  // padded plane strides summed (pool sizes)
+    long long Npop = 0;                      // those in use: pores hold fluid nodes only
     long long Nnodes = 0;                    // nodes of all instances
     void *pool = nullptr;
     void *Fbuf[2] = {nullptr, nullptr};     // force pools, storage precision
@@ -664,9 +665,11 @@ void compute_g(const lb_batch_ctx *h, int k, double g[3]) {
 lb_status rebuild_schedule(lb_batch_ctx *h) {
     std::vector<int> ts(h->n + 1, 0);
     long long acc = 0;
+    h->Npop = 0;
     for (int k = 0; k < h->n; ++k) {
         ts[k] = (int)acc;
         acc += ((long long)h->hinst[k].nwork + h->TS - 1) / h->TS;
+        h->Npop += h->hinst[k].ps;
     }
     ts[h->n] = (int)acc;
     if (acc > 2000000000LL) return bfail(h, LB_ERR_ARG, "too many work tiles");
@@ -999,7 +1002,9 @@ lb_status launch_step(lb_batch_ctx *h, int k, bool finish_prev, bool record, boo
     if (grid < 1) grid = 1;
     a.order = h->order == 1 ? 1 : 0;
     a.chunk = (h->ntiles + grid - 1) / grid;
-    a.ahead = h->fp32 && 19 * h->Ntot * 4 >= LB_AHEAD_BYTES ? (h->order == 1 ? LB_BATCH_AHEAD : LB_BATCH_AHEAD * h->sms * std::min(h->bpsm, res > 0 ? res : h->bpsm)) : 0;
+    a.ahead = 0;
+    if (h->fp32 && 19 * h->Npop * 4 >= LB_AHEAD_BYTES)
+        a.ahead = LB_BATCH_AHEAD * (h->order == 1 ? 1 : h->sms * std::min(h->bpsm, res > 0 ? res : h->bpsm));
     a.pool = h->pool;
     a.fluid = h->dfluid;
     a.F = coupled ? h->Fbuf[cur] : nullptr;
