@@ -599,6 +599,7 @@ struct Snapshot {
     int *tiles[2] = {nullptr, nullptr};
     int *tlist[2] = {nullptr, nullptr};   // list entries, then the count
     Body *bodies = nullptr;
+    double *Fbead = nullptr;              // bead forces of the last step (read by lb_forces)
     unsigned long long *dstep = nullptr;
     long long step = 0;
 };
@@ -643,18 +644,19 @@ void adj_free(lb_ctx *h) {
 namespace {
 
 struct Sizes {
-    size_t fbytes, Fbytes, tbytes, lbytes, bbytes;
+    size_t fbytes, Fbytes, tbytes, lbytes, bbytes, dbytes;
 };
 
 Sizes sizes_of(const lb_ctx *h) {
     const size_t es = h->fp32 ? 4 : 8;
     const size_t N = (size_t)h->g.N;
     return Sizes{es * 19 * N, es * 3 * N, sizeof(int) * (size_t)h->ntx * h->nty * h->ntz,
-                 sizeof(int) * (size_t)h->list_cap, sizeof(Body) * h->hb.size()};
+                 sizeof(int) * (size_t)h->list_cap, sizeof(Body) * h->hb.size(), 3 * sizeof(double) * h->hbody_of.size()};
 }
 
 size_t snapshot_bytes(const Sizes &z) {
-    return z.fbytes + 2 * (z.Fbytes + z.tbytes + z.lbytes + sizeof(int)) + z.bbytes + sizeof(unsigned long long);
+    return z.fbytes + 2 * (z.Fbytes + z.tbytes + z.lbytes + sizeof(int)) + z.bbytes + z.dbytes +
+           sizeof(unsigned long long);
 }
 
 size_t tape_bytes(const Sizes &z) { return z.fbytes + z.Fbytes + z.bbytes; }
@@ -712,6 +714,7 @@ lb_status ensure_work(lb_ctx *h, int nsnap, int ntape, int nsteps, double *alloc
             if (e == cudaSuccess) e = walloc(*w, &S.tlist[k], z.lbytes + sizeof(int));
         }
         if (e == cudaSuccess) e = walloc(*w, &S.bodies, z.bbytes);
+        if (e == cudaSuccess) e = walloc(*w, &S.Fbead, z.dbytes);
         if (e == cudaSuccess) e = walloc(*w, &S.dstep, sizeof(unsigned long long));
     }
     for (size_t k = 0; k < w->tape.size(); ++k) {
@@ -804,6 +807,7 @@ struct Run {
             add((char *)S.tlist[k] + z.lbytes, h->tcount[k], sizeof(int));
         }
         add(S.bodies, h->db, z.bbytes);
+        add(S.Fbead, h->dFbead, z.dbytes);
         add(S.dstep, h->step_dev, sizeof(unsigned long long));
         return L;
     }

@@ -265,3 +265,14 @@ def test_handle_reads_as_after_plain_steps(precision, schedule, snapshots):
     g.lb_step(3)
     twin.lb_step(3)
     assert np.abs(g.lb_get_body(0)["X"] - twin.lb_get_body(0)["X"]).max() <= tol * np.abs(b["X"]).max()
+
+
+@pytest.mark.parametrize("schedule,snapshots", [(0, 0), (0, 5), (1, 3)])
+def test_bead_forces_after_the_adjoint(schedule, snapshots):
+    """The forces of the single beads are those of the last step, too."""
+    g, _ = _pair(64, dict(MRT))
+    twin, _ = _pair(64, dict(MRT))
+    g.lb_adjoint_drag_ex(30, 10, body=0, axis=2, schedule=schedule, snapshots=snapshots)
+    twin.lb_step(30)
+    a, b = g.lb_forces(0, per_bead=True)[2], twin.lb_forces(0, per_bead=True)[2]
+    assert np.abs(a - b).max() <= 1e-11 * np.abs(b).max()
