@@ -872,6 +872,7 @@ struct Run {
 
     void mark_first() {
         if (first_sweep && timed) cudaEventRecord(ev_first, s);
+        if (first_sweep) lbk::ctx_pause_recorder(h, true);
         first_sweep = false;
     }
 
@@ -1187,7 +1188,10 @@ extern "C" lb_status lb_adjoint_drag_ex(lb_handle h, int nsteps, int window, int
     // not those of the state it leaves
     struct Stale {
         lb_ctx *h;
-        ~Stale() { h->out_fresh = false; }
+        ~Stale() {
+            h->out_fresh = false;
+            lbk::ctx_pause_recorder(h, false);
+        }
     } stale{h};
 
     int nsnap, ntape, c = 0, S = 0;

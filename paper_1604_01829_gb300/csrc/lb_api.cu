@@ -327,6 +327,15 @@ lb_status ctx_apply_external(lb_ctx *h) {
     if (s != LB_OK) return s;
     return push_bodies(h);
 }
+// the trajectory recorder off while steps are re-run, and on again: their
+// records are in the ring already, and older ones would take the newest's places
+void ctx_pause_recorder(lb_ctx *h, bool pause) {
+    double *&from = pause ? h->rec : h->rec_paused, *&to = pause ? h->rec_paused : h->rec;
+    if (!from) return;
+    to = from;
+    from = nullptr;
+    drop_graph(h);
+}
 lb_status ctx_fail(lb_ctx *h, lb_status s, const std::string &m) { return fail(h, s, m); }
 }  // namespace lbk
 

@@ -79,6 +79,7 @@ struct lb_ctx {
     // trajectory recorder: ring [rec_cap][nbodies][7] (X, q), one record
     // every rec_every steps; records k >= rec_k0 (k = step / rec_every)
     double *rec = nullptr;
+    double *rec_paused = nullptr;           // the ring while an adjoint re-runs steps (ctx_pause_recorder)
     int rec_every = 0, rec_cap = 0;
     long long rec_k0 = 0;
     // timing
@@ -107,5 +108,6 @@ lb_status ctx_fail(lb_ctx *h, lb_status s, const std::string &m);
 lb_status ctx_turn(lb_ctx *h, const void *src);
 lb_status ctx_step_oop(lb_ctx *h, const void *src, void *dst);
 lb_status ctx_tape_steps(lb_ctx *h, int n, void *const *f, Body *const *bodies, void *const *F, size_t Fbytes);
+void ctx_pause_recorder(lb_ctx *h, bool pause);
 void adj_free(lb_ctx *h);
 }  // namespace lbk

@@ -276,3 +276,23 @@ def test_bead_forces_after_the_adjoint(schedule, snapshots):
     twin.lb_step(30)
     a, b = g.lb_forces(0, per_bead=True)[2], twin.lb_forces(0, per_bead=True)[2]
     assert np.abs(a - b).max() <= 1e-11 * np.abs(b).max()
+
+
+@pytest.mark.parametrize("schedule,snapshots", [(0, 0), (0, 5), (1, 1), (1, 3), (1, 30)])
+@pytest.mark.parametrize("capacity", [8, 64])
+def test_recorded_trajectory_after_the_adjoint(schedule, snapshots, capacity):
+    """The recorder's ring holds the newest records of the steps taken, not those
+    of steps run again, and goes on recording."""
+    g, _ = _pair(64, dict(MRT))
+    twin, _ = _pair(64, dict(MRT))
+    for h in (g, twin):
+        h.lb_record_bodies(1, capacity)
+    g.lb_adjoint_drag_ex(30, 10, body=0, axis=2, schedule=schedule, snapshots=snapshots)
+    twin.lb_step(30)
+    for more in (0, 3):
+        if more:
+            g.lb_step(more)
+            twin.lb_step(more)
+        (sa, Xa, qa), (sb, Xb, qb) = g.lb_get_trajectory(0), twin.lb_get_trajectory(0)
+        assert np.array_equal(sa, sb) and len(sa) == min(capacity, 30 + more)
+        assert np.abs(Xa - Xb).max() <= 1e-12 and np.abs(qa - qb).max() <= 1e-13
