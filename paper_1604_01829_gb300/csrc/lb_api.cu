@@ -235,7 +235,6 @@ lbk::FluidArgs fluid_args(const lb_ctx *h, int cur, uint32_t step_off) {
         a.pf.ks[k] = (float)a.pd.ks[k];
     }
     for (int k = 0; k < 9; ++k) a.pf.kg[k] = (float)a.pd.kg[k];
-    for (int k = 0; k < 15; ++k) a.pf.kn[k] = (float)(a.pd.kn[k] * 2.3283064365386963e-10);
     a.gforce = h->gforce;
     a.gforce_f = h->gforce_f;
     const bool bodies = !h->hb.empty() && !h->hbody_of.empty();

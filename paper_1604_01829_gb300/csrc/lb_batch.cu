@@ -632,7 +632,6 @@ void fill_coll(const lb_params &p, BInst &I) {
         I.pf.ks[k] = (float)I.pd.ks[k];
     }
     for (int k = 0; k < 9; ++k) I.pf.kg[k] = (float)I.pd.kg[k];
-    for (int k = 0; k < 15; ++k) I.pf.kn[k] = (float)(I.pd.kn[k] * 2.3283064365386963e-10);
 }
 
 lb_status validate(const lb_params &p) {

@@ -300,14 +300,14 @@ __device__ __forceinline__ void collide_mrt_f32(float (&f)[19], float Fx, float 
     f[16] = a16.x; f[18] = a16.y;
 }
 
-// Collision of one FP32 node: MRT in pairs (PAIRS, and always with noise), or
-// as it stands.
 // Fetches [p, p + bytes) into L2, without waiting (16-byte aligned, a multiple
 // of 16 bytes).
 __device__ __forceinline__ void fetch_l2(const void *p, uint32_t bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "r"(bytes) : "memory");
 }
 
+// Collision of one FP32 node: MRT in pairs (PAIRS, and always with noise), or
+// as it stands.
 template <int COLL, bool NOISE, bool PAIRS>
 __device__ __forceinline__ void collide_f32(float (&f)[19], float Fx, float Fy, float Fz, const CollParams<float> &pf,
                                             const CollPairs &pk, uint2 key, uint32_t instance, uint32_t node,

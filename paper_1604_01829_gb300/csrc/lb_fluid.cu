@@ -24,12 +24,15 @@
 #include "lb_fix64.cuh"
 #include "lb_rigid.cuh"
 
-// Minimum resident blocks of 128 threads per SM requested for the FP32
-// collide kernels (caps their registers; FP64 kernels are not capped):
-// 8 blocks (64 registers) without noise, 7 (72 registers) with it, where the
-// Philox state needs the room (measured on GB300 at 256^3 with noise: 0.439 ms
-// per launch at 7 blocks, 0.452 at 8, 0.458 at 6, 0.488 at 5; without noise
-// 0.415 ms at 8, 0.419 at 7).
+// Minimum resident blocks of 128 threads per SM requested for the collide
+// kernels (caps their registers). FP32: 8 blocks (64 registers) without noise,
+// 7 (72 registers) with it, where the Philox state needs the room, and for BGK
+// where it fetches ahead; FP64: 4 (128). Measured on GB300, us per launch: 256^3
+// with noise 392 / 378 / 386 at 6 / 7 / 8 blocks, BGK 374 / 378 / 417; MRT
+// without noise 376 / 382 / 387 at 7 / 8 / 9, but with bodies held in it 150 x
+// 97 x 203 steps in 93.2 us at 7 and 90.1 at 8 (76.5 / 77.3 / 78.9 without
+// them); FP64 at 3 / 4 / 5, 94 x 81 x 103 with noise 74.7 / 76.6 / 83.2, 48^3
+// 16.0 / 15.5 / 16.4.
 #ifndef LB_CS_MINB
 #define LB_CS_MINB 8
 #endif

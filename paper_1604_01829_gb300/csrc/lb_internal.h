@@ -21,8 +21,8 @@ struct CollParams {
     R km[6];                     // c_k g_k: weight of the pre-collision moment
     R ks[6];                     // c_k (1 + g_k)/2: weight of the Guo source moment
     R kg[9];                     // ghost modes 10-18: c_k g_k
-    R kn[15];                    // noise modes 4-18: c_k sqrt(3 kT b_k (1 - g_k^2)) sqrt(12) / sqrt(rho),
-                                 //   applied to a centred uniform variate in (-1/2, 1/2) (FP32: times 2^-32)
+    R kn[15];                    // FP64: noise modes 4-18, c_k sqrt(3 kT b_k (1 - g_k^2)) sqrt(12) / sqrt(rho),
+                                 //   applied to a centred uniform variate in (-1/2, 1/2) (FP32: CollPairs)
 };
 
 // The MRT constants of the FP32 collision, paired as its two-wide arithmetic
@@ -38,7 +38,7 @@ struct alignas(8) CollPairs {
 inline CollPairs coll_pairs(const CollParams<double> &d) {
     CollPairs p{};
     auto two = [](double a, double b) { return make_float2((float)a, (float)b); };
-    const double n = 2.3283064365386963e-10;       // 2^-32 (CollParams::kn in FP32)
+    const double n = 2.3283064365386963e-10;       // 2^-32: the variates come times 2^32
     p.ke56 = two(d.ke[1], d.ke[2]); p.km56 = two(d.km[1], d.km[2]); p.ks56 = two(2 * d.ks[1], 2 * d.ks[2]);
     p.ke79 = two(d.ke[3], d.ke[5]); p.km79 = two(d.km[3], d.km[5]); p.ks79 = two(d.ks[3], d.ks[5]);
     p.kg1112 = two(d.kg[1], d.kg[2]); p.kg1415 = two(d.kg[4], d.kg[5]); p.kg1718 = two(d.kg[7], d.kg[8]);
@@ -124,13 +124,13 @@ struct StepExtra {
     unsigned by;
 };
 
-// Everything the fused collide-and-stream kernel reads besides populations.
 // bytes of populations from which the FP32 fluid kernels fetch ahead into L2:
 // below, the lattice (or batch) stays in its 129 MB from step to step
 #ifndef LB_AHEAD_BYTES
 #define LB_AHEAD_BYTES (100LL << 20)
 #endif
 
+// Everything the fused collide-and-stream kernel reads besides populations.
 struct FluidArgs {
     Geom g;
     void *f;                     // populations: double[19][N] (FP64) or float[19][N] deviations
