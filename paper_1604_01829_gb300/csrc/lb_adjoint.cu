@@ -787,8 +787,9 @@ struct Run {
     const void *pops() const { return cf ? cf : h->f; }
 
     // The state's parts as copy segments between a snapshot and the handle
-    // (to_snapshot: handle -> snapshot); the populations when with_f.
-    lbk::CopyList parts(const Snapshot &S, bool to_snapshot, bool with_f, const void *f_src) {
+    // (to_snapshot: handle -> snapshot); the populations when with_f, the bead
+    // forces (which no step reads) of the state that the handle is left with.
+    lbk::CopyList parts(const Snapshot &S, bool to_snapshot, bool with_f, const void *f_src, bool last) {
         lbk::CopyList L{};
         auto add = [&](void *snap, const void *hnd, size_t bytes) {
             lbk::CopySeg &c = L.seg[L.n++];
@@ -807,7 +808,7 @@ struct Run {
             add((char *)S.tlist[k] + z.lbytes, h->tcount[k], sizeof(int));
         }
         add(S.bodies, h->db, z.bbytes);
-        add(S.Fbead, h->dFbead, z.dbytes);
+        if (last) add(S.Fbead, h->dFbead, z.dbytes);
         add(S.dstep, h->step_dev, sizeof(unsigned long long));
         return L;
     }
@@ -822,9 +823,9 @@ struct Run {
 
     // One launch for the whole state (the populations only if they are not
     // already the snapshot's).
-    cudaError_t save(Snapshot &S) {
+    cudaError_t save(Snapshot &S, bool last = false) {
         S.step = h->step;
-        return copy(parts(S, true, pops() != S.f, pops()));
+        return copy(parts(S, true, pops() != S.f, pops(), last));
     }
     // Everything but the populations, which stay in the snapshot for the next
     // step or turn to read; whole: the populations too (the handle is left
@@ -832,7 +833,7 @@ struct Run {
     cudaError_t restore(const Snapshot &S, bool whole = false) {
         cf = whole ? nullptr : S.f;
         h->step = S.step;
-        return copy(parts(S, false, whole, nullptr));
+        return copy(parts(S, false, whole, nullptr, whole));
     }
 
     // Steps the handle from relative step a to b (its state is a), recording
@@ -976,7 +977,7 @@ lb_status run_two_level(Run &R, int c) {
         lb_status st = R.advance(a0, a1);
         if (st != LB_OK) return st;
     }
-    cudaError_t e = R.save(w->snaps[nseg]);
+    cudaError_t e = R.save(w->snaps[nseg], true);
     if (e != cudaSuccess) return R.fail_cuda(e, "snapshot");
     R.mark_first();
     // The re-run of steps [a0, a1) from the state in tape entry 0: each step
@@ -1088,7 +1089,7 @@ struct Binomial {
         if (st != LB_OK) return st;
         if (!final_saved) {
             if ((st = R.advance(a, a + 1)) != LB_OK) return st;
-            cudaError_t e = R.save(R.w->snaps[fin]);
+            cudaError_t e = R.save(R.w->snaps[fin], true);
             if (e != cudaSuccess) return R.fail_cuda(e, "snapshot");
             final_saved = true;
             R.mark_first();
@@ -1115,7 +1116,7 @@ struct Binomial {
                 // state n is held but has no slot: the final state needs it whole first
                 if (!final_saved) {
                     if ((st = R.advance(n, n + 1)) != LB_OK) return st;
-                    cudaError_t e = R.save(R.w->snaps[fin]);
+                    cudaError_t e = R.save(R.w->snaps[fin], true);
                     if (e != cudaSuccess) return R.fail_cuda(e, "snapshot");
                     final_saved = true;
                     R.mark_first();

@@ -524,18 +524,15 @@ size_t list_smem(size_t rsize, int max_count) {
     return 6 * rsize * (size_t)max_count + sizeof(uint16_t) * kListLen * (size_t)max_count;
 }
 
-// surface area by Thomsen's formula (within 1.1 %)
-double ellipsoid_area(const double *a) {
-    const double p = 1.6075, x = std::pow(a[0] * a[1], p) + std::pow(a[0] * a[2], p) + std::pow(a[1] * a[2], p);
-    return 4.0 * 3.141592653589793 * std::pow(x / 3.0, 1.0 / p);
-}
-
 // The longest list to keep for a shell of n beads: a spherical cap of chord
 // radius rl has the area pi rl^2, so n pi rl^2 / area beads lie within rl of an
-// evenly spread bead; half as many again, and a few, for uneven spreads. A
-// value of this shell alone: shells relaxed together are relaxed as each alone.
-int list_rows(const double *axes, int n, double sigma) {
-    const double rl = (kWcaCut + LB_LIST_SKIN) * sigma, near = n * 3.141592653589793 * rl * rl / ellipsoid_area(axes);
+// evenly spread bead, with 4 pi / 3 (ab + ac + bc) for the area (a sphere's; up
+// to 15 % too small for a long ellipsoid); half as many again, and a few, for
+// uneven spreads. A value of this shell alone: shells relaxed together are
+// relaxed as each alone.
+int list_rows(const double *a, int n, double sigma) {
+    const double rl = (kWcaCut + LB_LIST_SKIN) * sigma;
+    const double near = 0.75 * n * rl * rl / (a[0] * a[1] + a[0] * a[2] + a[1] * a[2]);
     if (n <= kListLen || !(near > kCrowded)) return kListLen;
     return (int)std::min((n + 3.0) / 4.0, 0.375 * near + 5.0) * 4;
 }

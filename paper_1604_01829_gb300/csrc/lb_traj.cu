@@ -473,14 +473,14 @@ __global__ void __launch_bounds__(32 * kWarps) k_msd_angle(const double *fq, con
                             t2 += (long long)e1 * e1;
                         }
                         z = t2 + ((t1 + (t0 >> 30) + (1LL << 27)) >> 28);
+                        if (z >= (1LL << 55)) z = (1LL << 55) - 1;           // a right angle: u stays below 1/2
                     }
-                    z = max(0LL, min(z, 1LL << 55));             // 2 may be passed by a rounding error
-                    // k by Horner's rule in u = z/2 - 1/2, |u| <= 1/2 (both ends are
-                    // reached: z = 0 and a right angle): the inner seven steps (below
-                    // 2^-14, and times u^12 at the end) in 32 bits
+                    if (z < 0) z = 0;
+                    // k by Horner's rule in u = z/2 - 1/2, -1/2 <= u < 1/2: the inner seven
+                    // steps (below 2^-14, and times u^12 at the end) in 32 bits
                     const long long half = z << 7;                           // z/2 at 2^62
-                    const long long u = (half - (1LL << 61)) << 1;           // at 2^63
-                    const int u32 = (int)min(u >> 31, 0x7FFFFFFFLL);         // at 2^32
+                    const long long u = (z << 8) - (1LL << 62);              // at 2^63
+                    const int u32 = (int)(u >> 31);                          // at 2^32
                     int ki = kAsinSq32[6];
 #pragma unroll
                     for (int j = 5; j >= 0; --j) ki = kAsinSq32[j] + __mulhi(ki, u32);
