@@ -61,11 +61,18 @@ struct ShellArgs {
     int max_cells;            // largest grid (shared-memory extent)
     int *err;                 // index checks of checked builds (LB_CHECKS): bit 2 on failure
     R rl2, move2;             // neighbour lists: (range + skin)^2 and the squared move that outdates them
-    // lists of crowded shells in device memory: [nshells][list_rows][max_count],
-    // the longest list of each shell
-    uint16_t *glist;
-    const int *list_len;
-    int list_rows;
+};
+
+// Lists of crowded shells in device memory: [nshells][rows][max_count], and the
+// longest list of each shell. Not among ShellArgs: the kernels without them keep
+// their arguments' places (a small shell's step 1.61 -> 1.70 us otherwise).
+template <bool LONG>
+struct LongLists {};
+template <>
+struct LongLists<true> {
+    uint16_t *list;
+    const int *len;
+    int rows;
 };
 
 __device__ __forceinline__ float rdiv(float a, float b) { return __fdividef(a, b); }
@@ -393,15 +400,17 @@ template <typename R>
 constexpr int list_threads() { return sizeof(R) == 8 ? 512 : 1024; }
 
 template <typename R, int BPT, bool LONG>
-__global__ void __launch_bounds__(list_threads<R>()) k_relax_list(const ShellArgs<R> a) {
+__global__ void __launch_bounds__(list_threads<R>()) k_relax_list(const ShellArgs<R> a, const LongLists<LONG> ll) {
     extern __shared__ unsigned char smem_raw[];
     R *pos = reinterpret_cast<R *>(smem_raw);                          // [2][3][max_count]
     const int M = a.max_count;
     const int s = blockIdx.x;
-    uint16_t *list;                                                    // [cap][max_count]
-    if constexpr (LONG) list = a.glist + (size_t)s * a.list_rows * M;
-    else list = reinterpret_cast<uint16_t *>(pos + 6 * (size_t)M);
-    const int cap = LONG ? a.list_len[s] : kListLen;
+    uint16_t *list = reinterpret_cast<uint16_t *>(pos + 6 * (size_t)M);   // [cap][max_count]
+    int cap = kListLen;
+    if constexpr (LONG) {
+        list = ll.list + (size_t)s * ll.rows * M;
+        cap = ll.len[s];
+    }
     const int n = a.count[s];
     double *X = a.xyz + 3 * a.offset[s];
     const R ax = (R)a.axes[3 * s], ay = (R)a.axes[3 * s + 1], az = (R)a.axes[3 * s + 2];
@@ -538,20 +547,21 @@ int list_rows(const double *a, int n, double sigma) {
 }
 
 template <typename R, int BPT, bool LONG>
-cudaError_t launch_list_t(const ShellArgs<R> &a, int nshells, int threads, cudaStream_t s) {
+cudaError_t launch_list_t(const ShellArgs<R> &a, const LongLists<LONG> &ll, int nshells, int threads, cudaStream_t s) {
     const size_t smem = LONG ? 6 * sizeof(R) * (size_t)a.max_count : list_smem(sizeof(R), a.max_count);
     cudaError_t e = cudaFuncSetAttribute(k_relax_list<R, BPT, LONG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
-    k_relax_list<R, BPT, LONG><<<nshells, threads, smem, s>>>(a);
+    k_relax_list<R, BPT, LONG><<<nshells, threads, smem, s>>>(a, ll);
     return cudaGetLastError();
 }
 
 template <typename R, bool LONG>
-cudaError_t launch_list(const ShellArgs<R> &a, int bpt, int nshells, int threads, cudaStream_t s) {
-    if (bpt == 1) return launch_list_t<R, 1, LONG>(a, nshells, threads, s);
-    if (bpt == 2) return launch_list_t<R, 2, LONG>(a, nshells, threads, s);
-    return launch_list_t<R, 4, LONG>(a, nshells, threads, s);
+cudaError_t launch_list(const ShellArgs<R> &a, const LongLists<LONG> &ll, int bpt, int nshells, int threads,
+                        cudaStream_t s) {
+    if (bpt == 1) return launch_list_t<R, 1, LONG>(a, ll, nshells, threads, s);
+    if (bpt == 2) return launch_list_t<R, 2, LONG>(a, ll, nshells, threads, s);
+    return launch_list_t<R, 4, LONG>(a, ll, nshells, threads, s);
 }
 
 size_t shell_smem(size_t rsize, int max_count, int max_cells, bool cells) {
@@ -570,7 +580,7 @@ cudaError_t launch_shells_t(const ShellArgs<R> &a, int nshells, int threads, cud
 
 template <typename R>
 cudaError_t launch_shells(ShellArgs<R> a, const lb_shell_params &p, int nshells, bool cells, bool lists,
-                          cudaStream_t s) {
+                          const LongLists<true> &ll, cudaStream_t s) {
     a.k2 = (R)(2.0 * p.k_surface);
     a.sig2 = (R)(p.sigma * p.sigma);
     a.rc2 = (R)(kWcaCut * kWcaCut * p.sigma * p.sigma);
@@ -592,7 +602,8 @@ cudaError_t launch_shells(ShellArgs<R> a, const lb_shell_params &p, int nshells,
         const double skin = LB_LIST_SKIN * p.sigma, rl = kWcaCut * p.sigma + skin;
         a.rl2 = (R)(rl * rl);
         a.move2 = (R)(0.98 * 0.25 * skin * skin);
-        return a.glist ? launch_list<R, true>(a, bpt, nshells, threads, s) : launch_list<R, false>(a, bpt, nshells, threads, s);
+        if (ll.list) return launch_list<R, true>(a, ll, bpt, nshells, threads, s);
+        return launch_list<R, false>(a, {}, bpt, nshells, threads, s);
     }
     if (cells) {
         if (bpt == 1) return launch_shells_t<R, 1, true>(a, nshells, threads, s);
@@ -728,14 +739,12 @@ extern "C" lb_status lb_relax_shells(int nshells, const double *axes, const int 
             lbk::ShellArgs<double> a{};
             a.axes = daxes; a.count = dcount; a.offset = doff; a.xyz = dxyz; a.max_count = max_count;
             a.cgrid = dgrid; a.cbox = dbox; a.max_cells = cells ? max_cells : 1; a.err = derr;
-            a.glist = dlong; a.list_len = drows; a.list_rows = max_rows;
-            e = lbk::launch_shells<double>(a, *p, nshells, cells, lists, st);
+            e = lbk::launch_shells<double>(a, *p, nshells, cells, lists, {dlong, drows, max_rows}, st);
         } else {
             lbk::ShellArgs<float> a{};
             a.axes = daxes; a.count = dcount; a.offset = doff; a.xyz = dxyz; a.max_count = max_count;
             a.cgrid = dgrid; a.cbox = dbox; a.max_cells = cells ? max_cells : 1; a.err = derr;
-            a.glist = dlong; a.list_len = drows; a.list_rows = max_rows;
-            e = lbk::launch_shells<float>(a, *p, nshells, cells, lists, st);
+            e = lbk::launch_shells<float>(a, *p, nshells, cells, lists, {dlong, drows, max_rows}, st);
         }
     }
     int herr = 0;
