@@ -8,10 +8,17 @@
 // pipes: populations become 64-bit integers at 2^-61 of a power of two near
 // rho0, the moments and the way back are exact integer sums, products keep the
 // top 64 of 128 bits with rounding, and only the results are rounded to
-// doubles (to nearest even), so the error per step is below that of the FP64
-// evaluation. The conserved moments are not recomputed: a population changes
-// by the relaxation of the 15 other moments and by its share of the force, so
-// mass is exact before the final rounding.
+// doubles (to nearest even). The conserved moments are not recomputed: a
+// population changes by the relaxation of the 15 other moments and by its
+// share of the force, so mass is exact before the final rounding.
+//
+// Error against the same runs in 80-bit arithmetic, this form and the FP64
+// evaluation: populations (rms, in units of rho0) 1.4e-17 and 2.9e-15 after 200
+// steps of a pulled sphere in 32^3, 1.4e-17 and 1.4e-15 after 100 in a driven
+// 48 x 48 x 96 pore, 1.5e-17 and 6e-16 after 50 with noise; momentum of a pore
+// driven by 1e-6 for 2000 steps 5e-14 and 1.2e-12 relative, by 1e-8 3e-12 and
+// 9e-11 (the share of the force is rounded to 2^-61, for a node always the same
+// way; FP64 rounds the sums that it is added to at 2^-58).
 //
 // Range: with rho0 scaled into [2/3, 4/3) the inputs must satisfy
 // |f_0| < 1/2, |f_1..6| < 1/8, |f_7..18| < 1/16 (about twice the values at

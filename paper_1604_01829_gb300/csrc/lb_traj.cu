@@ -122,9 +122,9 @@ __global__ void __launch_bounds__(kThreads) k_msd_scan(int nrec, double *work) {
 // ms for 64 bodies x 4000 records x 400 lags. As 57-bit integers the
 // differences are exact, the squares are three 32-bit products summed in 64
 // and then 128 bits, and the squared angle is a power series: integer work at
-// 64 times the rate. Measured for that case: 0.54 ms (k_msd_disp, 12 warp
-// instructions per 32 pairs and column) and 1.69 ms (k_msd_angle, bound by
-// its ~330, the polynomial mostly), the whole call 15.8 -> 2.85 ms.
+// 64 times the rate. Measured for that case: 0.55 ms (k_msd_disp, 9 warp
+// instructions per 32 pairs and column) and 1.70 ms (k_msd_angle, bound by
+// its ~350, the polynomial mostly), the whole call 15.8 -> 2.87 ms.
 // The integer columns take the place of what they come from: X's three that of
 // the quaternions (read last by k_msd_prep), the others that of the work
 // columns, so the analysis needs no more memory than in FP64.
