@@ -385,8 +385,8 @@ __global__ void __maxnreg__(sizeof(T) == 4 ? LB_BATCH_COUPLE_REGS : 255) k_batch
     a.step_base = b.step_base;
     a.step_off = b.step_off;
     couple_bead<T>(a, k, active ? b.bead_rng[k] : 0, t & 7, threadIdx.x & 31, active);
-    if (b.any_wall && active && (t & 7) == 1 && I.wall.on)
-        couple_wall(I.wall, b.bodies, chk(b.bead_body[k], b.nbodies, b.err), b.s, k);
+    if (b.any_wall && active && I.wall.on)
+        couple_wall(I.wall, b.bodies, chk(b.bead_body[k], b.nbodies, b.err), b.s, k, t & 7);
 }
 
 // previous step's second half kick (optional), this step's kick and drift,

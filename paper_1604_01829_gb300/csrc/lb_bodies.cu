@@ -75,8 +75,8 @@ __global__ void __launch_bounds__(128) __maxnreg__(sizeof(T) == 4 ? LB_COUPLE_RE
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int k = t >> 3;
     couple_bead<T>(a, k, k, t & 7, threadIdx.x & 31, k < a.nbeads);
-    if (a.wall.on && k < a.nbeads && (t & 7) == 1) 
-        couple_wall(a.wall, a.bodies, chk(a.bead_body[k], a.nbodies, a.err), a.s, k);
+    if (a.wall.on && k < a.nbeads)
+        couple_wall(a.wall, a.bodies, chk(a.bead_body[k], a.nbodies, a.err), a.s, k, t & 7);
 }
 
 }  // namespace

@@ -54,9 +54,10 @@ __device__ __forceinline__ void node_rho_j(const T *A, const Geom &g, int x, int
 
 // WCA force of the pore-wall beads on a colloid bead at r (lab frame), from
 // the wall beads in a window around the nearest one (the window covers every
-// wall bead within the cutoff), minimum image along the periodic axis.
-// Components are selected, not indexed, so nothing goes to local memory.
-__device__ __forceinline__ void wall_bead_force(const WallBeads &w, const double r[3], double F[3]) {
+// wall bead within the cutoff), minimum image along the periodic axis: the
+// part of lane c of 8, every eighth wall bead of the window. Components are
+// selected, not indexed, so nothing goes to local memory.
+__device__ __forceinline__ void wall_bead_force(const WallBeads &w, const double r[3], int c, double F[3]) {
     F[0] = F[1] = F[2] = 0.0;
     const int ax = w.axis;
     const double ru = ax == 0 ? r[1] : r[0], rv = ax == 2 ? r[1] : r[2], rz = ax == 0 ? r[0] : (ax == 1 ? r[1] : r[2]);
@@ -71,40 +72,50 @@ __device__ __forceinline__ void wall_bead_force(const WallBeads &w, const double
     const bool all_j = 2 * w.wt + 1 >= w.ntheta, all_k = 2 * w.wz + 1 >= w.nrow;
     const int jlo = all_j ? 0 : j0 - w.wt, jhi = all_j ? w.ntheta - 1 : j0 + w.wt;
     const int klo = all_k ? 0 : k0 - w.wz, khi = all_k ? w.nrow - 1 : k0 + w.wz;
-    for (int kk = klo; kk <= khi; ++kk) {
-        int k = kk % w.nrow;
-        if (k < 0) k += w.nrow;
-        for (int jj = jlo; jj <= jhi; ++jj) {
-            int j = jj % w.ntheta;
-            if (j < 0) j += w.ntheta;
-            double sn, cs;
-            sincos(twopi * j / w.ntheta, &sn, &cs);
-            const double eu = du - w.Rc * cs, ev = dv - w.Rc * sn;
-            double ez = rz - (k + 0.5) * w.L / w.nrow;
-            ez -= w.L * floor(ez / w.L + 0.5);
-            const double d2 = eu * eu + ev * ev + ez * ez;
-            if (d2 >= w.rcut2) continue;
-            const double sr2 = w.sigma2 / d2, sr6 = sr2 * sr2 * sr2;
-            const double fm = 24.0 * w.eps * (2.0 * sr6 * sr6 - sr6) / d2;
-            // back to x, y, z: (u, v, axis) = (y, z, x), (x, z, y) or (x, y, z)
-            if (ax == 0) { F[1] += fm * eu; F[2] += fm * ev; F[0] += fm * ez; }
-            else if (ax == 1) { F[0] += fm * eu; F[2] += fm * ev; F[1] += fm * ez; }
-            else { F[0] += fm * eu; F[1] += fm * ev; F[2] += fm * ez; }
+    for (int kk = klo, jj = jlo + c;; jj += 8) {
+        while (jj > jhi && kk <= khi) {
+            jj -= jhi - jlo + 1;
+            ++kk;
         }
+        if (kk > khi) break;
+        int k = kk % w.nrow, j = jj % w.ntheta;
+        if (k < 0) k += w.nrow;
+        if (j < 0) j += w.ntheta;
+        double sn, cs;
+        sincos(twopi * j / w.ntheta, &sn, &cs);
+        const double eu = du - w.Rc * cs, ev = dv - w.Rc * sn;
+        double ez = rz - (k + 0.5) * w.L / w.nrow;
+        ez -= w.L * floor(ez / w.L + 0.5);
+        const double d2 = eu * eu + ev * ev + ez * ez;
+        if (d2 >= w.rcut2) continue;
+        const double sr2 = w.sigma2 / d2, sr6 = sr2 * sr2 * sr2;
+        const double fm = 24.0 * w.eps * (2.0 * sr6 * sr6 - sr6) / d2;
+        // back to x, y, z: (u, v, axis) = (y, z, x), (x, z, y) or (x, y, z)
+        if (ax == 0) { F[1] += fm * eu; F[2] += fm * ev; F[0] += fm * ez; }
+        else if (ax == 1) { F[0] += fm * eu; F[2] += fm * ev; F[1] += fm * ez; }
+        else { F[0] += fm * eu; F[1] += fm * ev; F[2] += fm * ez; }
     }
 }
 
 // Force and torque of the pore-wall beads on bead k (FP64): added to the
 // body's accumulators, not the fluid. Out of line, so that the coupling's
-// registers do not include it: few beads come near the wall.
-inline __device__ __noinline__ void wall_bead_body(const WallBeads &w, Body &B, double s0, double s1, double s2) {
+// registers do not include it. By the bead's eight lanes (c; all of them call
+// it): a bead near the wall has tens to thousands of wall beads in its window,
+// at ~200 FP64 instructions each. Per step, all lanes, one lane of eight, and a
+// thread per bead in a kernel of its own: R = 8 colloid (2941 beads) along the
+// wall of an R = 20 pore 52 / 148 / 176 us, 32 of them in a batch 209 / 538 /
+// 440; 9036 beads, all within reach of wall beads 2 apart, 453 / 2061 / 1244.
+inline __device__ __noinline__ void wall_bead_body(const WallBeads &w, Body &B, double s0, double s1, double s2, int c) {
     double rel[3], r[3], F[3], tq[3];
     for (int q = 0; q < 3; ++q) {
         rel[q] = B.R[3 * q] * s0 + B.R[3 * q + 1] * s1 + B.R[3 * q + 2] * s2;
         r[q] = B.X[q] + rel[q];
     }
-    wall_bead_force(w, r, F);
-    if (F[0] == 0.0 && F[1] == 0.0 && F[2] == 0.0) return;
+    wall_bead_force(w, r, c, F);
+    const unsigned group = 0xFFu << (threadIdx.x & 24);
+    for (int o = 1; o < 8; o <<= 1)
+        for (int q = 0; q < 3; ++q) F[q] += __shfl_xor_sync(group, F[q], o);
+    if (c != 0 || (F[0] == 0.0 && F[1] == 0.0 && F[2] == 0.0)) return;
     cross3(rel, F, tq);
     for (int q = 0; q < 3; ++q) {
         atomicAdd(&B.acc[q], F[q]);
@@ -112,10 +123,10 @@ inline __device__ __noinline__ void wall_bead_body(const WallBeads &w, Body &B, 
     }
 }
 
-// The wall beads' part of a bead's coupling, by one lane: the bead is first
-// tested in FP32 (its distance from the axis to ~1e-5, against a margin of
+// The wall beads' part of a bead's coupling, by its eight lanes: the bead is
+// first tested in FP32 (its distance from the axis to ~1e-5, against a margin of
 // 1e-3 of the wall's reach) and left alone when no wall bead can be near.
-__device__ __forceinline__ void couple_wall(const WallBeads &w, Body *bodies, int body, const double *s, int k) {
+__device__ __forceinline__ void couple_wall(const WallBeads &w, Body *bodies, int body, const double *s, int k, int c) {
     Body &B = bodies[body];
     const int u = w.axis == 0 ? 1 : 0, v = w.axis == 2 ? 1 : 2;
     const float s0 = (float)s[3 * k], s1 = (float)s[3 * k + 1], s2 = (float)s[3 * k + 2];
@@ -123,7 +134,7 @@ __device__ __forceinline__ void couple_wall(const WallBeads &w, Body *bodies, in
     const float dv = (float)(B.X[v] - w.cv) + (B.Rf[3 * v] * s0 + B.Rf[3 * v + 1] * s1 + B.Rf[3 * v + 2] * s2);
     const float near = w.reach_f;
     if (near > 0.f && du * du + dv * dv < near * near) return;
-    wall_bead_body(w, B, s[3 * k], s[3 * k + 1], s[3 * k + 2]);
+    wall_bead_body(w, B, s[3 * k], s[3 * k + 1], s[3 * k + 2], c);
 }
 
 // Flags `tile` in the tile flags of this step's force buffer when this lane

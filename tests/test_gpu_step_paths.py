@@ -212,3 +212,27 @@ def test_fp64_rates_close_to_minus_one(gap, case):
     B.lb_batch_step(1)
     o = P.orc.populations()
     assert np.max(np.abs(B.lb_batch_get_populations(0) - o) / W19[:, None]) <= TOL[64]
+
+
+@pytest.mark.parametrize("precision", [64, 32])
+@pytest.mark.parametrize("axis,spacing,rp,rr", [(0, 40.0, 3.0, 3.0), (1, 7.0, 6.0, 2.0), (2, 1.5, 2.5, 2.5), (1, 0.7, 1.0, 1.0),
+                                                (0, 3.0, 0.5, 0.9)])
+def test_wall_beads_shared_by_a_beads_lanes(axis, spacing, rp, rr, precision):
+    """Windows of three wall beads, of a few columns, of hundreds, and the whole
+    ring and row; most of the raspberry's beads within reach of the wall."""
+    n = [19, 19, 19]
+    n[axis] = 14
+    P = Pair(*n, precision=precision, pore=(8.0, axis), gamma_bead=0.02, **MRT)
+    P.gpu.lb_set_pore_beads(spacing, rp, rr, 1e-4)
+    P.orc.set_pore_beads(8.0, axis, spacing, rp, rr, 1e-4)
+    P.set_populations(perturbed_populations(P.N, amp=0.005, u_amp=0.01, seed=axis))
+    X = np.array(n) / 2 + 0.2
+    X[(axis + 1) % 3] += 2.4
+    beads = Wl.sphere_raspberry(5.0)
+    P.add_body(beads, X, mass=5e4, inertia=(5e5, 5.2e5, 5.4e5))
+    near = sum(np.linalg.norm(P.orc.wall_force(x)) > 0 for x in X + beads)
+    assert near >= 5
+    P.step(3)
+    assert P.pop_error() <= TOL[precision]
+    e = P.body_errors(0)
+    assert max(e["X"], e["V"], e["q"], e["w"], _force_errors(P, 0)) <= 100 * TOL[precision]
