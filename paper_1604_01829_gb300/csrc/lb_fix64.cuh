@@ -378,14 +378,18 @@ __device__ __forceinline__ void collide_node_f64(double (&f)[19], double Fx, dou
 
 // The fixed-point constants of a parameter set. rate[k - 4]: the relaxation
 // rate g_k of mode k = 4..18 (BGK: 1 - 1/tau for all). Not usable (on = 0)
-// when the noise could leave the range above (kT > 0.01 rho0), the scaled
-// exponents the doubles', or a factor of the equilibrium fix_split's.
+// when the scaled exponents could leave the doubles', a factor of the
+// equilibrium fix_split's, or too many nodes the range above by their noise:
+// from kT = 0.002 rho0 on most warps hold a node that does, and pay for both
+// evaluations. 94 x 81 x 103, us per step in fixed point (FP64: 462): 74 at kT
+// = 5e-4, 98 at 1e-3 (0.1 % of the nodes leave), 239 at 1.5e-3, 421 at 2e-3
+// (6 %), 485 from 3e-3 (20 %) on; 40^3 67.8 at 2e-3, 74-75 beyond (FP64: 69).
 inline FixParams fix_params(double rho0, double kT, const double rate[15]) {
     FixParams P{};
     int e = 0;
     std::frexp(rho0 * 1.5, &e);
     const int k = e - 1;                       // rho0 2^-k in [2/3, 4/3)
-    P.on = k > -600 && k < 600 && kT <= 0.01 * rho0 ? 1 : 0;
+    P.on = k > -600 && k < 600 && kT <= 0.002 * rho0 ? 1 : 0;
     P.cb = 1023 + k;
     P.ce = (1023 + k) * (1 << 20);
     P.eh = (0x453 - 61 + k) * (1 << 20);

@@ -236,3 +236,13 @@ def test_wall_beads_shared_by_a_beads_lanes(axis, spacing, rp, rr, precision):
     assert P.pop_error() <= TOL[precision]
     e = P.body_errors(0)
     assert max(e["X"], e["V"], e["q"], e["w"], _force_errors(P, 0)) <= 100 * TOL[precision]
+
+
+@pytest.mark.parametrize("kT", [1.9e-3, 2.0e-3, 2.1e-3, 9e-3])
+def test_fp64_noise_on_both_sides_of_the_fixed_point_rule(kT):
+    """kT = 0.002 rho0, where a lattice changes to the FP64 evaluation; below it
+    nodes that the noise takes out of range, beside ordinary ones."""
+    P = Pair(17, 9, 8, precision=64, rho0=1.3, kT=kT * 1.3, seed=4, body_force=(0.0, 1e-5, 0.0), **MRT)
+    P.set_populations(perturbed_populations(P.N, rho0=1.3, seed=12))
+    P.step(4)
+    assert P.pop_error() <= TOL[64]
