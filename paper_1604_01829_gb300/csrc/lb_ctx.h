@@ -66,7 +66,9 @@ struct lb_ctx {
     // [0, 6 nb) external forces then torques ([3 nb] each, host-written, read
     // by each step's prologue), [6 nb, 12 nb) force and torque totals per body,
     // [12 nb] the error word and then 13 nb values of X, V, q, w per body
-    // (written at the end of each group of steps)
+    // (written by each group's last kernel: k_finish, or the extra blocks of a
+    // chained group's last fluid kernel, beside its fluid blocks; checked
+    // builds write the error word after it)
     double *io_map = nullptr;          // host address
     double *io_dmap = nullptr;         // device address of the same memory
     cudaEvent_t ev_io = nullptr;       // after the last group that reads the external forces
